@@ -187,4 +187,16 @@ struct Bufs {
   int32_t* pre_tok;  // [max_seq] prefill / teacher-forced token ids
 };
 
+// Buffers of a prompt chunk (bf16 models, wide.cu): up to cap rows.  The
+// inputs of the products are kept as bf16 high and low planes.
+struct WideBufs {
+  int32_t cap;
+  float* h;            // [cap][d] residual stream
+  float* xq;           // [cap][qd] rotated queries
+  __nv_bfloat16* xn;   // [2][cap][d] residual rows times the next norm's weights
+  __nv_bfloat16* xo;   // [2][cap][qd] attention outputs
+  __nv_bfloat16* xa;   // [2][cap][F] SwiGLU outputs
+  float* ss;           // [2][ceil(d / 128)][cap] sums of squares of h per 128 columns
+};
+
 }  // namespace ssd

@@ -45,7 +45,7 @@ constexpr int kMaxQHidden = 1024;
 constexpr int kPrefillChunk = 16;
 
 // Lays out every device buffer in the workspace; returns the total size.
-size_t layout(const ssd_model_cfg& c, char* base, Dims* D, Bufs* B) {
+size_t layout(const ssd_model_cfg& c, char* base, Dims* D, Bufs* B, WideBufs* P) {
   Dims d{};
   d.L = c.n_layers;
   d.d = c.d_model;
@@ -98,8 +98,21 @@ size_t layout(const ssd_model_cfg& c, char* base, Dims* D, Bufs* B) {
   b.out_tok = cv.take<int32_t>(sizeof(int32_t) * (size_t)d.max_seq);
   b.traces = cv.take<ssd_round_trace>(sizeof(ssd_round_trace) * (size_t)d.max_seq);
   b.pre_tok = cv.take<int32_t>(sizeof(int32_t) * (size_t)d.max_seq);
+  // prompt chunks (bf16): no longer than the cache
+  WideBufs w{};
+  if (c.dtype == SSD_DTYPE_BF16) {
+    w.cap = std::min(kWideCap, (d.max_seq + 127) / 128 * 128);
+    const size_t cap = (size_t)w.cap;
+    w.h = cv.take<float>(sizeof(float) * cap * d.d);
+    w.xq = cv.take<float>(sizeof(float) * cap * d.qd);
+    w.xn = cv.take<__nv_bfloat16>(4 * cap * d.d);
+    w.xo = cv.take<__nv_bfloat16>(4 * cap * d.qd);
+    w.xa = cv.take<__nv_bfloat16>(4 * cap * d.F);
+    w.ss = cv.take<float>(sizeof(float) * 2 * (size_t)((d.d + 127) / 128) * cap);
+  }
   if (D) *D = d;
   if (B) *B = b;
+  if (P) *P = w;
   return cv.off;
 }
 
@@ -128,12 +141,14 @@ struct ssd_ctx {
   ssd_model_cfg cfg{};
   Dims D{};
   Bufs B{};
+  WideBufs P{};                    // bf16: prompt chunks
   const void* embed = nullptr;
   const void* lm_head = nullptr;
   const void* final_norm = nullptr;
   std::vector<LayerW> layers;
   std::vector<CUtensorMap> wmaps;  // bf16: [L][4] layer matrices, then the LM head
   TileMaps tmaps{};                // bf16: the input buffers
+  WideMaps xmaps{};                // bf16: the prompt chunks' inputs
   cudaStream_t stream = nullptr;
   cudaStream_t cap = nullptr;
   std::string err;
@@ -385,11 +400,66 @@ ssd_status check_flag(ssd_ctx* x, const Ctl& c) {
   return SSD_OK;
 }
 
+// Splits a prompt of n rows (bf16) into chunks of at most P.cap rows: chunk
+// ends at multiples of 128 rows (and n) with the least total work on the
+// busiest SM, plus the launches of a pass (about 5 us a layer's kernel).
+std::vector<int> wide_chunks(const ssd_ctx* x, int n) {
+  const int nt = (n + 127) / 128, most = std::max(1, x->P.cap / 128);
+  const long long fixed = 5 * 10000;  // cycles of a layer's five launches
+  std::vector<long long> cost(nt + 1, 0);
+  std::vector<int> from(nt + 1, 0);
+  for (int e = 1; e <= nt; ++e) {
+    long long best = -1;
+    for (int b = std::max(0, e - most); b < e; ++b) {
+      const int rows = std::min(n, e * 128) - b * 128;
+      const long long c = cost[b] + fixed + wide_layer_cost(x->D, rows);
+      if (best < 0 || c < best) {
+        best = c;
+        from[e] = b;
+      }
+    }
+    cost[e] = best;
+  }
+  std::vector<int> rows;
+  for (int e = nt; e > 0; e = from[e]) rows.push_back(std::min(n, e * 128) - from[e] * 128);
+  std::reverse(rows.begin(), rows.end());
+  return rows;
+}
+
+// run_prompt for bf16 prompts longer than one decode tile: chunks of up to
+// P.cap rows through the wide kernels, then the exit head over the last
+// trace_T rows, at most kPrefillChunk at a time.
+ssd_status run_prompt_wide(ssd_ctx* x, int n, int* last_row) {
+  const int T = x->trace_T, L = x->D.L;
+  int c0 = 0;
+  for (int M : wide_chunks(x, n)) {
+    CK(x, launch_embed_wide(x->D, x->B, x->P, x->embed, x->layers[0].attn_norm, x->B.pre_tok + c0, M,
+                            x->stream));
+    for (int l = 0; l < L; ++l)
+      CK(x, launch_layer_wide(x->D, x->B, x->P, x->xmaps, x->layers[l],
+                              l + 1 < L ? x->layers[l + 1].attn_norm : nullptr, l, M, c0, x->stream));
+    for (int r = std::max(0, std::min(n - T, n - 1) - c0); r < M;) {
+      const int m = std::min(kPrefillChunk, M - r);
+      CK(x, launch_take_rows(x->D, x->B, x->P, r, m, x->stream));
+      CK(x, enqueue_head(x, rows_explicit(c0 + r, m, x->B.pre_tok + c0 + r), kPrefillChunk, x->topk,
+                         x->sampled, x->stream));
+      CK(x, launch_trace_push(x->B, 0, m, x->stream));
+      *last_row = m - 1;
+      r += m;
+    }
+    c0 += M;
+  }
+  return SSD_OK;
+}
+
 // Full-model pass over ids[0..n) (already in pre_tok) from position 0 in
 // chunks; max-probabilities of the last trace_T rows seed the C_trace window.
-ssd_status run_prompt(ssd_ctx* x, int n) {
+// *last_row: the row of the statistics that belongs to the last token.
+ssd_status run_prompt(ssd_ctx* x, int n, int* last_row) {
   const int T = x->trace_T;
+  *last_row = (n - 1) % kPrefillChunk;
   CK(x, launch_reset_sequence(x->B, x->stream));
+  if (x->cfg.dtype == SSD_DTYPE_BF16 && n > kPrefillChunk) return run_prompt_wide(x, n, last_row);
   for (int c0 = 0; c0 < n; c0 += kPrefillChunk) {
     const int M = std::min(kPrefillChunk, n - c0);
     const RowSel sel = rows_explicit(c0, M, x->B.pre_tok + c0);
@@ -435,7 +505,7 @@ extern "C" {
 
 size_t ssd_workspace_bytes(const ssd_model_cfg* cfg) {
   if (check_cfg(cfg)) return 0;
-  return layout(*cfg, nullptr, nullptr, nullptr);
+  return layout(*cfg, nullptr, nullptr, nullptr, nullptr);
 }
 
 ssd_status ssd_init_model(const ssd_model_cfg* cfg, const ssd_weights* w, void* workspace,
@@ -450,7 +520,7 @@ ssd_status ssd_init_model(const ssd_model_cfg* cfg, const ssd_weights* w, void* 
     if (!aligned16(w->attn_norm[l]) || !aligned16(w->wqkv[l]) || !aligned16(w->wo[l]) ||
         !aligned16(w->ffn_norm[l]) || !aligned16(w->w_gate_up[l]) || !aligned16(w->w_down[l]))
       return fail(nullptr, SSD_ERR_INVALID_ARG, "layer weights: NULL or unaligned pointer");
-  const size_t need = layout(*cfg, nullptr, nullptr, nullptr);
+  const size_t need = layout(*cfg, nullptr, nullptr, nullptr, nullptr);
   if (!workspace || ((uintptr_t)workspace & 255u))
     return fail(nullptr, SSD_ERR_INVALID_ARG, "workspace must be non-NULL and 256-byte aligned");
   if (workspace_bytes < need) return fail(nullptr, SSD_ERR_CAPACITY, "workspace too small");
@@ -463,12 +533,13 @@ ssd_status ssd_init_model(const ssd_model_cfg* cfg, const ssd_weights* w, void* 
   if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e0 == cudaSuccess) e0 = prepare_gemv_kernels();
   if (e0 == cudaSuccess && cfg->dtype == SSD_DTYPE_BF16) e0 = prepare_tile_kernels();
+  if (e0 == cudaSuccess && cfg->dtype == SSD_DTYPE_BF16) e0 = prepare_wide_kernels();
   if (e0 != cudaSuccess) return cuda_fail(nullptr, "ssd_init_model device query", e0);
   if (const char* v = getenv("SSD_NO_PDL")) g_pdl_enabled = !(v[0] == '1');
   if (const char* v = getenv("SSD_NO_CHAIN")) g_chain_enabled = !(v[0] == '1');
   ssd_ctx* x = new ssd_ctx();
   x->cfg = *cfg;
-  layout(*cfg, static_cast<char*>(workspace), &x->D, &x->B);
+  layout(*cfg, static_cast<char*>(workspace), &x->D, &x->B, &x->P);
   // persistent grids: one block per SM of this context, all resident at once
   // (their phase barriers and split-tile fix-ups wait on other blocks)
   int per_sm = 1;
@@ -504,7 +575,10 @@ ssd_status ssd_init_model(const ssd_model_cfg* cfg, const ssd_weights* w, void* 
     ok = ok && encode_weight_map(&x->wmaps[4 * (size_t)L], w->lm_head, cfg->vocab, d) &&
          encode_input_maps(x->tmaps.h, x->B.h, d) &&
          encode_input_maps(x->tmaps.attn_out, x->B.attn_out, qd) &&
-         encode_input_maps(x->tmaps.act, x->B.act, F);
+         encode_input_maps(x->tmaps.act, x->B.act, F) &&
+         encode_wide_maps(x->xmaps.xn, x->P.xn, d, x->P.cap) &&
+         encode_wide_maps(x->xmaps.xo, x->P.xo, qd, x->P.cap) &&
+         encode_wide_maps(x->xmaps.xa, x->P.xa, F, x->P.cap);
     if (!ok) {
       delete x;
       return fail(nullptr, SSD_ERR_CUDA, "tensor-map encoding failed");
@@ -650,10 +724,10 @@ ssd_status ssd_prefill(ssd_ctx* x, const int32_t* ids, int32_t n, int32_t* first
   x->have_x = false;
   x->async_pending = false;
   CK(x, cudaMemcpyAsync(x->B.pre_tok, ids, sizeof(int32_t) * n, cudaMemcpyHostToDevice, x->stream));
-  ssd_status s = run_prompt(x, n);
+  int last_row = 0;
+  ssd_status s = run_prompt(x, n, &last_row);
   if (s) return s;
-  const int last_M = (n - 1) % kPrefillChunk + 1;
-  CK(x, launch_set_pending(x->D, x->B, last_M - 1, -1, n, x->stream));
+  CK(x, launch_set_pending(x->D, x->B, last_row, -1, n, x->stream));
   Ctl c;
   if ((s = read_ctl(x, &c))) return s;
   CK(x, cudaStreamSynchronize(x->stream));
@@ -673,7 +747,8 @@ ssd_status ssd_resume(ssd_ctx* x, const int32_t* ids, int32_t n) {
   x->async_pending = false;
   CK(x, cudaMemcpyAsync(x->B.pre_tok, ids, sizeof(int32_t) * (n - 1), cudaMemcpyHostToDevice,
                         x->stream));
-  ssd_status s = run_prompt(x, n - 1);
+  int last_row = 0;
+  ssd_status s = run_prompt(x, n - 1, &last_row);
   if (s) return s;
   CK(x, launch_set_pending(x->D, x->B, 0, ids[n - 1], n - 1, x->stream));
   Ctl c;

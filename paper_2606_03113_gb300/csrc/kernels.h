@@ -48,6 +48,27 @@ cudaError_t launch_tile_head(const Dims& D, const Bufs& B, const TileMaps& tm,
 cudaError_t launch_tile_plain(const Dims& D, const Bufs& B, const CUtensorMap& wm, int rows,
                               int cols, const float* x, int M, float* y, cudaStream_t st);
 
+// Prompt chunks of the bf16 decoder (wide.cu): up to kWideCap rows a pass.
+constexpr int kWideCap = 1024;
+struct WideMaps {
+  CUtensorMap xn[3], xo[3], xa[3];  // hi/lo input planes, boxes of 32, 64, 128 tokens
+};
+// Tensor map of an input's hi and lo planes ([2][cap][cols] bf16), boxes of
+// 64 columns x box_rows tokens x both planes.
+bool encode_split_map(CUtensorMap* m, const void* x, int cols, int cap, int box_rows);
+bool encode_wide_maps(CUtensorMap (&m)[3], const void* x, int cols, int cap);
+cudaError_t prepare_wide_kernels();
+long long wide_layer_cost(const Dims& D, int M);
+cudaError_t launch_embed_wide(const Dims& D, const Bufs& B, const WideBufs& P, const void* embed,
+                              const void* gnorm, const int32_t* toks, int M, cudaStream_t st);
+// One layer over the chunk's M rows at positions pos0..; next_norm: the norm
+// weights of the layer after it (null: none).
+cudaError_t launch_layer_wide(const Dims& D, const Bufs& B, const WideBufs& P, const WideMaps& xm,
+                              const LayerW& w, const void* next_norm, int layer, int M, int pos0,
+                              cudaStream_t st);
+cudaError_t launch_take_rows(const Dims& D, const Bufs& B, const WideBufs& P, int row0, int M,
+                             cudaStream_t st);
+
 // mrows is the largest number of rows a launch may see: 1 selects the
 // single-row kernels, more the multi-row ones (bf16: the tensor-core instance
 // with 8, 16 or 24 token rows, the smallest that holds mrows).  big

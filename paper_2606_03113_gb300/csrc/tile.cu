@@ -1142,6 +1142,20 @@ bool encode_input_map(CUtensorMap* m, const float* x, int cols, int rows, int bo
                   CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool encode_split_map(CUtensorMap* m, const void* x, int cols, int cap, int box_rows) {
+  if (!get_encoder() || !x || ((uintptr_t)x & 15u) || ((size_t)cols * 2) % 16 || cap < 1 ||
+      box_rows < 1 || box_rows > 256)
+    return false;
+  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)cap, 2};
+  cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cap * cols * 2};
+  cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 2};
+  cuuint32_t es[3] = {1, 1, 1};
+  return g_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), dims, strides, box,
+                  es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 cudaError_t prepare_tile_kernels() {
   cudaError_t e;
   if ((e = prep_kind<kKPlain, false>()) != cudaSuccess) return e;

@@ -1,0 +1,852 @@
+// wide.cu -- prompt processing of the bf16 decoder (sm_103a): up to kWideCap
+// prompt rows per pass through all layers, so that a weight is read once per
+// chunk of the prompt and not once per 16 rows.
+//
+// Products (k_wide): C[token][row] = sum_k W[row][k] x[token][k] on the
+// 5th-generation tensor cores.  A tile is 128 weight rows x TT tokens; the
+// input rows enter as bf16 high and low parts (x = hi + lo to 16 significant
+// bits, the split of the decode kernels), which stand side by side as one
+// operand of N = 2 TT columns, so one weight tile in shared memory serves
+// both.  The kernel that produces an input row writes its two parts already
+// multiplied by the RMSNorm weights of the product that reads it; the
+// norm's scale is applied to the product (per-tile sums of squares travel
+// beside the rows).
+//  - persistent grid, tiles dealt round robin with the token tiles of one
+//    weight tile next to each other (they share it in L2);
+//  - warp roles (320 threads): a TMA warp fills a ring of 64-column stages
+//    (two 64 x 64 weight boxes, one hi/lo input box), one thread issues
+//    tcgen05.mma (M = 128, N = 2 TT, K = 16) into double-buffered TMEM
+//    accumulators, eight warps run the fused epilogue of one tile while the
+//    next one multiplies;
+//  - a rotary or gate/up pair of a tile sits in rows r and r + 64, that is in
+//    TMEM lanes of different warps: they swap halves through shared memory.
+// Bound by the tensor cores and by the copies out of L2 (48 KB per stage of
+// a 128-token tile in 512 cycles of tcgen05.mma at full rate).  512 rows of
+// the Llama-2-7B shape: gate/up 126.6 us (1.46 PFLOP/s with both parts), QKV
+// 83.7, down 75.0, O 35.3 us; a 512-token prompt through four layers takes
+// 1.9 ms against 18.0 ms in 32 passes of 16 rows, 2043 tokens of the 13B
+// shape 9.6 ms against 104.6 ms.
+// Attention (k_attn_wide): 64 query rows x one head per block, 64-key steps
+// with a running maximum; scores and outputs on mma.sync with the fp32
+// operand (queries, probabilities) in three bf16 parts, 24 bits, so nothing
+// is rounded below fp32.  Bound by mma.sync: 512 rows of the Llama-2-7B shape
+// take 42 us a layer, rows 1024-1919 of the 13B shape 262 us (315 TFLOP/s with
+// the three parts).
+#include <math.h>
+
+#include "kernels.h"
+#include "pipe.cuh"
+#include "tc.cuh"
+
+namespace ssd {
+
+namespace {
+
+constexpr int kWR = 128;              // weight rows per tile
+constexpr int kWK = 64;               // columns per stage
+constexpr int kWEpi = 8;              // epilogue warps
+constexpr int kWEThreads = kWEpi * 32;
+constexpr int kWTmaWarp = kWEpi, kWMmaWarp = kWEpi + 1;
+constexpr int kWThreads = (kWEpi + 2) * 32;
+constexpr int kWChunk = 16;           // tokens per epilogue step of a warp
+// Stages summed in one TMEM accumulator before the epilogue warps add it to
+// their registers: the tensor core's running sum is cut and not rounded at
+// each 16-column step, so a sum over all of K in TMEM would be off by up to
+// K / 16 units in the last place, to one side.  1024 columns at a time keep
+// that at 64, as in the decode kernels, whose blocks sum 450 to 2300 columns
+// of a row each.  The drain is hidden by the other accumulator but for its
+// own tensor-memory reads: 512 tokens of the 12288 x 4096 product take 83.7
+// us (94.5 us with 512 columns at a time, 76.5 us with all of K).
+constexpr int kWSeg = 16;
+
+enum WKind : int { kWQkv = 0, kWResid = 1, kWGateUp = 2 };
+
+template <int TT>
+struct WL {
+  static constexpr int N = 2 * TT;
+  static constexpr int A = kWR * kWK * 2;
+  static constexpr int X = N * kWK * 2;
+  static constexpr int Stage = A + X;
+  static constexpr int NS = TT == 128 ? 4 : (TT == 64 ? 6 : 8);
+  static constexpr uint32_t kCols = 2 * N;
+  static constexpr size_t exch = (size_t)NS * Stage;                  // [2][warps][8][32] floats
+  static constexpr size_t rs = exch + 2 * kWEpi * 8 * 32 * 4;          // [TT]
+  static constexpr size_t red = rs + TT * 4;                           // [4][TT]
+  static constexpr size_t bars = red + 4 * TT * 4;                     // full, empty, accfull, accempty
+  static constexpr size_t tslot = bars + 8 * (2 * NS + 4);
+  static constexpr size_t total = tslot + 16 + 1024;
+  static_assert(total <= 227 * 1024, "shared memory budget");
+};
+
+struct WArgs {
+  Dims D;
+  Bufs B;
+  WideBufs P;
+  int N, K, nks, nrt, ntt;     // rows, columns, stages, row tiles, token tiles
+  int M, pos0, layer;
+  const float* ss_in;          // per-tile sums of squares of the input rows, or null
+  float* ss_out;               // residual: the same for the rows written
+  const __nv_bfloat16* gnext;  // residual: norm weights of the next product (null: none)
+};
+
+__device__ __forceinline__ void w_flag(const Bufs& B) { atomicOr(&B.ctl->err, (int)kErrTimeout); }
+
+// 3-D tiled load (columns, rows, part).
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int c0, int r0,
+                                            int z0, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(r0), "r"(z0), "r"(smem_u32(bar))
+      : "memory");
+}
+
+__device__ __forceinline__ void tma_load_2d_plain(void* dst, const CUtensorMap* map, int c0, int r0,
+                                                  uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(r0), "r"(smem_u32(bar))
+      : "memory");
+}
+
+// 16 columns of the warp's TMEM lanes from two places (high and low parts), added.
+__device__ __forceinline__ void tc_ld16_sum(uint32_t hi, uint32_t lo, float (&v)[16]) {
+  uint32_t a[16], b[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+      "%15}, [%16];"
+      : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]),
+        "=r"(a[7]), "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]),
+        "=r"(a[14]), "=r"(a[15])
+      : "r"(hi)
+      : "memory");
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+      "%15}, [%16];"
+      : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]),
+        "=r"(b[7]), "=r"(b[8]), "=r"(b[9]), "=r"(b[10]), "=r"(b[11]), "=r"(b[12]), "=r"(b[13]),
+        "=r"(b[14]), "=r"(b[15])
+      : "r"(lo)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(a[i]) + __uint_as_float(b[i]);
+}
+
+// Sums of 16 values over the warp's 32 lanes in a fixed order; lane 2 i (and
+// 2 i + 1) returns the sum of value i.
+__device__ __forceinline__ float warp_sum16(float (&v)[16], int lane) {
+#pragma unroll
+  for (int off = 16, n = 8; n >= 1; off >>= 1, n >>= 1) {
+    const bool up = lane & off;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i < n) {
+        const float keep = up ? v[i + n] : v[i], give = up ? v[i] : v[i + n];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+      }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// x as bf16 high and low parts into the two planes of an operand buffer.
+__device__ __forceinline__ void put_split(__nv_bfloat16* p, size_t plane, float x) {
+  const __nv_bfloat16 h = __float2bfloat16_rn(x);
+  p[0] = h;
+  p[plane] = __float2bfloat16_rn(x - __bfloat162float(h));
+}
+
+}  // namespace
+
+template <int TT, int KIND>
+__global__ void __launch_bounds__(kWThreads, 1)
+    k_wide(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap,
+           const WArgs a) {
+  using S = WL<TT>;
+  constexpr int NS = S::NS, N = S::N;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::bars);
+  uint64_t* empty = full + NS;
+  uint64_t* accfull = empty + NS;
+  uint64_t* accempty = accfull + 2;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + S::tslot);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+  if (tid == 0) {
+    for (int i = 0; i < NS; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&accfull[i], 1);
+      mbar_init(&accempty[i], kWEpi);
+    }
+    mbar_init_fence();
+  }
+  if (warp == kWMmaWarp) tc_alloc(tslot, S::kCols);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tslot;
+  pdl_launch_dependents();
+
+  const int ntiles = a.nrt * a.ntt;
+  if (warp == kWTmaWarp) {
+    if (lane == 0) {
+      tma_prefetch_desc(&wmap);
+      tma_prefetch_desc(&xmap);
+      // weight boxes of the first stages need nothing from earlier kernels
+      auto weights = [&](int slot, int tile, int kc) {
+        const int rt = tile / a.ntt;
+        unsigned char* dst = smem + (size_t)slot * S::Stage;
+        mbar_arrive_expect_tx(&full[slot], (uint32_t)S::Stage);
+        const int r0 = KIND == kWGateUp ? rt * 64 : rt * 128;
+        const int r1 = KIND == kWGateUp ? a.N / 2 + rt * 64 : rt * 128 + 64;
+        tma_load_2d_plain(dst, &wmap, kc * kWK, r0, &full[slot]);
+        tma_load_2d_plain(dst + S::A / 2, &wmap, kc * kWK, r1, &full[slot]);
+      };
+      bool ok = true;
+      int npre = 0;
+      if ((int)blockIdx.x < ntiles)
+        for (; npre < NS && npre < a.nks; ++npre) weights(npre, blockIdx.x, npre);
+      pdl_wait();
+      asm volatile("fence.proxy.async.global;" ::: "memory");
+      int slot = 0, it = 0;
+      uint32_t ph = 1;
+      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+        const int tt = tile % a.ntt;
+        for (int kc = 0; kc < a.nks; ++kc, ++it) {
+          if (it >= npre) {
+            if (!mbar_wait(&empty[slot], ph)) {
+              ok = false;
+              break;
+            }
+            weights(slot, tile, kc);
+          }
+          tma_load_3d(smem + (size_t)slot * S::Stage + S::A, &xmap, kc * kWK, tt * TT, 0, &full[slot]);
+          if (++slot == NS) {
+            slot = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+      if (!ok) w_flag(a.B);
+      // every copy has landed before the block exits
+      for (int j = it > NS ? it - NS : 0; j < it; ++j) mbar_wait(&full[j % NS], (uint32_t)(j / NS) & 1u);
+    }
+  } else if (warp == kWMmaWarp) {
+    if (lane == 0) {
+      constexpr uint32_t idesc = idesc_bf16_f32(128, N);
+      bool ok = true;
+      int slot = 0, sc = 0;
+      uint32_t ph = 0;
+      for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+        for (int kc = 0; kc < a.nks; ++kc) {
+          const bool first = kc % kWSeg == 0;
+          if (first && !(ok = mbar_wait(&accempty[sc & 1], ((uint32_t)(sc >> 1) & 1u) ^ 1u))) break;
+          if (!(ok = mbar_wait(&full[slot], ph))) break;
+          tc_fence_after();
+          const uint32_t d = tmem + (uint32_t)((sc & 1) * N);
+          const uint32_t ab = smem_u32(smem + (size_t)slot * S::Stage);
+          const uint32_t xb = ab + S::A;
+#pragma unroll
+          for (int kk = 0; kk < kWK / 16; ++kk)
+            tc_mma_bf16(d, sdesc_k128(ab + kk * 32), sdesc_k128(xb + kk * 32), idesc,
+                        !first || kk > 0);
+          tc_commit(&empty[slot]);
+          if (kc % kWSeg == kWSeg - 1 || kc == a.nks - 1) tc_commit(&accfull[sc++ & 1]);
+          if (++slot == NS) {
+            slot = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+      if (!ok) w_flag(a.B);
+    }
+  } else {
+    // ---------------- epilogue warps: lane quarter q, token half th
+    pdl_wait();
+    float* exch = reinterpret_cast<float*>(smem + S::exch);
+    float* srs = reinterpret_cast<float*>(smem + S::rs);
+    float* red = reinterpret_cast<float*>(smem + S::red);
+    const Dims& D = a.D;
+    const int q = warp & 3, th = warp >> 2;
+    bool ok = true;
+    int sc = 0, xp = 0;
+    const int nseg = (a.nks + kWSeg - 1) / kWSeg;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+      const int rt = tile / a.ntt, t0 = (tile % a.ntt) * TT;
+      if constexpr (KIND != kWResid) {
+        // RMSNorm scale of the tile's input rows: their sums of squares per
+        // 128 columns, added in column order
+        for (int t = tid; t < TT; t += kWEThreads) {
+          float sum = 0.f;
+          if (t0 + t < a.M) {
+            const float* sp = a.ss_in + t0 + t;
+            const int np = (a.K + kWR - 1) / kWR;
+#pragma unroll 8
+            for (int c = 0; c < np; ++c) sum += __ldcg(sp + (size_t)c * a.P.cap);
+          }
+          srs[t] = 1.0f / sqrtf(sum / (float)a.K + D.eps);
+        }
+        named_sync(1, kWEThreads);
+      }
+      // the tile's sums: segments added in K order, high plus low parts
+      float acc[TT / 2];
+#pragma unroll
+      for (int c = 0; c < TT / 2; ++c) acc[c] = 0.f;
+      for (int g = 0; g < nseg; ++g, ++sc) {
+        if (ok) {
+          ok = __all_sync(0xffffffffu, mbar_wait(&accfull[sc & 1], (uint32_t)(sc >> 1) & 1u));
+          if (!ok && lane == 0) w_flag(a.B);
+        }
+        tc_fence_after();
+        const uint32_t src = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((sc & 1) * N + th * (TT / 2));
+#pragma unroll
+        for (int c = 0; c < TT / 2; c += kWChunk)
+          if (ok && t0 + th * (TT / 2) + c < a.M) {
+            float v[kWChunk];
+            tc_ld16_sum(src + c, src + TT + c, v);
+#pragma unroll
+            for (int j = 0; j < kWChunk; ++j) acc[c + j] += v[j];
+          }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&accempty[sc & 1]);
+      }
+#pragma unroll
+      for (int c = 0; c < TT / 2; c += kWChunk) {
+        const int tl = th * (TT / 2) + c;  // the step's first token in the tile
+        if (t0 + tl >= a.M) break;
+        float v[kWChunk];
+#pragma unroll
+        for (int j = 0; j < kWChunk; ++j) v[j] = acc[c + j];
+        const int nt = min(kWChunk, a.M - t0 - tl);
+        if constexpr (KIND == kWResid) {
+          const int row = rt * kWR + 32 * q + lane;
+          const bool in = row < a.N;
+          float* h = a.P.h + (size_t)(t0 + tl) * D.d + row;
+          float hp[kWChunk];
+#pragma unroll
+          for (int j = 0; j < kWChunk; ++j) hp[j] = (in && j < nt) ? h[(size_t)j * D.d] : 0.f;
+          const float g = (in && a.gnext) ? __bfloat162float(a.gnext[row]) : 0.f;
+          const size_t plane = (size_t)a.P.cap * D.d;
+          __nv_bfloat16* xn = a.P.xn + (size_t)(t0 + tl) * D.d + row;
+          float sq[kWChunk];
+#pragma unroll
+          for (int j = 0; j < kWChunk; ++j) {
+            const float x = hp[j] + v[j];
+            sq[j] = (in && j < nt) ? x * x : 0.f;
+            if (in && j < nt) {
+              h[(size_t)j * D.d] = x;
+              if (a.gnext) put_split(xn + (size_t)j * D.d, plane, x * g);
+            }
+          }
+          const float s = warp_sum16(sq, lane);
+          if (!(lane & 1)) red[q * TT + tl + (lane >> 1)] = s;
+        } else {
+          // swap halves: warps of rows 0-63 finish tokens 0-7 of the step,
+          // warps of rows 64-127 tokens 8-15
+          const bool low = q < 2;
+          float* mine = exch + ((size_t)xp * kWEpi + warp) * 256 + lane;
+          const float* other = exch + ((size_t)xp * kWEpi + (warp ^ 2)) * 256 + lane;
+          xp ^= 1;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) mine[j * 32] = low ? v[8 + j] : v[j];
+          named_sync(2 + th, 128);
+          const int i = 32 * (q & 1) + lane;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int tj = low ? j : 8 + j;
+            if (tj >= nt) continue;
+            const int t = t0 + tl + tj;
+            const float rs = srs[tl + tj];
+            const float o = other[j * 32];
+            const float y0 = (low ? v[j] : o) * rs, y1 = (low ? o : v[8 + j]) * rs;
+            if constexpr (KIND == kWGateUp) {
+              const int jj = rt * 64 + i;
+              if (jj < D.F)
+                put_split(a.P.xa + (size_t)t * D.F + jj, (size_t)a.P.cap * D.F,
+                          y0 / (1.0f + expf(-y0)) * y1);
+            } else {
+              // one head per tile: rotary pair (i, i + 64) or two value rows
+              const int head = rt, pos = a.pos0 + t;
+              __nv_bfloat16* kv = static_cast<__nv_bfloat16*>(a.B.kv) +
+                                  (size_t)a.layer * 2 * D.Hkv * D.max_seq * D.hd;
+              if (head < D.Hq + D.Hkv) {
+                const float2 cs = a.B.rope[(size_t)pos * 64 + i];
+                const float r0 = y0 * cs.x - y1 * cs.y, r1 = y1 * cs.x + y0 * cs.y;
+                if (head < D.Hq) {
+                  float* qo = a.P.xq + (size_t)t * D.qd + head * 128 + i;
+                  qo[0] = r0;
+                  qo[64] = r1;
+                } else {
+                  __nv_bfloat16* kr = kv + ((size_t)(head - D.Hq) * D.max_seq + pos) * 128 + i;
+                  kr[0] = __float2bfloat16_rn(r0);
+                  kr[64] = __float2bfloat16_rn(r1);
+                }
+              } else {
+                __nv_bfloat16* vr =
+                    kv + ((size_t)(head - D.Hq) * D.max_seq + pos) * 128 + i;  // Hkv + g
+                vr[0] = __float2bfloat16_rn(y0);
+                vr[64] = __float2bfloat16_rn(y1);
+              }
+            }
+          }
+        }
+      }
+      named_sync(1, kWEThreads);
+      if constexpr (KIND == kWResid) {
+        for (int t = tid; t < TT && t0 + t < a.M; t += kWEThreads)
+          a.ss_out[(size_t)rt * a.P.cap + t0 + t] =
+              red[t] + red[TT + t] + red[2 * TT + t] + red[3 * TT + t];
+        named_sync(1, kWEThreads);
+      }
+    }
+  }
+  // TMEM is released once every accumulator has been read
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == kWMmaWarp) tc_dealloc(tmem, S::kCols);
+}
+
+// ------------------------------------------------------------- attention
+
+namespace {
+
+constexpr int kAQ = 64;   // query rows per block (16 per warp)
+constexpr int kAKB = 64;  // keys per step
+constexpr int kAHd = 128;
+constexpr int kAWThreads = 128;
+constexpr size_t kAQBytes = (size_t)3 * kAQ * kAHd * 2;  // queries, three bf16 parts
+constexpr size_t kAKBytes = (size_t)kAKB * kAHd * 2;
+constexpr size_t kAWSmem = kAQBytes + 4 * kAKBytes;      // + keys and values, double buffered
+
+// Byte offset of 16-byte chunk c of a 256-byte row (swizzled by row % 8).
+__device__ __forceinline__ uint32_t aw_off(int row, int c) {
+  return (uint32_t)(row * 256 + ((c ^ (row & 7)) << 4));
+}
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
+               "r"(valid ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
+                                         uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// (x, y) as three packed bf16 pairs whose sum keeps 24 bits of each.
+__device__ __forceinline__ void split3(float x, float y, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
+  auto pack = [](float u, float w) -> uint32_t {
+    const __nv_bfloat162 b = __floats2bfloat162_rn(u, w);
+    return *reinterpret_cast<const uint32_t*>(&b);
+  };
+  auto lo = [](uint32_t p) { return __uint_as_float(p << 16); };
+  auto hi = [](uint32_t p) { return __uint_as_float(p & 0xffff0000u); };
+  p0 = pack(x, y);
+  const float x1 = x - lo(p0), y1 = y - hi(p0);
+  p1 = pack(x1, y1);
+  p2 = pack(x1 - lo(p1), y1 - hi(p1));
+}
+
+}  // namespace
+
+__global__ void __launch_bounds__(kAWThreads, 2)
+    k_attn_wide(const Dims D, const Bufs B, const WideBufs P, int layer, int M, int pos0) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  pdl_wait();
+  pdl_launch_dependents();
+  const int head = blockIdx.x;
+  const int q0 = (int)(gridDim.y - 1 - blockIdx.y) * kAQ;  // longest blocks first
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+  const int g = head / (D.Hq / D.Hkv);
+  const __nv_bfloat16* kv =
+      static_cast<const __nv_bfloat16*>(B.kv) + (size_t)layer * 2 * D.Hkv * D.max_seq * kAHd;
+  const __nv_bfloat16* kb = kv + (size_t)g * D.max_seq * kAHd;
+  const __nv_bfloat16* vb = kv + (size_t)(D.Hkv + g) * D.max_seq * kAHd;
+  const uint32_t sq = smem_u32(smem), sk = sq + (uint32_t)kAQBytes;
+  const int last = pos0 + min(M, q0 + kAQ) - 1;  // last key any row of the block sees
+  const int nkb = last / kAKB + 1;
+
+  auto stage = [&](int b) {
+    const uint32_t kd = sk + (uint32_t)((b & 1) * 2) * (uint32_t)kAKBytes;
+    const uint32_t vd = kd + (uint32_t)kAKBytes;
+#pragma unroll
+    for (int j = 0; j < kAKB * 16 / kAWThreads; ++j) {
+      const int c = tid + j * kAWThreads, row = c >> 4, ch = c & 15;
+      const int key = b * kAKB + row;
+      const bool in = key <= last;  // keys past the last one read zeros
+      const size_t off = (size_t)(in ? key : 0) * kAHd + ch * 8;
+      cp16(kd + aw_off(row, ch), kb + off, in);
+      cp16(vd + aw_off(row, ch), vb + off, in);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  stage(0);
+  // queries: three bf16 parts
+  for (int c = tid; c < kAQ * 16; c += kAWThreads) {
+    const int row = c >> 4, ch = c & 15;
+    float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), x1 = x0;
+    if (q0 + row < M) {
+      const float4* p =
+          reinterpret_cast<const float4*>(P.xq + (size_t)(q0 + row) * D.qd + head * kAHd + ch * 8);
+      x0 = p[0];
+      x1 = p[1];
+    }
+    uint4 w[3];
+    split3(x0.x, x0.y, w[0].x, w[1].x, w[2].x);
+    split3(x0.z, x0.w, w[0].y, w[1].y, w[2].y);
+    split3(x1.x, x1.y, w[0].z, w[1].z, w[2].z);
+    split3(x1.z, x1.w, w[0].w, w[1].w, w[2].w);
+#pragma unroll
+    for (int s = 0; s < 3; ++s)
+      *reinterpret_cast<uint4*>(smem + (size_t)s * kAQ * 256 + aw_off(row, ch)) = w[s];
+  }
+
+  float o[16][4];
+#pragma unroll
+  for (int n = 0; n < 16; ++n)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) o[n][e] = 0.f;
+  float mx[2] = {-INFINITY, -INFINITY}, ls[2] = {0.f, 0.f};
+  const float scale = 1.0f / sqrtf((float)kAHd);
+  const int r0 = pos0 + q0 + 16 * warp + (lane >> 2);  // position of the thread's first row
+  const int lrow = 16 * warp + (lane & 15), lch = lane >> 4;  // ldmatrix row / chunk of queries
+
+  for (int b = 0; b < nkb; ++b) {
+    if (b + 1 < nkb) {
+      stage(b + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    const uint32_t kd = sk + (uint32_t)((b & 1) * 2) * (uint32_t)kAKBytes;
+    const uint32_t vd = kd + (uint32_t)kAKBytes;
+    float s[8][4];
+#pragma unroll
+    for (int n = 0; n < 8; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s[n][e] = 0.f;
+    // the queries' two lower parts first: the running sum is cut at its own
+    // last place, so the small terms lose nothing to it
+#pragma unroll
+    for (int pass = 0; pass < 2; ++pass)
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk) {
+        uint32_t qa[2][4];
+        const int np = pass ? 1 : 2;
+#pragma unroll
+        for (int p = 0; p < np; ++p)
+          ldsm4(sq + (uint32_t)((pass ? 0 : 2 - p) * kAQ * 256) + aw_off(lrow, 2 * kk + lch), qa[p]);
+#pragma unroll
+        for (int n2 = 0; n2 < 4; ++n2) {
+          // keys 16 n2 .. + 15 x 16 columns: two n-tiles
+          uint32_t kf[4];
+          ldsm4(kd + aw_off(16 * n2 + (lane & 7) + ((lane >> 4) << 3), 2 * kk + ((lane >> 3) & 1)),
+                kf);
+#pragma unroll
+          for (int p = 0; p < np; ++p) {
+            mma16816(s[2 * n2], qa[p], kf[0], kf[1]);
+            mma16816(s[2 * n2 + 1], qa[p], kf[2], kf[3]);
+          }
+        }
+      }
+    // scale, causal mask, running maximum
+    const int kbase = b * kAKB + 2 * (lane & 3);
+    float nm[2] = {mx[0], mx[1]};
+#pragma unroll
+    for (int n = 0; n < 8; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int key = kbase + 8 * n + (e & 1), row = r0 + 8 * (e >> 1);
+        s[n][e] = key <= row ? s[n][e] * scale : -INFINITY;
+        nm[e >> 1] = fmaxf(nm[e >> 1], s[n][e]);
+      }
+    float f[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      nm[r] = fmaxf(nm[r], __shfl_xor_sync(0xffffffffu, nm[r], 1));
+      nm[r] = fmaxf(nm[r], __shfl_xor_sync(0xffffffffu, nm[r], 2));
+      // block 0 holds key 0, which every row sees: the maximum is finite
+      f[r] = expf(mx[r] - nm[r]);
+      mx[r] = nm[r];
+      ls[r] *= f[r];
+    }
+#pragma unroll
+    for (int n = 0; n < 8; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        s[n][e] = expf(s[n][e] - mx[e >> 1]);
+        ls[e >> 1] += s[n][e];
+      }
+    uint32_t pa[4][3][4];
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        split3(s[2 * ks + (e >> 1)][2 * (e & 1)], s[2 * ks + (e >> 1)][2 * (e & 1) + 1],
+               pa[ks][0][e], pa[ks][1][e], pa[ks][2][e]);
+#pragma unroll
+    for (int n2 = 0; n2 < 8; ++n2) {
+      // this step's share of 16 columns in sums of its own, then one rounded
+      // fused multiply-add into the running output
+      float t[2][4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) t[0][e] = t[1][e] = 0.f;
+      uint32_t vf[4][4];
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks)
+        ldsm4t(vd + aw_off(16 * ks + (lane & 15), 2 * n2 + (lane >> 4)), vf[ks]);
+#pragma unroll
+      for (int p = 2; p >= 0; --p)
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+          mma16816(t[0], pa[ks][p], vf[ks][0], vf[ks][1]);
+          mma16816(t[1], pa[ks][p], vf[ks][2], vf[ks][3]);
+        }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        o[2 * n2][e] = fmaf(o[2 * n2][e], f[e >> 1], t[0][e]);
+        o[2 * n2 + 1][e] = fmaf(o[2 * n2 + 1][e], f[e >> 1], t[1][e]);
+      }
+    }
+    __syncthreads();  // the buffer is staged again two steps on
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    ls[r] += __shfl_xor_sync(0xffffffffu, ls[r], 1);
+    ls[r] += __shfl_xor_sync(0xffffffffu, ls[r], 2);
+  }
+  const size_t plane = (size_t)P.cap * D.qd;
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int m = q0 + 16 * warp + (lane >> 2) + 8 * r;
+    if (m >= M) continue;
+    __nv_bfloat16* out = P.xo + (size_t)m * D.qd + head * kAHd + 2 * (lane & 3);
+#pragma unroll
+    for (int n = 0; n < 16; ++n) {
+      const float x = o[n][2 * r] / ls[r], y = o[n][2 * r + 1] / ls[r];
+      const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+      const __nv_bfloat162 l =
+          __floats2bfloat162_rn(x - __low2float(h), y - __high2float(h));
+      *reinterpret_cast<__nv_bfloat162*>(out + 8 * n) = h;
+      *reinterpret_cast<__nv_bfloat162*>(out + plane + 8 * n) = l;
+    }
+  }
+}
+
+// ----------------------------------------------- embedding and row hand-over
+
+// Row m of a chunk: h = embed[tok[m]], its split parts under the first norm's
+// weights, and its sums of squares per 128 columns.
+__global__ void __launch_bounds__(256)
+    k_embed_wide(const Dims D, const Bufs B, const WideBufs P, const __nv_bfloat16* __restrict__ emb,
+                 const __nv_bfloat16* __restrict__ gnorm, const int32_t* __restrict__ toks) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int m = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int tok = toks[m];
+  if (tok < 0 || tok >= D.V) {
+    if (threadIdx.x == 0) atomicOr(&B.ctl->err, (int)kErrToken);
+    tok = 0;
+  }
+  const __nv_bfloat16* row = emb + (size_t)tok * D.d;
+  float* h = P.h + (size_t)m * D.d;
+  __nv_bfloat16* xn = P.xn + (size_t)m * D.d;
+  const size_t plane = (size_t)P.cap * D.d;
+  for (int c = warp; c * kWR < D.d; c += 8) {
+    float sp = 0.f;
+#pragma unroll
+    for (int j = 0; j < kWR / 32; ++j) {
+      const int i = c * kWR + j * 32 + lane;
+      if (i < D.d) {
+        const float v = __bfloat162float(row[i]);
+        h[i] = v;
+        put_split(xn + i, plane, v * __bfloat162float(gnorm[i]));
+        sp = fmaf(v, v, sp);
+      }
+    }
+    sp = warp_sum(sp);
+    if (lane == 0) P.ss[(size_t)c * P.cap + m] = sp;
+  }
+}
+
+// Rows row0.. of the chunk's residual stream as rows 0.. of the decode
+// buffers, with their sums of squares per 256 columns, for the exit head.
+__global__ void __launch_bounds__(256)
+    k_take_rows(const Dims D, const Bufs B, const WideBufs P, int row0) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int m = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float* src = P.h + (size_t)(row0 + m) * D.d;
+  float* dst = B.h + (size_t)m * D.d;
+  for (int c = warp; c < D.ss_nt; c += 8) {
+    float sp = 0.f;
+    for (int i = c * 256 + lane; i < min(D.d, c * 256 + 256); i += 32) {
+      const float v = src[i];
+      dst[i] = v;
+      sp = fmaf(v, v, sp);
+    }
+    sp = warp_sum(sp);
+    if (lane == 0) B.ss_part[(size_t)c * kMaxM + m] = sp;
+  }
+}
+
+// ------------------------------------------------------------- host side
+
+namespace {
+
+template <int TT, int KIND>
+cudaError_t wide_prep() {
+  return cudaFuncSetAttribute(k_wide<TT, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)WL<TT>::total);
+}
+template <int TT>
+cudaError_t wide_prep_all() {
+  cudaError_t e = wide_prep<TT, kWQkv>();
+  if (e == cudaSuccess) e = wide_prep<TT, kWResid>();
+  return e != cudaSuccess ? e : wide_prep<TT, kWGateUp>();
+}
+
+// Cycles of one 64-column stage of a tile of tt tokens on one SM: the copy of
+// its 16 KB of weights and 256 tt bytes of input rows out of L2 (about 60
+// bytes a cycle and SM with all SMs reading), or 4 tt cycles of tcgen05.mma.
+int stage_cost(int tt) { return 273 + 4 * tt + tt / 4; }
+
+int row_tiles(int N, bool pairs) { return pairs ? (N / 2 + 63) / 64 : (N + kWR - 1) / kWR; }
+
+// Token tile (index 0, 1, 2 = 32, 64, 128 tokens) of the product of N rows
+// with M tokens that has the least work on the busiest SM.
+int pick_tile(int sms, int nrt, int M, long long* cost) {
+  int best = 0;
+  long long bc = 0;
+  for (int i = 0; i < 3; ++i) {
+    const int tt = 32 << i;
+    const long long tiles = (long long)nrt * ((M + tt - 1) / tt);
+    const long long c = (tiles + sms - 1) / sms * stage_cost(tt);
+    if (i == 0 || c < bc) {
+      bc = c;
+      best = i;
+    }
+  }
+  if (cost) *cost = bc;
+  return best;
+}
+
+template <int KIND>
+cudaError_t wide_launch(const CUtensorMap& wm, const CUtensorMap* xm, WArgs& a, cudaStream_t st) {
+  a.nks = (a.K + kWK - 1) / kWK;
+  a.nrt = row_tiles(a.N, KIND == kWGateUp);
+  const int ti = pick_tile(a.D.num_sms, a.nrt, a.M, nullptr);
+  a.ntt = (a.M + (32 << ti) - 1) / (32 << ti);
+  const long long tiles = (long long)a.nrt * a.ntt;
+  const dim3 grid((unsigned)(tiles < a.D.num_sms ? tiles : a.D.num_sms)), blk(kWThreads);
+  switch (ti) {
+    case 0: return launch_ex(k_wide<32, KIND>, grid, blk, WL<32>::total, st, wm, xm[0], a);
+    case 1: return launch_ex(k_wide<64, KIND>, grid, blk, WL<64>::total, st, wm, xm[1], a);
+    default: return launch_ex(k_wide<128, KIND>, grid, blk, WL<128>::total, st, wm, xm[2], a);
+  }
+}
+
+}  // namespace
+
+bool encode_wide_maps(CUtensorMap (&m)[3], const void* x, int cols, int cap) {
+  for (int i = 0; i < 3; ++i)
+    if (!encode_split_map(&m[i], x, cols, cap, 32 << i)) return false;
+  return true;
+}
+
+cudaError_t prepare_wide_kernels() {
+  cudaError_t e;
+  if ((e = wide_prep_all<32>()) != cudaSuccess) return e;
+  if ((e = wide_prep_all<64>()) != cudaSuccess) return e;
+  if ((e = wide_prep_all<128>()) != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_attn_wide, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)kAWSmem);
+}
+
+// Work of one layer of a chunk of M rows on the busiest SM (stage cycles).
+long long wide_layer_cost(const Dims& D, int M) {
+  auto mat = [&](int N, int K, bool pairs) {
+    long long c;
+    pick_tile(D.num_sms, row_tiles(N, pairs), M, &c);
+    return c * ((K + kWK - 1) / kWK);
+  };
+  return mat((D.Hq + 2 * D.Hkv) * D.hd, D.d, false) + mat(D.d, D.qd, false) +
+         mat(2 * D.F, D.d, true) + mat(D.d, D.F, false);
+}
+
+cudaError_t launch_embed_wide(const Dims& D, const Bufs& B, const WideBufs& P, const void* embed,
+                              const void* gnorm, const int32_t* toks, int M, cudaStream_t st) {
+  return launch_ex(k_embed_wide, dim3(M), dim3(256), 0, st, D, B, P,
+                   static_cast<const __nv_bfloat16*>(embed),
+                   static_cast<const __nv_bfloat16*>(gnorm), toks);
+}
+
+cudaError_t launch_take_rows(const Dims& D, const Bufs& B, const WideBufs& P, int row0, int M,
+                             cudaStream_t st) {
+  return launch_ex(k_take_rows, dim3(M), dim3(256), 0, st, D, B, P, row0);
+}
+
+cudaError_t launch_layer_wide(const Dims& D, const Bufs& B, const WideBufs& P, const WideMaps& xm,
+                              const LayerW& w, const void* next_norm, int layer, int M, int pos0,
+                              cudaStream_t st) {
+  float* ss[2] = {P.ss, P.ss + (size_t)((D.d + kWR - 1) / kWR) * P.cap};
+  WArgs a{};
+  a.D = D;
+  a.B = B;
+  a.P = P;
+  a.M = M;
+  a.pos0 = pos0;
+  a.layer = layer;
+  cudaError_t e;
+  // RMSNorm + QKV + RoPE + KV rows
+  a.N = (D.Hq + 2 * D.Hkv) * D.hd;
+  a.K = D.d;
+  a.ss_in = ss[0];
+  if ((e = wide_launch<kWQkv>(*w.tm[0], xm.xn, a, st)) != cudaSuccess) return e;
+  if ((e = launch_ex(k_attn_wide, dim3(D.Hq, (M + kAQ - 1) / kAQ), dim3(kAWThreads), kAWSmem, st, D,
+                     B, P, layer, M, pos0)) != cudaSuccess)
+    return e;
+  // O projection + residual
+  a.N = D.d;
+  a.K = D.qd;
+  a.ss_in = nullptr;
+  a.ss_out = ss[1];
+  a.gnext = static_cast<const __nv_bfloat16*>(w.ffn_norm);
+  if ((e = wide_launch<kWResid>(*w.tm[1], xm.xo, a, st)) != cudaSuccess) return e;
+  // RMSNorm + gate/up + SwiGLU
+  a.N = 2 * D.F;
+  a.K = D.d;
+  a.ss_in = ss[1];
+  if ((e = wide_launch<kWGateUp>(*w.tm[2], xm.xn, a, st)) != cudaSuccess) return e;
+  // down projection + residual
+  a.N = D.d;
+  a.K = D.F;
+  a.ss_in = nullptr;
+  a.ss_out = ss[0];
+  a.gnext = static_cast<const __nv_bfloat16*>(next_norm);
+  return wide_launch<kWResid>(*w.tm[3], xm.xa, a, st);
+}
+
+}  // namespace ssd
