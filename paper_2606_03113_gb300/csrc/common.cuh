@@ -174,9 +174,9 @@ struct Bufs {
   float* draft_logits;     // [kMaxDraft][V] exit logits of each draft (sampled decoding)
   float* attn_out;   // [kMaxM][qd]
   float* act;        // [kMaxM][F]
-  float* logits;     // [kMaxM][V] (written only when requested)
-  void* head_part;   // [2][max blocks][kMaxM] per-block (running, split) statistics
-  uint32_t* head_counter;  // block ticket of the exit head
+  float* logits;     // [kMaxM][V] of the last exit head
+  void* head_part;   // [kMaxM][kHeadParts] statistics of a row's chunks
+  uint32_t* head_counter;  // [kMaxM] chunk tickets of the exit-head statistics
   RowStats* stats;   // [kMaxM]
   float2* rope;      // [max_seq][hd/2] (cos, sin)
   void* kv;          // [L][2][Hkv][max_seq][hd]

@@ -87,8 +87,8 @@ size_t layout(const ssd_model_cfg& c, char* base, Dims* D, Bufs* B, WideBufs* P)
   b.act = cv.take<float>(sizeof(float) * kMaxM * d.F);
   b.logits = cv.take<float>(sizeof(float) * kMaxM * (size_t)d.V);
   b.draft_logits = cv.take<float>(sizeof(float) * kMaxDraft * (size_t)d.V);
-  b.head_part = cv.take<void>(sizeof(HeadPart) * kMaxM * 2 * (size_t)kMaxBlocks);
-  b.head_counter = cv.take<uint32_t>(sizeof(uint32_t));
+  b.head_part = cv.take<void>(sizeof(HeadPart) * kMaxM * (size_t)kHeadParts);
+  b.head_counter = cv.take<uint32_t>(sizeof(uint32_t) * kMaxM);
   b.stats = cv.take<RowStats>(sizeof(RowStats) * kMaxM);
   b.rope = cv.take<float2>(sizeof(float2) * (size_t)d.max_seq * (d.hd / 2));
   b.kv = cv.take<void>(elt * (size_t)d.L * 2 * d.Hkv * (size_t)d.max_seq * d.hd);
@@ -158,7 +158,6 @@ struct ssd_ctx {
   std::vector<int> cand;
   int kmax = 0, static_l = 0, static_k = 0, q_hidden = 0, trace_T = 20, topk = 5, fixed_k = 0;
   int q_in = 3;
-  bool sampled = false;  // temperature > 0: the exit heads write their logits
   // graphs
   cudaGraph_t round_g = nullptr, gen_g = nullptr;
   cudaGraphExec_t round_x = nullptr, gen_x = nullptr;
@@ -269,10 +268,9 @@ cudaError_t enqueue_layers(ssd_ctx* x, int l_from, int l_to, RowSel sel, int mro
   return cudaSuccess;
 }
 
-cudaError_t enqueue_head(ssd_ctx* x, RowSel sel, int mrows, int topk, bool logits,
-                         cudaStream_t st) {
+cudaError_t enqueue_head(ssd_ctx* x, RowSel sel, int mrows, int topk, cudaStream_t st) {
   return launch_head(x->D, x->B, x->cfg.dtype, x->lm_head, lm_map(x), tile_maps(x), x->final_norm,
-                     topk, logits, sel, mrows, st);
+                     topk, sel, mrows, st);
 }
 
 // Walk segment j: layers (done, c_j], exit head, decision; nested IF for j+1.
@@ -284,7 +282,7 @@ cudaError_t build_walk(ssd_ctx* x, Seq& s, const std::vector<int>& cands, int j,
   GK(s.begin());
   if (j == 0) GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, rows(kRowsWalk), false, 0, x->cap));
   GK(enqueue_layers(x, done, cands[j], rows(kRowsWalk), 1, x->cap));
-  GK(enqueue_head(x, rows(kRowsWalk), 1, x->topk, x->sampled, x->cap));
+  GK(enqueue_head(x, rows(kRowsWalk), 1, x->topk, x->cap));
   GK(launch_decide(x->D, x->B, kDecideWalk, j, last ? 1 : 0, cands[j], x->final_norm,
                    x->cfg.dtype, next, 0, x->cap));
   GK(s.end());
@@ -329,7 +327,7 @@ cudaError_t build_draft_phase(ssd_ctx* x, cudaGraph_t body) {
     GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, rows(kRowsDraft), false, 0, x->cap));
     GK(enqueue_layers(x, 0, cands[0], rows(kRowsDraft), 1, x->cap));
   }
-  GK(enqueue_head(x, rows(kRowsDraft), 1, x->topk, x->sampled, x->cap));
+  GK(enqueue_head(x, rows(kRowsDraft), 1, x->topk, x->cap));
   GK(launch_decide(x->D, x->B, kDecideDraft, 0, 0, 0, x->final_norm, x->cfg.dtype, 0, hw,
                    x->cap));
   return w.end();
@@ -354,7 +352,7 @@ cudaError_t build_round(ssd_ctx* x, cudaGraph_t g, cudaGraphConditionalHandle ge
   GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, rows(kRowsVerify), spec, 0, x->cap));
   const int mrows = spec ? std::min(x->kmax + 1, kMaxM) : 1;
   GK(enqueue_layers(x, 0, x->D.L, rows(kRowsVerify), mrows, x->cap));
-  GK(enqueue_head(x, rows(kRowsVerify), mrows, x->topk, x->sampled, x->cap));
+  GK(enqueue_head(x, rows(kRowsVerify), mrows, x->topk, x->cap));
   GK(launch_accept(x->D, x->B, gen, x->cap));
   return s.end();
 }
@@ -442,7 +440,7 @@ ssd_status run_prompt_wide(ssd_ctx* x, int n, int* last_row) {
       const int m = std::min(kPrefillChunk, M - r);
       CK(x, launch_take_rows(x->D, x->B, x->P, r, m, x->stream));
       CK(x, enqueue_head(x, rows_explicit(c0 + r, m, x->B.pre_tok + c0 + r), kPrefillChunk, x->topk,
-                         x->sampled, x->stream));
+                         x->stream));
       CK(x, launch_trace_push(x->B, 0, m, x->stream));
       *last_row = m - 1;
       r += m;
@@ -466,7 +464,7 @@ ssd_status run_prompt(ssd_ctx* x, int n, int* last_row) {
     CK(x, launch_embed(x->D, x->B, x->cfg.dtype, x->embed, sel, true, 0, x->stream));
     CK(x, enqueue_layers(x, 0, x->D.L, sel, kPrefillChunk, x->stream));
     if (c0 + M > n - T || c0 + M == n) {
-      CK(x, enqueue_head(x, sel, kPrefillChunk, x->topk, x->sampled, x->stream));
+      CK(x, enqueue_head(x, sel, kPrefillChunk, x->topk, x->stream));
       const int first = std::max(c0, n - T) - c0;
       if (first < M) CK(x, launch_trace_push(x->B, first, M - first, x->stream));
     }
@@ -603,7 +601,7 @@ ssd_status ssd_init_model(const ssd_model_cfg* cfg, const ssd_weights* w, void* 
   e = cudaMemcpyAsync(x->B.rope, rope.data(), sizeof(float2) * rope.size(), cudaMemcpyHostToDevice,
                       x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->B.ctl, 0, sizeof(Ctl), x->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(x->B.head_counter, 0, sizeof(uint32_t), x->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(x->B.head_counter, 0, sizeof(uint32_t) * kMaxM, x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->B.ss, 0, sizeof(float) * 2 * kMaxM, x->stream);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(x->B.ss_part, 0, sizeof(float) * 2 * (size_t)x->D.ss_nt * kMaxM, x->stream);
@@ -687,13 +685,12 @@ ssd_status ssd_set_policy(ssd_ctx* x, const ssd_policy* p) {
                           cudaMemcpyHostToDevice, x->stream));
   CK(x, cudaStreamSynchronize(x->stream));
   // The graphs depend on the policy kind, the candidate (or static) exit
-  // layers, kmax, topk and whether the heads write logits; everything else
-  // is read on the device from the policy just copied.
+  // layers, kmax and topk; everything else is read on the device from the
+  // policy just copied.
   const int kmax_new = p->kind == SSD_POLICY_AR ? 0 : p->kmax;
-  const bool sampled = p->temperature > 0.f;
   const bool same_graphs = x->have_policy && x->kind == p->kind && x->cand == cand &&
                            x->kmax == kmax_new && x->static_l == p->static_l &&
-                           x->topk == dp.topk && x->sampled == sampled;
+                           x->topk == dp.topk;
   x->kind = p->kind;
   x->cand = cand;
   x->kmax = kmax_new;
@@ -704,7 +701,6 @@ ssd_status ssd_set_policy(ssd_ctx* x, const ssd_policy* p) {
   x->q_in = dp.q_in;
   x->trace_T = dp.trace_T;
   x->topk = dp.topk;
-  x->sampled = sampled;
   if (same_graphs) return SSD_OK;
   cudaError_t e = build_graphs(x);
   if (e != cudaSuccess) {
@@ -886,7 +882,7 @@ ssd_status ssd_forward_exit(ssd_ctx* x, const int32_t* ids, int32_t M, int32_t p
   const RowSel sel = rows_explicit(pos0, M, x->B.pre_tok);
   CK(x, launch_embed(x->D, x->B, x->cfg.dtype, x->embed, sel, true, 0, x->stream));
   CK(x, enqueue_layers(x, 0, l_exit, sel, M, x->stream));
-  CK(x, enqueue_head(x, sel, M, topk, logits != nullptr, x->stream));
+  CK(x, enqueue_head(x, sel, M, topk, x->stream));
   std::vector<RowStats> st(M);
   CK(x, cudaMemcpyAsync(st.data(), x->B.stats, sizeof(RowStats) * M, cudaMemcpyDeviceToHost,
                         x->stream));
@@ -1006,7 +1002,7 @@ ssd_status ssd_op_layer(ssd_ctx* x, int32_t kernel, int32_t layer, int32_t M, in
   cudaStream_t st = stream ? static_cast<cudaStream_t>(stream) : x->stream;
   const RowSel sel = rows_explicit(pos0, M, x->B.pre_tok);
   if (kernel == 5)
-    CK(x, enqueue_head(x, sel, M, x->topk, false, st));
+    CK(x, enqueue_head(x, sel, M, x->topk, st));
   else if (kernel == 6)
     CK(x, launch_tile_chain(x->D, x->B, *tile_maps(x), x->layers[layer],
                             layer + 1 < x->cfg.n_layers ? &x->layers[layer + 1] : nullptr, layer,

@@ -31,7 +31,6 @@
 #include <mutex>
 #include <type_traits>
 
-#include "headpart.cuh"
 #include "kernels.h"
 #include "pipe.cuh"
 
@@ -120,7 +119,7 @@ struct SmemLayout {
   static constexpr size_t rs = bars + 2 * kNS * sizeof(uint64_t);
   static constexpr size_t flag = rs + sizeof(float) * 32;
   static constexpr size_t scratch = flag + 64;  // cross-warp combine buffer
-  static constexpr size_t red = scratch + (size_t)(kCWarps + 1) * kMaxM * sizeof(HeadPart);
+  static constexpr size_t red = scratch + (size_t)kCWarps * kMaxM * sizeof(float);
   template <int MM>
   static constexpr size_t total() {  // + tensor-core partial sums [4 K-quarters][32][8 kNB]
     return red + sizeof(float) * 4 * kRT * 8 * kNB;
@@ -140,7 +139,7 @@ __device__ inline bool has_split_slot(const Geom& g, int b) {
 struct Shared {
   float* rs;       // [MM] input RMSNorm scale
   int* flag;
-  void* scratch;   // [kCWarps][MM] floats or HeadParts
+  float* scratch;  // [kCWarps][kMaxM]
 };
 
 // ------------------------------------------------------------ epilogues
@@ -233,7 +232,7 @@ struct EpiGateUp {
 // Combines the per-lane float state of the 8 warps (lane m of each) in warp
 // order; every consumer thread calls it; returns the sum in thread m < M.
 __device__ inline float combine_warps(float v, const Shared& sh, int tid, int M) {
-  float* buf = static_cast<float*>(sh.scratch);
+  float* buf = sh.scratch;
   const int warp = tid >> 5, lane = tid & 31;
   if (lane < M) buf[warp * kMaxM + lane] = v;
   named_sync(1, kCThreads);
@@ -287,7 +286,7 @@ struct EpiResid {
     if (!*sh.flag) return;
     __threadfence();
     // every thread loads its slots first, then a fixed reduction tree
-    float* buf = static_cast<float*>(sh.scratch);
+    float* buf = sh.scratch;
     const int warp = tid >> 5, lane = tid & 31;
     for (int m = 0; m < M; ++m) {
       float v = 0.f;
@@ -309,101 +308,18 @@ struct EpiResid {
   }
 };
 
-// Merges the per-lane statistics of the 8 warps (lane m of each) with a
-// fixed shuffle tree and leaves row m's result in out[m] (shared memory).
-__device__ inline void combine_parts(const HeadPart& p, const Shared& sh, int tid, int M,
-                                     HeadPart* out) {
-  HeadPart* buf = static_cast<HeadPart*>(sh.scratch);
-  const int warp = tid >> 5, lane = tid & 31;
-  if (lane < M) buf[warp * kMaxM + lane] = p;
-  named_sync(1, kCThreads);
-  for (int m = warp; m < M; m += kCWarps) {
-    HeadPart q;
-    if (lane < kCWarps)
-      q = buf[lane * kMaxM + m];
-    else
-      part_empty(q);
-    for (int off = 4; off > 0; off >>= 1) part_merge(q, part_shfl(q, off));
-    if (lane == 0) out[m] = q;
-  }
-  named_sync(1, kCThreads);
-}
-
-// Exit head: z = W_lm RMSNorm_final(h).  Lane m keeps running statistics of
-// the logits it produced (max, sum exp, sum exp*(z-max), top-k); per block
-// they are merged in warp order, and the last block merges the blocks (and
-// the split slots) in a fixed shuffle tree, giving argmax (lowest id on
-// ties), log-sum-exp, entropy H = log S - T/S, C_k = lse - mean(top-k
-// logits) and pmax = 1/S.
+// Exit head: z = W_lm RMSNorm_final(h); k_head_stats reads the logits back.
 struct EpiHead {
-  struct State {
-    HeadPart p;
-  };
-  int topk, write_logits;
-  __device__ void init(State& s) const { part_empty(s.p); }
+  using State = NoState;
+  __device__ void init(State&) const {}
   __device__ void pair(const StreamArgs& a, int tile, int w, int m, int, float rs, float v0,
-                       float v1, State& st) const {
+                       float v1, State&) const {
     const int r0 = map_row(a.g, a.D, tile, w), r1 = map_row(a.g, a.D, tile, w + 16);
-    if (r0 >= 0) {
-      const float z = v0 * rs;
-      part_add(st.p, z, r0);
-      if (write_logits) a.B.logits[(size_t)m * a.D.V + r0] = z;
-    }
-    if (r1 >= 0) {
-      const float z = v1 * rs;
-      part_add(st.p, z, r1);
-      if (write_logits) a.B.logits[(size_t)m * a.D.V + r1] = z;
-    }
+    if (r0 >= 0) a.B.logits[(size_t)m * a.D.V + r0] = v0 * rs;
+    if (r1 >= 0) a.B.logits[(size_t)m * a.D.V + r1] = v1 * rs;
   }
-  __device__ HeadPart* slots(const StreamArgs& a) const {
-    return static_cast<HeadPart*>(a.B.head_part);
-  }
-  __device__ void split_done(const StreamArgs& a, int b0, State& st, const Shared& sh, int tid,
-                             int M) const {
-    HeadPart* out = static_cast<HeadPart*>(sh.scratch) + kCWarps * kMaxM;
-    combine_parts(st.p, sh, tid, M, out);
-    if (tid < M) slots(a)[((size_t)kMaxBlocksDev + b0) * kMaxM + tid] = out[tid];
-  }
-  __device__ void finish(const StreamArgs& a, State& st, const Shared& sh, int tid, int M) const {
-    HeadPart* out = static_cast<HeadPart*>(sh.scratch) + kCWarps * kMaxM;
-    combine_parts(st.p, sh, tid, M, out);
-    HeadPart* sl = slots(a);
-    if (tid < M) sl[(size_t)blockIdx.x * kMaxM + tid] = out[tid];
-    __threadfence();
-    named_sync(1, kCThreads);
-    if (tid == 0) *sh.flag = atomicAdd(a.B.head_counter, 1u) == (unsigned)(a.g.P - 1);
-    named_sync(1, kCThreads);
-    if (!*sh.flag) return;
-    __threadfence();
-    // every thread merges its slots, then a fixed shuffle tree per warp and
-    // one over the eight warp results
-    HeadPart* buf = static_cast<HeadPart*>(sh.scratch);
-    const int warp = tid >> 5, lane = tid & 31;
-    for (int m = 0; m < M; ++m) {
-      HeadPart p;
-      part_empty(p);
-      for (int b = tid; b < a.g.P; b += kCThreads) {
-        part_merge(p, part_load_cg(&sl[(size_t)b * kMaxM + m]));
-        if (has_split_slot(a.g, b)) part_merge(p, part_load_cg(&sl[((size_t)kMaxBlocksDev + b) * kMaxM + m]));
-      }
-      for (int off = 16; off > 0; off >>= 1) part_merge(p, part_shfl(p, off));
-      if (lane == 0) buf[warp] = p;
-      named_sync(1, kCThreads);
-      if (warp == 0) {
-        HeadPart f;
-        if (lane < kCWarps)
-          f = buf[lane];
-        else
-          part_empty(f);
-        for (int off = 4; off > 0; off >>= 1) part_merge(f, part_shfl(f, off));
-        if (lane == 0) {
-          write_row_stats(a.B.stats[m], f, topk);
-        }
-      }
-      named_sync(1, kCThreads);
-    }
-    if (tid == 0) *a.B.head_counter = 0u;
-  }
+  __device__ void split_done(const StreamArgs&, int, State&, const Shared&, int, int) const {}
+  __device__ void finish(const StreamArgs&, State&, const Shared&, int, int) const {}
 };
 
 // ------------------------------------------------------------ the kernel
@@ -468,7 +384,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_stream(const StreamArgs a, cons
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + SmemLayout::bars);
   uint64_t* empty = full + kNS;
   const Shared sh{reinterpret_cast<float*>(smem + SmemLayout::rs),
-                  reinterpret_cast<int*>(smem + SmemLayout::flag), smem + SmemLayout::scratch};
+                  reinterpret_cast<int*>(smem + SmemLayout::flag), reinterpret_cast<float*>(smem + SmemLayout::scratch)};
 
   const Geom& g = a.g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -927,8 +843,8 @@ cudaError_t launch_layer(const Dims& D, const Bufs& B, int dtype, const LayerW& 
 }
 
 template <typename T, int MM>
-static cudaError_t head_t(const Dims& D, const Bufs& B, const void* lm, const void* fn, int topk,
-                          bool logits, RowSel sel, cudaStream_t st) {
+static cudaError_t head_t(const Dims& D, const Bufs& B, const void* lm, const void* fn, RowSel sel,
+                          cudaStream_t st) {
   StreamArgs a{};
   a.D = D;
   a.B = B;
@@ -938,18 +854,21 @@ static cudaError_t head_t(const Dims& D, const Bufs& B, const void* lm, const vo
   a.gnorm = fn;
   a.x = B.h;
   a.ss_in = 0;
-  return stream_launch<T, MM, true>(a, EpiHead{topk, logits ? 1 : 0}, st);
+  return stream_launch<T, MM, true>(a, EpiHead{}, st);
 }
 
 cudaError_t launch_head(const Dims& D, const Bufs& B, int dtype, const void* lm_head,
                         const CUtensorMap* lm_map, const TileMaps* tm, const void* final_norm,
-                        int topk, bool write_logits, RowSel sel, int mrows, cudaStream_t st) {
+                        int topk, RowSel sel, int mrows, cudaStream_t st) {
+  cudaError_t e;
   if (dtype == SSD_DTYPE_BF16) {
     if (!tm || !lm_map) return cudaErrorInvalidValue;
-    return launch_tile_head(D, B, *tm, *lm_map, final_norm, topk, write_logits, sel, mrows, st);
+    e = launch_tile_head(D, B, *tm, *lm_map, final_norm, sel, mrows, st);
+  } else {
+    e = mrows > 1 ? head_t<float, kMaxM>(D, B, lm_head, final_norm, sel, st)
+                  : head_t<float, 1>(D, B, lm_head, final_norm, sel, st);
   }
-  return mrows > 1 ? head_t<float, kMaxM>(D, B, lm_head, final_norm, topk, write_logits, sel, st)
-                   : head_t<float, 1>(D, B, lm_head, final_norm, topk, write_logits, sel, st);
+  return e != cudaSuccess ? e : launch_head_stats(D, B, topk, sel, mrows, st);
 }
 
 template <typename T, int MM>

@@ -5,14 +5,16 @@
 
 namespace ssd {
 
-// Statistics partial of one block of vocabulary rows (exit head, first stage).
+// Statistics of one chunk of a row's logits (exit head), merged by the row's
+// last chunk.
 struct HeadPart {
-  float mx;  // max logit (== tv[0] when the block has rows)
+  float mx;  // max logit
   float S;   // sum exp(z - mx)
   float T;   // sum exp(z - mx) (z - mx)
   float tv[kTopK];
   int32_t ti[kTopK];
 };
+constexpr int kHeadParts = 256;  // chunks of a row, at most
 
 // Per-block partial slots of the streamed kernels (running + split), for up
 // to kMaxBlocks blocks.
@@ -43,8 +45,8 @@ cudaError_t launch_tile_chain(const Dims& D, const Bufs& B, const TileMaps& tm, 
                               const LayerW* next, int layer, RowSel sel, int mrows,
                               cudaStream_t st);
 cudaError_t launch_tile_head(const Dims& D, const Bufs& B, const TileMaps& tm,
-                             const CUtensorMap& lm, const void* final_norm, int topk,
-                             bool write_logits, RowSel sel, int mrows, cudaStream_t st);
+                             const CUtensorMap& lm, const void* final_norm, RowSel sel, int mrows,
+                             cudaStream_t st);
 cudaError_t launch_tile_plain(const Dims& D, const Bufs& B, const CUtensorMap& wm, int rows,
                               int cols, const float* x, int M, float* y, cudaStream_t st);
 
@@ -83,7 +85,9 @@ cudaError_t launch_layer_part(const Dims& D, const Bufs& B, int dtype, const Lay
                               cudaStream_t st);
 cudaError_t launch_head(const Dims& D, const Bufs& B, int dtype, const void* lm_head,
                         const CUtensorMap* lm_map, const TileMaps* tm, const void* final_norm,
-                        int topk, bool write_logits, RowSel sel, int mrows, cudaStream_t st);
+                        int topk, RowSel sel, int mrows, cudaStream_t st);
+cudaError_t launch_head_stats(const Dims& D, const Bufs& B, int topk, RowSel sel, int mrows,
+                              cudaStream_t st);
 cudaError_t launch_round_begin(const Dims& D, const Bufs& B, cudaGraphConditionalHandle draft_if,
                                cudaStream_t st);
 cudaError_t launch_decide(const Dims& D, const Bufs& B, int mode, int cand_idx, int is_last,

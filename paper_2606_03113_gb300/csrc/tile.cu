@@ -35,7 +35,6 @@
 #include <mutex>
 #include <type_traits>
 
-#include "headpart.cuh"
 #include "kernels.h"
 #include "pipe.cuh"
 #include "tc.cuh"
@@ -65,10 +64,10 @@ constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // in rows TP..2TP-1).  Every ring slot holds a unit's weights, its operand
 // tile and its input slice, all released by the one commit of the unit's
 // MMAs.
-template <int TP, bool HEAD>
+template <int TP>
 struct TL {
   static constexpr int N = 2 * TP;
-  static constexpr int NS = TP == 24 ? 4 : (TP == 8 && !HEAD ? 6 : 5);  // ring depth
+  static constexpr int NS = TP == 24 ? 4 : (TP == 8 ? 6 : 5);  // ring depth
   static constexpr int XB = TP * kKC * 4;                   // input box: TP rows x 64 fp32
   static constexpr int XS = (int)align_up(XB + kKC * 2, 128);  // + RMSNorm weight slice
   static constexpr int BB = N * 128;                        // operand tile (multiple of 1024)
@@ -83,11 +82,7 @@ struct TL {
   static constexpr size_t flag = tslot + 8;
   static constexpr size_t rs = flag + 8;
   static constexpr size_t red = rs + 4 * 32;
-  // exit-head statistics (running, split tile, merge), only in the head's instances
-  static constexpr size_t run = align_up(red + 4 * (size_t)kWorkers * kLT, 16);
-  static constexpr size_t spl = run + (HEAD ? sizeof(HeadPart) * kWorkers * kLT : 0);
-  static constexpr size_t comb = spl + (HEAD ? sizeof(HeadPart) * kWorkers * kLT : 0);
-  static constexpr size_t used = comb + (HEAD ? sizeof(HeadPart) * kMaxM : 0);
+  static constexpr size_t used = red + 4 * (size_t)kWorkers * kLT;
   static constexpr size_t total = used + 1024;  // the base is aligned up to 1024 in the kernel
   static_assert(total <= 227 * 1024, "shared memory budget");
   static_assert(BB % 1024 == 0 && XS % 128 == 0, "operand / slice alignment");
@@ -111,7 +106,6 @@ struct TArgs {
   RowSel sel;
   int layer;                   // QKV: KV-cache layer
   int which;                   // residual: sum-of-squares buffer written
-  int topk, write_logits;      // exit head
   float* y;                    // plain product output [M][N]
 };
 
@@ -127,16 +121,6 @@ __device__ inline int t_block_of(const TGeom& g, int s) {
   while (b + 1 < g.P && t_start(g, b + 1) <= s) ++b;
   while (b > 0 && t_start(g, b) > s) --b;
   return b;
-}
-
-// Block b owns the split slot of the tile it starts and shares with the next
-// block(s), if its last tile is such a tile.
-__device__ inline bool t_has_split_slot(const TGeom& g, int b) {
-  const int sb = t_start(g, b), se = t_start(g, b + 1);
-  if (se <= sb) return false;
-  const int t = (se - 1) / g.nks;
-  if ((t + 1) * g.nks <= se) return false;
-  return t * g.nks >= sb;
 }
 
 // Global row of stage row s (0..255) of a tile, or -1 past the end.
@@ -197,6 +181,10 @@ __device__ __forceinline__ void t_pair(const TArgs& a, int tile, int s, int t, i
     const int r0 = trow(a.g, tile, s), r1 = trow(a.g, tile, s + 128);
     if (r0 >= 0) a.y[(size_t)t * a.g.N + r0] = v0;
     if (r1 >= 0) a.y[(size_t)t * a.g.N + r1] = v1;
+  } else if constexpr (KIND == kKHead) {
+    const int r0 = trow(a.g, tile, s), r1 = trow(a.g, tile, s + 128);
+    if (r0 >= 0) a.B.logits[(size_t)t * D.V + r0] = v0 * rs;
+    if (r1 >= 0) a.B.logits[(size_t)t * D.V + r1] = v1 * rs;
   } else if constexpr (KIND == kKQKV) {
     // rotary embedding of the pair (i, i + hd/2) of a query / key head
     // (angle pos * theta^(-2i/hd) from the table), or two value rows
@@ -269,28 +257,6 @@ __device__ __forceinline__ void t_resid_pre(const TArgs& a, int tile, int s, int
   }
 }
 
-// Exit head, one token, whole warp: the logits of the lane's two rows enter
-// a per-lane partial, merged over the warp by a fixed shuffle tree; lane 0
-// merges the result into `acc` (shared memory, one slot per warp and token).
-__device__ __forceinline__ void t_head_token(const TArgs& a, int tile, int s, int t, float rs,
-                                             float v0, float v1, HeadPart* acc, int lane) {
-  const int r0 = trow(a.g, tile, s), r1 = trow(a.g, tile, s + 128);
-  HeadPart p;
-  part_empty(p);
-  if (r0 >= 0) {
-    const float z = v0 * rs;
-    part_add(p, z, r0);
-    if (a.write_logits) a.B.logits[(size_t)t * a.D.V + r0] = z;
-  }
-  if (r1 >= 0) {
-    const float z = v1 * rs;
-    part_add(p, z, r1);
-    if (a.write_logits) a.B.logits[(size_t)t * a.D.V + r1] = z;
-  }
-  for (int off = 16; off > 0; off >>= 1) part_merge(p, part_shfl(p, off));
-  if (lane == 0) part_merge(*acc, p);
-}
-
 }  // namespace
 
 // ------------------------------------------------------------ the kernels
@@ -307,16 +273,15 @@ __device__ __forceinline__ bool counter_wait(const uint32_t* bar, uint32_t targe
 }
 
 
-// Shared-memory views of one block (layout TL<TP, HEAD>).
-template <int TP, bool HEAD>
+// Shared-memory views of one block (layout TL<TP>).
+template <int TP>
 struct Blk {
-  using S = TL<TP, HEAD>;
+  using S = TL<TP>;
   unsigned char* smem;
   uint64_t *full, *xfull, *empty, *bfull, *accfull, *accempty, *drain;
   uint32_t* tslot;
   int* sflag;
   float *srs, *red;
-  HeadPart *run, *spl, *comb;
 
   __device__ explicit Blk(unsigned char* raw) {
     smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(raw) + 1023) &
@@ -332,9 +297,6 @@ struct Blk {
     sflag = reinterpret_cast<int*>(smem + S::flag);
     srs = reinterpret_cast<float*>(smem + S::rs);
     red = reinterpret_cast<float*>(smem + S::red);
-    run = reinterpret_cast<HeadPart*>(smem + S::run);
-    spl = reinterpret_cast<HeadPart*>(smem + S::spl);
-    comb = reinterpret_cast<HeadPart*>(smem + S::comb);
   }
 
   // barriers (thread 0), TMEM allocation (the MMA warp); every thread waits
@@ -360,12 +322,10 @@ struct Blk {
     return *tslot;
   }
 
-  // workers: zeroed operand tiles (rows past M stay zero), empty statistics
+  // workers: zeroed operand tiles (rows past M stay zero)
   __device__ void clear_operands(int tid) {
     uint4* z = reinterpret_cast<uint4*>(smem + S::bt);
     for (int i = tid; i < S::NS * S::BB / 16; i += kWThreads) z[i] = make_uint4(0, 0, 0, 0);
-    if constexpr (HEAD)
-      for (int i = tid; i < kWorkers * kLT; i += kWThreads) part_empty(run[i]);
     fence_proxy_async_smem();
     named_sync(1, kWThreads);
   }
@@ -376,10 +336,10 @@ struct Blk {
 // parts as one N = 2 TP operand.  gi0 is the block's count of units before
 // this matrix (ring slot and phase parity continue across the matrices of a
 // chain), tc the running tile count (double-buffered TMEM accumulator).
-template <int TP, bool HEAD>
-__device__ bool mma_units(const Blk<TP, HEAD>& k, const TGeom& g, int u_begin, int n, int gi0,
+template <int TP>
+__device__ bool mma_units(const Blk<TP>& k, const TGeom& g, int u_begin, int n, int gi0,
                           int& tc, uint32_t tmem) {
-  using S = TL<TP, HEAD>;
+  using S = TL<TP>;
   constexpr int NS = S::NS, N = S::N;
   constexpr uint32_t idesc = idesc_bf16_f32(128, N);
   for (int i = 0; i < n; ++i) {
@@ -414,9 +374,9 @@ __device__ bool mma_units(const Blk<TP, HEAD>& k, const TGeom& g, int u_begin, i
 // from the input slices, then the fused epilogue of every tile.  The RMSNorm
 // scale of the input rows is read first (from the sum-of-squares parts).
 template <int TP, int KIND, bool NORM>
-__device__ void worker_units(const TArgs& a, const Blk<TP, KIND == kKHead>& k, uint32_t tmem,
+__device__ void worker_units(const TArgs& a, const Blk<TP>& k, uint32_t tmem,
                              int u_begin, int n, int gi0, int& tc, bool& ok, int pos0, int M) {
-  using S = TL<TP, KIND == kKHead>;
+  using S = TL<TP>;
   constexpr int NS = S::NS, N = S::N;
   constexpr int LTN = TP / 2;                 // tokens per parity group read back
   constexpr int LTR = LTN < kLT ? LTN : kLT;  // ... of which can be rows (t < kMaxM)
@@ -425,8 +385,6 @@ __device__ void worker_units(const TArgs& a, const Blk<TP, KIND == kKHead>& k, u
   float* srs = k.srs;
   float* red = k.red;
   int* sflag = k.sflag;
-  HeadPart* run = k.run;
-  HeadPart* spl = k.spl;
   if (tid < 32) {
     // RMSNorm scale of row tid: the input's sum of squares is kept as parts
     // of 256 elements, added here in part order
@@ -510,10 +468,7 @@ __device__ void worker_units(const TArgs& a, const Blk<TP, KIND == kKHead>& k, u
         if (t >= M) break;
         const float v0 = grp ? v[0][2 * lt + 1] : v[0][2 * lt];
         const float v1 = grp ? v[1][2 * lt + 1] : v[1][2 * lt];
-        if constexpr (KIND == kKHead)
-          t_head_token(a, tile, srow, t, rs_t[lt], v0, v1, &run[warp * kLT + lt], lane);
-        else
-          t_pair<KIND>(a, tile, srow, t, pos0, rs_t[lt], v0, v1, ssv[lt]);
+        t_pair<KIND>(a, tile, srow, t, pos0, rs_t[lt], v0, v1, ssv[lt]);
       }
       if constexpr (KIND == kKResid) tile_ss(ssv, tile);
       return;
@@ -562,11 +517,6 @@ __device__ void worker_units(const TArgs& a, const Blk<TP, KIND == kKHead>& k, u
     float ss_sp[LTN];
 #pragma unroll
     for (int lt = 0; lt < LTN; ++lt) ss_sp[lt] = 0.f;
-    if constexpr (KIND == kKHead) {
-      if (lane == 0)
-        for (int lt = 0; lt < kLT; ++lt) part_empty(spl[warp * kLT + lt]);
-      __syncwarp();
-    }
     // Partial sums of the contributors, added in block order (independent of
     // who finishes last).  The loads of several contributors (and all
     // tokens) are issued before any is used, so the fix-up costs a few L2
@@ -642,27 +592,13 @@ __device__ void worker_units(const TArgs& a, const Blk<TP, KIND == kKHead>& k, u
     for (int lt = 0; lt < LTN; ++lt) {
       const int t = 2 * lt + grp;
       if (t >= M) break;
-      if constexpr (KIND == kKHead)
-        t_head_token(a, tile, srow, t, rs_t[lt], u0[lt], u1[lt], &spl[warp * kLT + lt], lane);
-      else if constexpr (KIND == kKResid)
+      if constexpr (KIND == kKResid)
         t_resid_pre(a, tile, srow, t, u0[lt], u1[lt], hp0[lt], hp1[lt], ss_sp[lt]);
       else
         t_pair<KIND>(a, tile, srow, t, pos0, rs_t[lt], u0[lt], u1[lt], ss_sp[lt]);
     }
-    // the split tile's statistics: residual sums of squares as the tile's
-    // part; exit-head statistics to the split slot of its first block
-    if constexpr (KIND == kKResid) {
-      tile_ss(ss_sp, tile);
-    } else if constexpr (KIND == kKHead) {
-      named_sync(1, kWThreads);
-      if (tid < M) {
-        HeadPart p;
-        part_empty(p);
-        for (int qq = 0; qq < 4; ++qq) part_merge(p, spl[((tid & 1) * 4 + qq) * kLT + (tid >> 1)]);
-        static_cast<HeadPart*>(a.B.head_part)[((size_t)kMaxBlocksDev + b0) * kMaxM + tid] = p;
-      }
-      named_sync(1, kWThreads);
-    }
+    // the split tile's sums of squares are the tile's part
+    if constexpr (KIND == kKResid) tile_ss(ss_sp, tile);
   };
 
   int prev_tile = -1;
@@ -728,10 +664,10 @@ template <int TP, int KIND, bool NORM>
 __global__ void __launch_bounds__(kTThreads, 1)
     k_tile(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap,
            const TArgs a) {
-  using S = TL<TP, KIND == kKHead>;
+  using S = TL<TP>;
   constexpr int NS = S::NS;
   extern __shared__ unsigned char smem_raw[];
-  Blk<TP, KIND == kKHead> k(smem_raw);
+  Blk<TP> k(smem_raw);
   unsigned char* smem = k.smem;
   const TGeom& g = a.g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
@@ -802,54 +738,6 @@ __global__ void __launch_bounds__(kTThreads, 1)
     int tc = -1;
     bool ok = true;
     worker_units<TP, KIND, NORM>(a, k, tmem, u_begin, n, 0, tc, ok, pos0, M);
-
-    // ---- exit head: per-block statistics, and the last block's fixed-order merge
-    if constexpr (KIND == kKHead) {
-      HeadPart* run = k.run;
-      HeadPart* comb = k.comb;
-      int* sflag = k.sflag;
-      HeadPart* sl = static_cast<HeadPart*>(a.B.head_part);
-      named_sync(1, kWThreads);
-      if (tid < M) {
-        HeadPart p;
-        part_empty(p);
-        for (int qq = 0; qq < 4; ++qq) part_merge(p, run[((tid & 1) * 4 + qq) * kLT + (tid >> 1)]);
-        sl[(size_t)blockIdx.x * kMaxM + tid] = p;
-      }
-      named_sync(1, kWThreads);
-      if (tid == 0) *sflag = atom_add_acq_rel_gpu(a.B.head_counter, 1u) == (unsigned)(g.P - 1);
-      named_sync(1, kWThreads);
-      if (*sflag) {
-        // per row: every worker thread takes blocks tid, tid + 256, ... (the
-        // running and split slots loaded together), then a shuffle tree per
-        // warp and a tree over the eight warps; the order does not depend on M
-        for (int m = 0; m < M; ++m) {
-          HeadPart p;
-          part_empty(p);
-          for (int b = tid; b < g.P; b += kWThreads) {
-            const bool sp = t_has_split_slot(g, b);
-            const HeadPart x = part_load_cg(&sl[(size_t)b * kMaxM + m]);
-            const HeadPart y = part_load_cg(&sl[((size_t)kMaxBlocksDev + (sp ? b : 0)) * kMaxM + m]);
-            part_merge(p, x);
-            if (sp) part_merge(p, y);
-          }
-          for (int off = 16; off > 0; off >>= 1) part_merge(p, part_shfl(p, off));
-          if (lane == 0) comb[warp] = p;
-          named_sync(1, kWThreads);
-          if (warp == 0) {
-            HeadPart f;
-            if (lane < kWorkers)
-              f = comb[lane];
-            else
-              part_empty(f);
-            for (int off = 4; off > 0; off >>= 1) part_merge(f, part_shfl(f, off));
-            if (lane == 0) write_row_stats(a.B.stats[m], f, a.topk);
-          }
-          named_sync(1, kWThreads);
-        }
-        if (tid == 0) *a.B.head_counter = 0u;
-      }
-    }
   }
 
   // TMEM is released once every MMA has completed and every read is done
@@ -890,11 +778,11 @@ struct ChainMaps {
 template <int TP, bool QKV4>
 __global__ void __launch_bounds__(kCThreads, 1)
     k_chain(const __grid_constant__ ChainMaps maps, const __grid_constant__ ChainArgs ca) {
-  using S = TL<TP, false>;
+  using S = TL<TP>;
   constexpr int NS = S::NS;
   constexpr int NPH = QKV4 ? 4 : 3;
   extern __shared__ unsigned char smem_raw[];
-  Blk<TP, false> k(smem_raw);
+  Blk<TP> k(smem_raw);
   unsigned char* smem = k.smem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
   const int P = ca.ph[0].g.P;
@@ -1071,7 +959,7 @@ cudaError_t tile_launch(const CUtensorMap& wm, const CUtensorMap& xm, const TArg
   if (a.g.T < 1 || a.g.T > (1 << 22) || a.g.P < 1 || a.g.P > kMaxBlocksDev)
     return cudaErrorInvalidValue;
   return launch_ex(k_tile<TP, KIND, NORM>, dim3(a.g.P), dim3(kTThreads),
-                   TL<TP, KIND == kKHead>::total, st, wm, xm, a);
+                   TL<TP>::total, st, wm, xm, a);
 }
 
 // Token rows of the instance for launches of up to mrows rows.
@@ -1090,22 +978,22 @@ cudaError_t tile_dispatch(const CUtensorMap& wm, const CUtensorMap* xm3, const T
 template <int TP, int KIND, bool NORM>
 cudaError_t prep_one() {
   return cudaFuncSetAttribute(k_tile<TP, KIND, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)TL<TP, KIND == kKHead>::total);
+                              (int)TL<TP>::total);
 }
 
 template <int TP, bool QKV4>
 cudaError_t chain_launch(const ChainMaps& m, const ChainArgs& a, cudaStream_t st) {
-  return launch_ex(k_chain<TP, QKV4>, dim3(a.ph[0].g.P), dim3(kCThreads), TL<TP, false>::total, st,
+  return launch_ex(k_chain<TP, QKV4>, dim3(a.ph[0].g.P), dim3(kCThreads), TL<TP>::total, st,
                    m, a);
 }
 
 template <int TP>
 cudaError_t prep_chain() {
   cudaError_t e = cudaFuncSetAttribute(k_chain<TP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)TL<TP, false>::total);
+                                       (int)TL<TP>::total);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_chain<TP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)TL<TP, false>::total);
+                              (int)TL<TP>::total);
 }
 
 template <int KIND, bool NORM>
@@ -1179,11 +1067,11 @@ int tile_blocks_per_sm() {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, threads, smem) != cudaSuccess) nb = 0;
     lo = nb < lo ? nb : lo;
   };
-  occ((const void*)k_chain<8, true>, kCThreads, TL<8, false>::total);
-  occ((const void*)k_chain<16, true>, kCThreads, TL<16, false>::total);
-  occ((const void*)k_chain<24, true>, kCThreads, TL<24, false>::total);
-  occ((const void*)k_tile<8, kKHead, true>, kTThreads, TL<8, true>::total);
-  occ((const void*)k_tile<24, kKQKV, true>, kTThreads, TL<24, false>::total);
+  occ((const void*)k_chain<8, true>, kCThreads, TL<8>::total);
+  occ((const void*)k_chain<16, true>, kCThreads, TL<16>::total);
+  occ((const void*)k_chain<24, true>, kCThreads, TL<24>::total);
+  occ((const void*)k_tile<8, kKHead, true>, kTThreads, TL<8>::total);
+  occ((const void*)k_tile<24, kKQKV, true>, kTThreads, TL<24>::total);
   return lo;
 }
 
@@ -1279,8 +1167,8 @@ cudaError_t launch_tile_chain(const Dims& D, const Bufs& B, const TileMaps& tm, 
 }
 
 cudaError_t launch_tile_head(const Dims& D, const Bufs& B, const TileMaps& tm,
-                             const CUtensorMap& lm, const void* final_norm, int topk,
-                             bool write_logits, RowSel sel, int mrows, cudaStream_t st) {
+                             const CUtensorMap& lm, const void* final_norm, RowSel sel, int mrows,
+                             cudaStream_t st) {
   TArgs a{};
   a.D = D;
   a.B = B;
@@ -1288,8 +1176,6 @@ cudaError_t launch_tile_head(const Dims& D, const Bufs& B, const TileMaps& tm,
   a.g = make_tgeom(D, D.V, D.d, kTMapLinear);
   a.gnorm = static_cast<const __nv_bfloat16*>(final_norm);
   a.ss_in = 0;
-  a.topk = topk;
-  a.write_logits = write_logits ? 1 : 0;
   return tile_dispatch<kKHead, true>(lm, tm.h, a, mrows, st);
 }
 
