@@ -1,8 +1,9 @@
 // attention.cu -- split-K decode attention over the contiguous KV cache for
-// 1 (drafting, autoregressive) or k + 1 (verification) query rows, with GQA,
-// in one kernel.
+// 1 (drafting, autoregressive) or k + 1 (verification) query rows, with GQA:
+// k_attn (fp32 models, CUDA cores, one kernel) and k_attn_rows with
+// k_attn_merge (bf16 models, tensor cores; below).
 //
-// Grid = (key splits of kAttnKeys, KV heads).  A block stages its keys and
+// k_attn: grid = (key splits of kAttnKeys, KV heads).  A block stages its keys and
 // values once (fp32 in shared memory) and serves every query head of the KV
 // group and every query row with them, so a GQA group of G heads and M rows
 // share one KV read.  Row m sits at position pos0 + m and attends causally to
@@ -24,6 +25,7 @@
 #include <math.h>
 
 #include "kernels.h"
+#include "mma.cuh"
 #include "pipe.cuh"
 
 namespace ssd {
@@ -286,22 +288,358 @@ size_t attn_smem(const Dims& D) {
   return sizeof(float) * ((kv > merge ? kv : merge) + (size_t)kAWarps * kAK) + sizeof(int) * kMaxM;
 }
 
-template <typename T>
-static cudaError_t attn_t(const Dims& D, const Bufs& B, int layer, RowSel sel, cudaStream_t st) {
+// ------------------------------------------------------------ bf16 models
+//
+// k_attn_rows: block = (split of D.attn_keys keys, KV head); its keys and
+// values are staged once as bf16 and serve the group's G x M query rows, 16
+// rows at a time per group of four warps.  Scores and outputs run on
+// mma.sync; the fp32 operand (queries, probabilities) enters in three bf16
+// parts, 24 bits, so nothing is rounded below fp32.  Of a 64-key step a warp
+// scores 16 keys; the four warps then share the row maxima and the
+// probabilities through shared memory and each multiplies all 64 keys with
+// its 32 of the 128 output columns.  A row's sums depend on its position
+// alone, not on the number of rows or on the other rows of its tile.
+// k_attn_merge: a warp per (row, head) adds the splits' partials in split
+// order.  A launch of its own: the last block of a KV head used to merge
+// alone, 136 rows x 17 splits in the widest verification.
+//
+// Bound by the chain of load, score, exchange, multiply within a block (the
+// KV rows are 1 to 45 MB).  us a call against the earlier kernel on CUDA
+// cores (one warp per (row, head) pair and 64 keys, merge by the last block):
+// 13 rows of the 8B widths after 1100 tokens, 4 layers, 1276 to 974; 17 rows
+// (70B, 1024 tokens, 2 layers) 1336 to 937; 2 rows (13B, 2176 tokens, 4
+// layers) 886 to 800; one row (7B, 640 tokens, 4 layers) 603 to 572.
+
+namespace {
+
+constexpr int kRHd = 128;
+constexpr int kRStep = kAttnKeys;                    // keys per step
+constexpr int kRGThreads = 128;                      // a row group: four warps
+constexpr int kRMaxGroups = 4;
+constexpr size_t kRKeyBytes = (size_t)kRStep * kRHd * 2;      // keys (or values) of a step
+constexpr size_t kRQBytes = (size_t)3 * 16 * kRHd * 2;        // 16 query rows, three parts
+constexpr size_t kRPBytes = (size_t)3 * 16 * kRStep * 2;      // their probabilities
+constexpr size_t kRGroupBytes = kRQBytes + kRPBytes + 2 * 4 * 16 * sizeof(float);
+
+}  // namespace
+
+__global__ void __launch_bounds__(kRGThreads * kRMaxGroups)
+    k_attn_rows(const Dims D, const Bufs B, int layer, RowSel sel) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  const int split = blockIdx.x, g = blockIdx.y;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int rg = tid / kRGThreads, ngrp = (int)blockDim.x / kRGThreads;
+  const int w = (tid >> 5) & 3;
+  const int G = D.Hq / D.Hkv;
+  const int len = D.attn_keys, s0 = split * len;
+  const __nv_bfloat16* kv =
+      static_cast<const __nv_bfloat16*>(B.kv) + (size_t)layer * 2 * D.Hkv * D.max_seq * kRHd;
+  const __nv_bfloat16* kb = kv + ((size_t)g * D.max_seq + s0) * kRHd;
+  const __nv_bfloat16* vb = kv + ((size_t)(D.Hkv + g) * D.max_seq + s0) * kRHd;
+  const uint32_t sbase = smem_u32(smem);
+
+  // keys [k0, k1) of the split; those from kend on are filled with zeros
+  auto stage = [&](int k0, int k1, int kend) {
+    for (int c = tid; c < (k1 - k0) * 16; c += (int)blockDim.x) {
+      const int key = k0 + (c >> 4), ch = c & 15;
+      const bool in = key < kend;
+      const size_t off = (size_t)(in ? key : 0) * kRHd + ch * 8;
+      const uint32_t dst = sbase + (uint32_t)(key / kRStep) * (uint32_t)(2 * kRKeyBytes) +
+                           sw256(key % kRStep, ch);
+      cp_async16(dst, kb + off, in);
+      cp_async16(dst + (uint32_t)kRKeyBytes, vb + off, in);
+    }
+  };
+
+  // keys written by earlier passes: loaded before the wait
+  int pos0, M;
+  resolve_rows(B.ctl, sel, pos0, M);
+  int nold = min(max(min(pos0, D.max_seq) - s0, 0), len);  // clamped: never past the cache
+  if (pos0 + M <= s0) nold = 0;
+  stage(0, nold, nold);
+  pdl_wait();
+  pdl_launch_dependents();
+  {
+    int p2, m2;
+    resolve_rows(B.ctl, sel, p2, m2);
+    if (p2 != pos0 || m2 != M) {  // the window moved: reload every key
+      if (tid == 0) atomicOr(&B.ctl->err, (int)kErrControl);
+      cp_async_wait_all();
+      __syncthreads();
+      pos0 = p2;
+      M = m2;
+      nold = 0;
+    }
+  }
+  if (s0 > pos0 + M - 1) {  // beyond every row's causal window
+    cp_async_wait_all();
+    return;
+  }
+  const int nkeys = min(len, pos0 + M - s0);
+  const int nsteps = (nkeys + kRStep - 1) / kRStep;
+  stage(nold, nsteps * kRStep, nkeys);
+
+  unsigned char* grp = smem + (size_t)(len / kRStep) * 2 * kRKeyBytes + (size_t)rg * kRGroupBytes;
+  const uint32_t qs = smem_u32(grp), ps = qs + (uint32_t)kRQBytes;
+  float* smx = reinterpret_cast<float*>(grp + kRQBytes + kRPBytes);  // [warp][row] maxima
+  float* sls = smx + 4 * 16;                                         // [warp][row] sums
+  const int gt = tid % kRGThreads;
+  const float scale = 1.0f / sqrtf((float)kRHd);
+  const int row_lo = max(0, s0 - pos0) * G, nrows = G * M;  // rows that see a key here
+  const int rr = lane >> 2;  // the thread's rows of a tile: rr and rr + 8
+  bool staged = false;
+
+  for (int r0 = row_lo + 16 * rg; r0 < nrows; r0 += 16 * ngrp) {
+    // queries of the tile: three bf16 parts (rows past the last are zero)
+    for (int c = gt; c < 16 * 16; c += kRGThreads) {
+      const int row = c >> 4, ch = c & 15, r = r0 + row;
+      float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), x1 = x0;
+      if (r < nrows) {
+        const int m = r / G, h = g * G + r - m * G;
+        const float4* p =
+            reinterpret_cast<const float4*>(B.xq + (size_t)m * D.qd + (size_t)h * kRHd + ch * 8);
+        x0 = p[0];
+        x1 = p[1];
+      }
+      uint4 q3[3];
+      split3(x0.x, x0.y, q3[0].x, q3[1].x, q3[2].x);
+      split3(x0.z, x0.w, q3[0].y, q3[1].y, q3[2].y);
+      split3(x1.x, x1.y, q3[0].z, q3[1].z, q3[2].z);
+      split3(x1.z, x1.w, q3[0].w, q3[1].w, q3[2].w);
+#pragma unroll
+      for (int s = 0; s < 3; ++s)
+        *reinterpret_cast<uint4*>(grp + (size_t)s * 16 * 256 + sw256(row, ch)) = q3[s];
+    }
+    if (!staged) {
+      cp_async_wait_all();
+      __syncthreads();
+      staged = true;
+    } else {
+      named_sync(1 + rg, kRGThreads);
+    }
+    int pos[2];
+    float mx[2], ls[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int r = r0 + rr + 8 * e;
+      pos[e] = r < nrows ? pos0 + r / G : s0;  // an unused row sees the split's first key
+      mx[e] = -INFINITY;
+      ls[e] = 0.f;
+    }
+    float o[4][4];
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o[n][e] = 0.f;
+
+    for (int st = 0; st < nsteps; ++st) {
+      const uint32_t kd = sbase + (uint32_t)st * (uint32_t)(2 * kRKeyBytes);
+      const uint32_t vd = kd + (uint32_t)kRKeyBytes;
+      // scores of the warp's 16 keys: two n-tiles, even and odd 16-column
+      // steps summed apart; the lower parts first, since the running sum is
+      // cut at its own last place
+      float s[2][2][4];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) s[i][n][e] = 0.f;
+#pragma unroll
+      for (int pass = 0; pass < 2; ++pass)
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) {
+          uint32_t kf[4];
+          ldsm4(kd + sw256(16 * w + (lane & 7) + ((lane >> 4) << 3), 2 * kk + ((lane >> 3) & 1)), kf);
+#pragma unroll
+          for (int p = pass ? 0 : 2; p >= (pass ? 0 : 1); --p) {
+            uint32_t qa[4];
+            ldsm4(qs + (uint32_t)(p * 16 * 256) + sw256(lane & 15, 2 * kk + (lane >> 4)), qa);
+            mma16816(s[kk & 1][0], qa, kf[0], kf[1]);
+            mma16816(s[kk & 1][1], qa, kf[2], kf[3]);
+          }
+        }
+      const int kbase = s0 + st * kRStep + 16 * w + 2 * (lane & 3);
+      float z[2][4], nm[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int key = kbase + 8 * n + (e & 1);
+          z[n][e] = key <= pos[e >> 1] ? (s[0][n][e] + s[1][n][e]) * scale : -INFINITY;
+          nm[e >> 1] = fmaxf(nm[e >> 1], z[n][e]);
+        }
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        nm[e] = fmaxf(nm[e], __shfl_xor_sync(0xffffffffu, nm[e], 1));
+        nm[e] = fmaxf(nm[e], __shfl_xor_sync(0xffffffffu, nm[e], 2));
+        if ((lane & 3) == 0) smx[w * 16 + rr + 8 * e] = nm[e];
+      }
+      named_sync(1 + rg, kRGThreads);
+      float f[2], rs[2] = {0.f, 0.f};
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        float m = mx[e];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) m = fmaxf(m, smx[i * 16 + rr + 8 * e]);
+        // every row sees the split's first key: finite from the first step on
+        f[e] = expf(mx[e] - m);
+        mx[e] = m;
+      }
+#pragma unroll
+      for (int n = 0; n < 2; ++n) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          z[n][e] = expf(z[n][e] - mx[e >> 1]);
+          rs[e >> 1] += z[n][e];
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          uint32_t q[3];
+          split3(z[n][2 * e], z[n][2 * e + 1], q[0], q[1], q[2]);
+#pragma unroll
+          for (int p = 0; p < 3; ++p)
+            *reinterpret_cast<uint32_t*>(grp + kRQBytes + (size_t)p * 16 * 128 +
+                                         sw128(rr + 8 * e, 2 * w + n) + 4 * (lane & 3)) = q[p];
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        rs[e] += __shfl_xor_sync(0xffffffffu, rs[e], 1);
+        rs[e] += __shfl_xor_sync(0xffffffffu, rs[e], 2);
+        if ((lane & 3) == 0) sls[w * 16 + rr + 8 * e] = rs[e];
+      }
+      named_sync(1 + rg, kRGThreads);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float* l = sls + rr + 8 * e;
+        ls[e] = fmaf(ls[e], f[e], (l[0] + l[16]) + (l[32] + l[48]));
+      }
+      // outputs: columns 32 w .. 32 w + 31, this step's share in sums of its
+      // own, then one rounded multiply-add into the running output
+      float t[4][4];
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) t[n][e] = 0.f;
+#pragma unroll
+      for (int p = 2; p >= 0; --p)
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+          uint32_t pa[4];
+          ldsm4(ps + (uint32_t)(p * 16 * 128) + sw128(lane & 15, 2 * ks + (lane >> 4)), pa);
+#pragma unroll
+          for (int n2 = 0; n2 < 2; ++n2) {
+            uint32_t vf[4];
+            ldsm4t(vd + sw256(16 * ks + (lane & 15), 4 * w + 2 * n2 + (lane >> 4)), vf);
+            mma16816(t[2 * n2], pa, vf[0], vf[1]);
+            mma16816(t[2 * n2 + 1], pa, vf[2], vf[3]);
+          }
+        }
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[n][e] = fmaf(o[n][e], f[e >> 1], t[n][e]);
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int r = r0 + rr + 8 * e;
+      if (r >= nrows) continue;
+      const int m = r / G, h = g * G + r - m * G;
+      const size_t pidx = ((size_t)m * D.Hq + h) * D.nsplit + split;
+      float* part = B.attn_part + pidx * kRHd + 32 * w + 2 * (lane & 3);
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+        *reinterpret_cast<float2*>(part + 8 * n) = make_float2(o[n][2 * e], o[n][2 * e + 1]);
+      if (w == 0 && (lane & 3) == 0)
+        *reinterpret_cast<float2*>(B.attn_ml + 2 * pidx) = make_float2(mx[e], ls[e]);
+    }
+  }
+  if (!staged) {  // a group without rows: the others' barrier
+    cp_async_wait_all();
+    __syncthreads();
+  }
+}
+
+// Merge of the splits: a warp per (row, head), four columns per lane.
+__global__ void __launch_bounds__(256) k_attn_merge(const Dims D, const Bufs B, RowSel sel) {
+  pdl_wait();
+  pdl_launch_dependents();
+  int pos0, M;
+  resolve_rows(B.ctl, sel, pos0, M);
+  const int lane = threadIdx.x & 31;
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int m = i / D.Hq;
+  if (m >= M) return;
+  const int nsp = (pos0 + m) / D.attn_keys + 1;
+  const float2* ml = reinterpret_cast<const float2*>(B.attn_ml) + (size_t)i * D.nsplit;
+  const float4* part =
+      reinterpret_cast<const float4*>(B.attn_part + (size_t)i * D.nsplit * kRHd) + lane;
+  constexpr int kBatch = 8;
+  float gmax = -INFINITY;
+  for (int s = lane; s < nsp; s += 32) gmax = fmaxf(gmax, __ldcg(&ml[s]).x);
+  gmax = warp_max(gmax);
+  float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
+  float L = 0.f;
+  for (int s0 = 0; s0 < nsp; s0 += kBatch) {
+    float4 p[kBatch];
+    float2 a[kBatch];
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) {
+      const int s = s0 + j < nsp ? s0 + j : s0;
+      p[j] = __ldcg(part + (size_t)s * (kRHd / 4));
+      a[j] = __ldcg(&ml[s]);
+    }
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) {
+      const float wj = s0 + j < nsp ? expf(a[j].x - gmax) : 0.f;
+      L = fmaf(wj, a[j].y, L);
+      O.x = fmaf(wj, p[j].x, O.x);
+      O.y = fmaf(wj, p[j].y, O.y);
+      O.z = fmaf(wj, p[j].z, O.z);
+      O.w = fmaf(wj, p[j].w, O.w);
+    }
+  }
+  *reinterpret_cast<float4*>(B.attn_out + (size_t)i * kRHd + 4 * lane) =
+      make_float4(O.x / L, O.y / L, O.z / L, O.w / L);
+}
+
+// Keys per split of the bf16 kernel: 64, or 128 where 64 would make more
+// blocks than the SMs hold at once (three each) with a full cache.
+int attn_split_keys(int n_kv_heads, int max_seq, int sms) {
+  const int n = (max_seq + kRStep - 1) / kRStep;
+  return n_kv_heads * n > 3 * sms ? 2 * kRStep : kRStep;
+}
+
+static cudaError_t attn_bf16(const Dims& D, const Bufs& B, int layer, RowSel sel, int mrows,
+                             cudaStream_t st) {
+  const int rows = mrows * (D.Hq / D.Hkv);
+  const int groups = rows <= 16 ? 1 : (rows <= 32 ? 2 : kRMaxGroups);
+  const size_t smem = (size_t)(D.attn_keys / kRStep) * 2 * kRKeyBytes + groups * kRGroupBytes;
+  cudaError_t e =
+      cudaFuncSetAttribute(k_attn_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((D.max_seq + D.attn_keys - 1) / D.attn_keys, D.Hkv);
+  e = launch_ex(k_attn_rows, grid, dim3(groups * kRGThreads), smem, st, D, B, layer, sel);
+  if (e != cudaSuccess) return e;
+  return launch_ex(k_attn_merge, dim3((mrows * D.Hq + 7) / 8), dim3(256), 0, st, D, B, sel);
+}
+
+static cudaError_t attn_f32(const Dims& D, const Bufs& B, int layer, RowSel sel, cudaStream_t st) {
   dim3 grid(D.nsplit, D.Hkv);
   const size_t smem = attn_smem(D);
   if (smem > 48 * 1024) {
     cudaError_t e =
-        cudaFuncSetAttribute(k_attn<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_attn<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  return launch_ex(k_attn<T>, grid, dim3(kAThreads), smem, st, D, B, layer, sel);
+  return launch_ex(k_attn<float>, grid, dim3(kAThreads), smem, st, D, B, layer, sel);
 }
 
 cudaError_t launch_attention(const Dims& D, const Bufs& B, int dtype, int layer, RowSel sel,
-                             bool /*big*/, cudaStream_t st) {
-  if (dtype == SSD_DTYPE_BF16) return attn_t<__nv_bfloat16>(D, B, layer, sel, st);
-  return attn_t<float>(D, B, layer, sel, st);
+                             int mrows, cudaStream_t st) {
+  if (dtype == SSD_DTYPE_BF16) return attn_bf16(D, B, layer, sel, mrows, st);
+  return attn_f32(D, B, layer, sel, st);
 }
 
 }  // namespace ssd

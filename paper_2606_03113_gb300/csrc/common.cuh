@@ -150,6 +150,7 @@ struct LayerW {
 // Shapes and buffers every kernel may need.
 struct Dims {
   int32_t L, d, Hq, Hkv, hd, F, V, max_seq, qd, kvd, nsplit, num_sms, ss_tiles, max_tiles;
+  int32_t attn_keys;  // keys per attention split (bf16 kernel)
   int32_t ss_nt;  // 256-row tiles of a residual row (tensor-core kernels' sum-of-squares parts)
   float eps;
 };

@@ -549,6 +549,7 @@ ssd_status ssd_init_model(const ssd_model_cfg* cfg, const ssd_weights* w, void* 
     }
   }
   x->D.num_sms = std::min(sms * std::min(per_sm, 1), kMaxBlocks);
+  x->D.attn_keys = attn_split_keys(cfg->n_kv_heads, cfg->max_seq, x->D.num_sms);
   x->embed = w->embed;
   x->lm_head = w->lm_head;
   x->final_norm = w->final_norm;

@@ -773,7 +773,7 @@ cudaError_t prepare_gemv_kernels() {
 
 // Attention launchers live in attention.cu.
 cudaError_t launch_attention(const Dims& D, const Bufs& B, int dtype, int layer, RowSel sel,
-                             bool big, cudaStream_t st);
+                             int mrows, cudaStream_t st);
 
 template <typename T, int MM>
 static cudaError_t part_t(const Dims& D, const Bufs& B, const LayerW& w, int layer, int part,
@@ -793,7 +793,7 @@ static cudaError_t part_t(const Dims& D, const Bufs& B, const LayerW& w, int lay
       return stream_launch<T, MM, true>(a, EpiQKV<T>{layer}, st);
     case 1:
       return launch_attention(D, B, std::is_same<T, float>::value ? SSD_DTYPE_F32 : SSD_DTYPE_BF16,
-                              layer, sel, MM > 1, st);
+                              layer, sel, MM, st);
     case 2:
       a.g = make_geom(D, D.d, D.qd, elt, kMapLinear);
       a.W = w.wo;
@@ -825,7 +825,7 @@ cudaError_t launch_layer_part(const Dims& D, const Bufs& B, int dtype, const Lay
                               cudaStream_t st) {
   const bool big = mrows > 1;
   if (dtype == SSD_DTYPE_BF16) {
-    if (part == 1) return launch_attention(D, B, dtype, layer, sel, big, st);
+    if (part == 1) return launch_attention(D, B, dtype, layer, sel, mrows, st);
     if (!tm) return cudaErrorInvalidValue;
     return launch_tile_part(D, B, *tm, w, layer, part, sel, mrows, st);
   }

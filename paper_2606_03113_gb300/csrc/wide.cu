@@ -35,6 +35,7 @@
 #include <math.h>
 
 #include "kernels.h"
+#include "mma.cuh"
 #include "pipe.cuh"
 #include "tc.cuh"
 
@@ -425,49 +426,6 @@ constexpr size_t kAQBytes = (size_t)3 * kAQ * kAHd * 2;  // queries, three bf16 
 constexpr size_t kAKBytes = (size_t)kAKB * kAHd * 2;
 constexpr size_t kAWSmem = kAQBytes + 4 * kAKBytes;      // + keys and values, double buffered
 
-// Byte offset of 16-byte chunk c of a 256-byte row (swizzled by row % 8).
-__device__ __forceinline__ uint32_t aw_off(int row, int c) {
-  return (uint32_t)(row * 256 + ((c ^ (row & 7)) << 4));
-}
-__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool valid) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
-               "r"(valid ? 16 : 0)
-               : "memory");
-}
-__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr)
-               : "memory");
-}
-__device__ __forceinline__ void ldsm4t(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr)
-               : "memory");
-}
-__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
-                                         uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-      "{%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// (x, y) as three packed bf16 pairs whose sum keeps 24 bits of each.
-__device__ __forceinline__ void split3(float x, float y, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
-  auto pack = [](float u, float w) -> uint32_t {
-    const __nv_bfloat162 b = __floats2bfloat162_rn(u, w);
-    return *reinterpret_cast<const uint32_t*>(&b);
-  };
-  auto lo = [](uint32_t p) { return __uint_as_float(p << 16); };
-  auto hi = [](uint32_t p) { return __uint_as_float(p & 0xffff0000u); };
-  p0 = pack(x, y);
-  const float x1 = x - lo(p0), y1 = y - hi(p0);
-  p1 = pack(x1, y1);
-  p2 = pack(x1 - lo(p1), y1 - hi(p1));
-}
-
 }  // namespace
 
 __global__ void __launch_bounds__(kAWThreads, 2)
@@ -496,8 +454,8 @@ __global__ void __launch_bounds__(kAWThreads, 2)
       const int key = b * kAKB + row;
       const bool in = key <= last;  // keys past the last one read zeros
       const size_t off = (size_t)(in ? key : 0) * kAHd + ch * 8;
-      cp16(kd + aw_off(row, ch), kb + off, in);
-      cp16(vd + aw_off(row, ch), vb + off, in);
+      cp_async16(kd + sw256(row, ch), kb + off, in);
+      cp_async16(vd + sw256(row, ch), vb + off, in);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
@@ -519,7 +477,7 @@ __global__ void __launch_bounds__(kAWThreads, 2)
     split3(x1.z, x1.w, w[0].w, w[1].w, w[2].w);
 #pragma unroll
     for (int s = 0; s < 3; ++s)
-      *reinterpret_cast<uint4*>(smem + (size_t)s * kAQ * 256 + aw_off(row, ch)) = w[s];
+      *reinterpret_cast<uint4*>(smem + (size_t)s * kAQ * 256 + sw256(row, ch)) = w[s];
   }
 
   float o[16][4];
@@ -557,12 +515,12 @@ __global__ void __launch_bounds__(kAWThreads, 2)
         const int np = pass ? 1 : 2;
 #pragma unroll
         for (int p = 0; p < np; ++p)
-          ldsm4(sq + (uint32_t)((pass ? 0 : 2 - p) * kAQ * 256) + aw_off(lrow, 2 * kk + lch), qa[p]);
+          ldsm4(sq + (uint32_t)((pass ? 0 : 2 - p) * kAQ * 256) + sw256(lrow, 2 * kk + lch), qa[p]);
 #pragma unroll
         for (int n2 = 0; n2 < 4; ++n2) {
           // keys 16 n2 .. + 15 x 16 columns: two n-tiles
           uint32_t kf[4];
-          ldsm4(kd + aw_off(16 * n2 + (lane & 7) + ((lane >> 4) << 3), 2 * kk + ((lane >> 3) & 1)),
+          ldsm4(kd + sw256(16 * n2 + (lane & 7) + ((lane >> 4) << 3), 2 * kk + ((lane >> 3) & 1)),
                 kf);
 #pragma unroll
           for (int p = 0; p < np; ++p) {
@@ -616,7 +574,7 @@ __global__ void __launch_bounds__(kAWThreads, 2)
       uint32_t vf[4][4];
 #pragma unroll
       for (int ks = 0; ks < 4; ++ks)
-        ldsm4t(vd + aw_off(16 * ks + (lane & 15), 2 * n2 + (lane >> 4)), vf[ks]);
+        ldsm4t(vd + sw256(16 * ks + (lane & 15), 2 * n2 + (lane >> 4)), vf[ks]);
 #pragma unroll
       for (int p = 2; p >= 0; --p)
 #pragma unroll
