@@ -16,6 +16,7 @@ constexpr int kMaxM = 17;          // rows of one verify pass: pending token + u
 constexpr int kMaxDraft = 16;
 constexpr int kMaxCand = SSD_TRACE_MAXC;
 constexpr int kTraceCap = 64;      // C_trace window capacity
+constexpr int kSampChunks = 256;  // chunk sums of a row's sampling weights, at most
 constexpr int kTopK = 8;           // max k of the token confidence
 constexpr int kWarps = 8;          // warps per block of the matrix-vector kernels
 constexpr int kAttnKeys = 64;      // keys per attention split (two per lane)
@@ -173,6 +174,8 @@ struct Bufs {
   uint32_t* attn_counter;  // [Hkv][kMaxM] split tickets of the attention merge
   uint32_t* chain_bar;     // [2] grid-wide phase arrivals / blocks done of the chain kernel
   float* draft_logits;     // [kMaxDraft][V] exit logits of each draft (sampled decoding)
+  float* row_sums;         // [kMaxM][kSampChunks] sampling weights of each row's chunks
+  float* res_sums;         // [kSampChunks] the same of a rejected draft's residual
   float* attn_out;   // [kMaxM][qd]
   float* act;        // [kMaxM][F]
   float* logits;     // [kMaxM][V] of the last exit head

@@ -35,116 +35,129 @@ __device__ float trace_conf(const Ctl* c, int T) {
 // Speculative sampling draws drafts from the exit distribution and emitted
 // tokens from the full model's, both at temperature T:
 // P(v) = exp((z_v - max z) / T) / sum_w exp((z_w - max z) / T).
-// Every reduction below runs in a fixed order (contiguous per-thread chunks
-// of the vocabulary, chunk sums added in chunk order by one thread), so a
-// draw depends only on the logits and the uniform, never on scheduling.
+// k_row_weights reads the rows' logits on all SMs and leaves the weights' sums
+// over at most kSampChunks runs of the vocabulary; a draw then scans those
+// sums and walks the one run that holds it.  One block used to read whole
+// rows, each thread a run of its own: @SAMP@
+// Every reduction below runs in a fixed order that depends on the vocabulary
+// alone, so a draw depends only on the logits and the uniform, never on
+// scheduling.
 // The uniforms come from synth_sample_uniform keyed by the round's pending
 // position: purpose 0 the draw of draft i, 1 the acceptance test of draft i,
 // 2 the round's last draw.
 
-constexpr int kSampleThreads = 256;  // block size of k_decide and k_accept
+constexpr int kSampleThreads = 256;  // block size of the sampling kernels
+
+// Tokens per chunk: a multiple of 8 per thread, at most kSampChunks chunks.
+__host__ __device__ inline int samp_chunk(int V) {
+  const int unit = kSampleThreads * 8;
+  return unit * ((V + unit * kSampChunks - 1) / (unit * kSampChunks));
+}
 
 struct SampleSmem {
-  float part[kSampleThreads];  // chunk sums, then their exclusive prefix
+  float part[kSampleThreads];  // inclusive prefix sums, one per thread
   float red[kSampleThreads / 32];
-  float total, zmax;
-  int tok;
+  float rows[kMaxM];           // row totals
+  float pd[kMaxDraft], qd[kMaxDraft];
+  int first, tok;
   float margin;
 };
 
-__device__ __forceinline__ void chunk_of(int V, int& v0, int& v1) {
-  const int C = (V + (int)blockDim.x - 1) / (int)blockDim.x;
-  v0 = min(V, (int)threadIdx.x * C);
-  v1 = min(V, v0 + C);
-}
-
-// Maximum of z[0..V) broadcast to the block (exact in any order).
-__device__ float block_zmax(const float* __restrict__ z, int V, SampleSmem& sm) {
-  int v0, v1;
-  chunk_of(V, v0, v1);
-  float m = -INFINITY;
-  for (int v = v0; v < v1; ++v) m = fmaxf(m, z[v]);
-  m = warp_max(m);
-  if ((threadIdx.x & 31) == 0) sm.red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float r = sm.red[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = fmaxf(r, sm.red[w]);
-    sm.zmax = r;
+// Inclusive prefix sums of x over the block's threads into sm.part (fixed
+// tree); every thread calls it, and the sums are visible on return.
+__device__ __forceinline__ void block_prefix(float x, SampleSmem& sm) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const float y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
   }
+  if (lane == 31) sm.red[warp] = x;
   __syncthreads();
-  const float r = sm.zmax;
+  float base = 0.f;
+  for (int w = 0; w < warp; ++w) base += sm.red[w];
+  sm.part[threadIdx.x] = base + x;
   __syncthreads();
-  return r;
 }
 
-// Sum of w(v) over [0, V) in the fixed chunk order; leaves the exclusive
-// prefix of the chunk sums in sm.part and returns the total to every thread.
+// First token (in token order) and sum of the calling thread's run of chunk c.
+__device__ __forceinline__ void thread_run(int V, int c, int& v0, int& v1) {
+  const int C = samp_chunk(V), per = C / kSampleThreads;
+  v0 = min(V, c * C + (int)threadIdx.x * per);
+  v1 = min(V, v0 + per);
+}
+
 template <typename W>
-__device__ float block_chunk_sums(int V, W w, SampleSmem& sm) {
-  int v0, v1;
-  chunk_of(V, v0, v1);
+__device__ __forceinline__ float run_sum(int v0, int v1, const W& w) {
   float acc = 0.f;
+#pragma unroll 8
   for (int v = v0; v < v1; ++v) acc += w(v);
-  sm.part[threadIdx.x] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float c = 0.f;
-    for (int i = 0; i < (int)blockDim.x; ++i) {
-      const float x = sm.part[i];
-      sm.part[i] = c;
-      c += x;
-    }
-    sm.total = c;
-  }
-  __syncthreads();
-  return sm.total;
+  return acc;
 }
 
-// Inverse-CDF draw from non-negative weights w(v): with W the total and
-// C_v = w(0) + ... + w(v) in token order, the token is the first v with
-// C_v > u W; *margin = min(u W - C_{v-1}, C_v - u W) / W.  Returns -1 when W
-// is not positive; when rounding leaves u W at or beyond the total, the last
-// token of positive weight (margin 0).  Every thread of the block calls it.
+// Total of a row's chunk sums, one warp (fixed order).
+__device__ __forceinline__ float warp_row_total(const float* sums, int nch) {
+  float t = 0.f;
+#pragma unroll
+  for (int i = 0; i < kSampChunks / 32; ++i) {
+    const int c = i * 32 + (int)(threadIdx.x & 31);
+    if (c < nch) t += __ldcg(sums + c);
+  }
+  return warp_sum(t);
+}
+
+// Inverse-CDF draw from non-negative weights w(v) whose chunk sums are given:
+// with W their total and C_v = w(0) + ... + w(v) in token order, the token is
+// the first v with C_v > u W; *margin = min(u W - C_{v-1}, C_v - u W) / W.
+// Returns -1 when W is not positive; when rounding leaves u W at or beyond
+// the total (of the vocabulary or of the chunk), the last token of positive
+// weight before it (margin 0).  Every thread of the block calls it.
 template <typename W>
-__device__ int block_draw(int V, W w, float u, float* margin, SampleSmem& sm) {
-  const float S = block_chunk_sums(V, w, sm);
-  int v0, v1;
-  chunk_of(V, v0, v1);
-  if (threadIdx.x == 0) {
-    sm.tok = -1;
+__device__ int block_draw(int V, const W& w, const float* sums, float u, float* margin,
+                          SampleSmem& sm) {
+  const int tid = threadIdx.x;
+  const int nch = (V + samp_chunk(V) - 1) / samp_chunk(V);
+  static_assert(kSampChunks <= kSampleThreads, "a chunk per thread");
+  if (tid == 0) {
+    sm.first = kSampChunks;
+    sm.tok = 0x7fffffff;
     sm.margin = 0.f;
   }
+  block_prefix(tid < nch ? __ldcg(sums + tid) : 0.f, sm);
+  const float S = sm.part[kSampleThreads - 1];
+  const float T = u * S;
+  if (tid < nch && sm.part[tid] > T) atomicMin(&sm.first, tid);
   __syncthreads();
-  if (S > 0.f) {
-    const float T = u * S;
-    const float lo = sm.part[threadIdx.x];
-    const float hi = threadIdx.x + 1 < blockDim.x ? sm.part[threadIdx.x + 1] : S;
-    // chunk intervals [lo, hi) are disjoint: at most one thread holds T
-    if (v1 > v0 && T >= lo && T < hi) {
-      float c = lo, mg = 0.f;
-      int found = -1, last = -1;
-      for (int v = v0; v < v1; ++v) {
-        const float wv = w(v);
-        const float nx = c + wv;
-        if (wv > 0.f) last = v;
-        if (nx > T) {
-          found = v;
-          mg = fminf(T - c, nx - T) / S;
-          break;
-        }
-        c = nx;
+  int c = sm.first;
+  if (!(S > 0.f)) return -1;
+  const bool beyond = c >= nch;
+  if (beyond) c = nch - 1;
+  const float base = c > 0 ? sm.part[c - 1] : 0.f;
+  __syncthreads();
+  int v0, v1;
+  thread_run(V, c, v0, v1);
+  if (!beyond) {
+    block_prefix(run_sum(v0, v1, w), sm);
+    float cum = base + (tid > 0 ? sm.part[tid - 1] : 0.f), mg = 0.f;
+    int found = 0x7fffffff;
+    for (int v = v0; v < v1; ++v) {
+      const float nx = cum + w(v);
+      if (nx > T) {
+        found = v;
+        mg = fmaxf(fminf(T - cum, nx - T), 0.f) / S;
+        break;
       }
-      sm.tok = found >= 0 ? found : last;
-      sm.margin = found >= 0 ? mg : 0.f;
+      cum = nx;
     }
+    if (found != 0x7fffffff) atomicMin(&sm.tok, found);
+    __syncthreads();
+    if (sm.tok == found && found != 0x7fffffff) sm.margin = mg;
+    __syncthreads();
   }
-  __syncthreads();
-  if (threadIdx.x == 0 && S > 0.f && sm.tok < 0) {
-    int v = V - 1;
+  if (tid == 0 && sm.tok == 0x7fffffff) {
+    int v = min(V, (c + 1) * samp_chunk(V)) - 1;
     while (v > 0 && !(w(v) > 0.f)) --v;
     sm.tok = v;
-    sm.margin = 0.f;
   }
   __syncthreads();
   const int tok = sm.tok;
@@ -165,6 +178,101 @@ struct Residual {
   float sp, sq;  // normalisers of p and q
   __device__ float operator()(int v) const { return fmaxf(p(v) / sp - q(v) / sq, 0.f); }
 };
+
+// Weight sums of the logits rows `sel` (the statistics kernel has left their
+// maxima), one chunk per block; keep >= 0: also stores the row as draft 0
+// (kKeepWalk) or draft k of the round (kKeepDraft) for the acceptance test.
+enum KeepMode : int { kKeepNone = 0, kKeepWalk = 1, kKeepDraft = 2 };
+__global__ void __launch_bounds__(kSampleThreads)
+    k_row_weights(const Dims D, const Bufs B, RowSel sel, int keep) {
+  pdl_wait();
+  pdl_launch_dependents();
+  __shared__ SampleSmem sm;
+  const Ctl* c = B.ctl;
+  int pos0, M;
+  resolve_rows(c, sel, pos0, M);
+  const int m = blockIdx.y;
+  if (m >= M) return;
+  const float* z = B.logits + (size_t)m * D.V;
+  const Tempered w{z, B.stats[m].zmax, c->pol.temp};
+  int v0, v1;
+  thread_run(D.V, blockIdx.x, v0, v1);
+  block_prefix(run_sum(v0, v1, w), sm);
+  if (threadIdx.x == 0) B.row_sums[(size_t)m * kSampChunks + blockIdx.x] = sm.part[kSampleThreads - 1];
+  if (keep == kKeepNone) return;
+  const int slot = keep == kKeepDraft ? c->k : 0;
+  if (slot < 0 || slot >= kMaxDraft) return;
+  float* dst = B.draft_logits + (size_t)slot * D.V;
+  const int C = samp_chunk(D.V), e = min(D.V, (int)(blockIdx.x + 1) * C);
+  for (int v = blockIdx.x * C + threadIdx.x; v < e; v += kSampleThreads) dst[v] = z[v];
+}
+
+// Row of the round's last draw (the first draft whose test fails, or k) from
+// the verification rows' weight sums; every thread calls it.  Leaves p's
+// totals in sm.rows and the acceptance margins in sm.pd.
+__device__ int accept_tests(const Dims& D, const Bufs& B, SampleSmem& sm) {
+  const Ctl* c = B.ctl;
+  const int tid = threadIdx.x, nch = (D.V + samp_chunk(D.V) - 1) / samp_chunk(D.V);
+  const float temp = c->pol.temp;
+  const int k = min(c->k, kMaxDraft);
+  for (int m = tid >> 5; m <= k; m += kSampleThreads / 32) {
+    const float t = warp_row_total(B.row_sums + (size_t)m * kSampChunks, nch);
+    if ((tid & 31) == 0) sm.rows[m] = t;
+  }
+  if (tid < k) {
+    const int d = c->tok[tid + 1];
+    float pw = 0.f, qw = 0.f;
+    if (d >= 0 && d < D.V) {
+      pw = Tempered{B.logits + (size_t)tid * D.V, B.stats[tid].zmax, temp}(d);
+      qw = Tempered{B.draft_logits + (size_t)tid * D.V, c->dq_zmax[tid], temp}(d);
+    }
+    sm.pd[tid] = pw;
+    sm.qd[tid] = qw;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    int a = 0;
+    for (; a < k; ++a) {
+      const int d = c->tok[a + 1];
+      const float sp = sm.rows[a], sq = c->dq_sum[a];
+      const bool ok_d = d >= 0 && d < D.V && sp > 0.f && sq > 0.f;
+      const float pd = ok_d ? sm.pd[a] / sp : 0.f;
+      const float qd = ok_d ? sm.qd[a] / sq : 0.f;
+      const float rq = synth_sample_uniform(c->pol.seed, (uint32_t)c->pos, 1u, (uint32_t)a) * qd;
+      const float den = fmaxf(pd, rq);
+      sm.pd[a] = den > 0.f ? (pd - rq) / den : 0.f;
+      if (!(ok_d && rq < pd)) break;
+    }
+    sm.first = a;
+  }
+  __syncthreads();
+  const int a = sm.first;
+  __syncthreads();
+  return a;
+}
+
+__device__ __forceinline__ Residual residual_of(const Dims& D, const Bufs& B, int a, float sp) {
+  const Ctl* c = B.ctl;
+  const float temp = c->pol.temp;
+  return Residual{Tempered{B.logits + (size_t)a * D.V, B.stats[a].zmax, temp},
+                  Tempered{B.draft_logits + (size_t)a * D.V, c->dq_zmax[a], temp}, sp,
+                  c->dq_sum[a]};
+}
+
+// Chunk sums of the residual max(0, p - q) of the round's first rejected
+// draft, if there is one.
+__global__ void __launch_bounds__(kSampleThreads) k_residual_weights(const Dims D, const Bufs B) {
+  pdl_wait();
+  pdl_launch_dependents();
+  __shared__ SampleSmem sm;
+  const int a = accept_tests(D, B, sm);
+  if (a >= min(B.ctl->k, kMaxDraft)) return;
+  const Residual res = residual_of(D, B, a, sm.rows[a]);
+  int v0, v1;
+  thread_run(D.V, blockIdx.x, v0, v1);
+  block_prefix(run_sum(v0, v1, res), sm);
+  if (threadIdx.x == 0) B.res_sums[blockIdx.x] = sm.part[kSampleThreads - 1];
+}
 
 // h[m] = embed[token_m] (fp32) and the row's sum of squares for the first
 // RMSNorm.  One block per row.  Optionally sets the drafting switch handle to
@@ -444,17 +552,21 @@ __global__ void k_decide(Dims D, Bufs B, int mode, int cand_idx, int is_last, in
     __syncthreads();
     const int slot = s_slot;
     if (slot >= 0) {
-      const float* z = B.logits;  // row 0: this exit's logits
-      float* keep = B.draft_logits + (size_t)slot * D.V;
-      for (int v = tid; v < D.V; v += blockDim.x) keep[v] = z[v];
-      const float zmax = block_zmax(z, D.V, sm);
-      const Tempered q{z, zmax, P.temp};
+      // row 0: this exit's logits, their weight sums and the kept copy are
+      // k_row_weights' work
+      const float zmax = st.zmax;
+      const Tempered q{B.logits, zmax, P.temp};
+      if (tid < 32) {
+        const float t = warp_row_total(B.row_sums, (D.V + samp_chunk(D.V) - 1) / samp_chunk(D.V));
+        if (tid == 0) sm.rows[0] = t;
+      }
       float mg = 0.f;
-      const int d = block_draw(D.V, q, synth_sample_uniform(P.seed, (uint32_t)c->pos, 0u,
-                                                            (uint32_t)slot), &mg, sm);
+      const int d = block_draw(D.V, q, B.row_sums,
+                               synth_sample_uniform(P.seed, (uint32_t)c->pos, 0u, (uint32_t)slot),
+                               &mg, sm);
       if (tid == 0) {
         c->dq_zmax[slot] = zmax;
-        c->dq_sum[slot] = sm.total;
+        c->dq_sum[slot] = sm.rows[0];
         s_tok = d;
         s_margin = mg;
       }
@@ -547,39 +659,17 @@ __global__ void k_accept(Dims D, Bufs B, cudaGraphConditionalHandle gen_while) {
   const bool sampled = P.temp > 0.f;
   const int k = c->k;
   if (sampled) {
-    const uint32_t pos = (uint32_t)c->pos;
-    const float u_last = synth_sample_uniform(P.seed, pos, 2u, 0u);
-    int a = 0, last = -1;
+    const float u_last = synth_sample_uniform(P.seed, (uint32_t)c->pos, 2u, 0u);
+    const int a = accept_tests(D, B, sm);
+    if (threadIdx.x <= a && threadIdx.x < k && threadIdx.x < kMaxDraft)
+      r.accept_margin[threadIdx.x] = sm.pd[threadIdx.x];
+    int last = -1;
     float fix = 0.f;
-    while (a < k && a < kMaxDraft) {
-      const float* zp = B.logits + (size_t)a * D.V;
-      const float* zq = B.draft_logits + (size_t)a * D.V;
-      const float zmp = block_zmax(zp, D.V, sm);
-      const Tempered pt{zp, zmp, P.temp};
-      const float sp = block_chunk_sums(D.V, pt, sm);
-      const Tempered qt{zq, c->dq_zmax[a], P.temp};
-      const float sq = c->dq_sum[a];
-      const int d = c->tok[a + 1];
-      const bool ok_d = d >= 0 && d < D.V && sp > 0.f && sq > 0.f;
-      const float pd = ok_d ? pt(d) / sp : 0.f;
-      const float qd = ok_d ? qt(d) / sq : 0.f;
-      const float rq = synth_sample_uniform(P.seed, pos, 1u, (uint32_t)a) * qd;
-      const float den = fmaxf(pd, rq);
-      if (threadIdx.x == 0) r.accept_margin[a] = den > 0.f ? (pd - rq) / den : 0.f;
-      if (ok_d && rq < pd) {
-        ++a;
-        continue;
-      }
-      const Residual res{pt, qt, sp, sq};
-      last = block_draw(D.V, res, u_last, &fix, sm);
-      if (last < 0) last = block_draw(D.V, pt, u_last, &fix, sm);
-      break;
-    }
-    if (last < 0) {
-      const float* zp = B.logits + (size_t)a * D.V;
-      const float zmp = block_zmax(zp, D.V, sm);
-      last = block_draw(D.V, Tempered{zp, zmp, P.temp}, u_last, &fix, sm);
-    }
+    if (a < min(k, kMaxDraft))
+      last = block_draw(D.V, residual_of(D, B, a, sm.rows[a]), B.res_sums, u_last, &fix, sm);
+    if (last < 0)
+      last = block_draw(D.V, Tempered{B.logits + (size_t)a * D.V, B.stats[a].zmax, P.temp},
+                        B.row_sums + (size_t)a * kSampChunks, u_last, &fix, sm);
     if (threadIdx.x == 0) {
       s_a = a;
       s_last = last;
@@ -664,9 +754,8 @@ __global__ void k_set_pending(Dims D, Bufs B, int row, int token, int pos) {
   const DevPolicy& P = c->pol;
   int x = token;
   if (token < 0 && P.temp > 0.f) {
-    const float* z = B.logits + (size_t)row * D.V;
-    const float zmax = block_zmax(z, D.V, sm);
-    x = block_draw(D.V, Tempered{z, zmax, P.temp},
+    x = block_draw(D.V, Tempered{B.logits + (size_t)row * D.V, B.stats[row].zmax, P.temp},
+                   B.row_sums + (size_t)row * kSampChunks,
                    synth_sample_uniform(P.seed, (uint32_t)(pos - 1), 2u, 0u), nullptr, sm);
   }
   if (threadIdx.x != 0) return;
@@ -761,6 +850,18 @@ cudaError_t launch_draft_begin(const Bufs& B, cudaGraphConditionalHandle draft_w
 cudaError_t launch_accept(const Dims& D, const Bufs& B, cudaGraphConditionalHandle gen_while,
                           cudaStream_t st) {
   return launch_ex(k_accept, dim3(1), dim3(kSampleThreads), 0, st, D, B, gen_while);
+}
+
+cudaError_t launch_row_weights(const Dims& D, const Bufs& B, RowSel sel, int mrows, int keep_mode,
+                               cudaStream_t st) {
+  const int C = samp_chunk(D.V);
+  return launch_ex(k_row_weights, dim3((D.V + C - 1) / C, mrows), dim3(kSampleThreads), 0, st, D, B,
+                   sel, keep_mode);
+}
+
+cudaError_t launch_residual_weights(const Dims& D, const Bufs& B, cudaStream_t st) {
+  const int C = samp_chunk(D.V);
+  return launch_ex(k_residual_weights, dim3((D.V + C - 1) / C), dim3(kSampleThreads), 0, st, D, B);
 }
 
 cudaError_t launch_begin_call(const Bufs& B, int max_new, cudaStream_t st) {

@@ -8,6 +8,7 @@
 //   walk  = embed(x) · layers(1..c_1) · head · decide_1 ·
 //           IF(continue) { layers(c_1+1..c_2) · head · decide_2 · IF(continue) { ... } }
 //   draft = embed(d_k) · SWITCH(l* index) { layers(1..c_j) } · head · decide
+//   (sampled decoding: the weight sums of a row after its head)
 //   verify = embed(x, d_1..d_k) · layers(1..L) · head over k + 1 rows
 // Generation graph: WHILE(emitted < max_new) { round }.
 #include <stdio.h>
@@ -87,6 +88,8 @@ size_t layout(const ssd_model_cfg& c, char* base, Dims* D, Bufs* B, WideBufs* P)
   b.act = cv.take<float>(sizeof(float) * kMaxM * d.F);
   b.logits = cv.take<float>(sizeof(float) * kMaxM * (size_t)d.V);
   b.draft_logits = cv.take<float>(sizeof(float) * kMaxDraft * (size_t)d.V);
+  b.row_sums = cv.take<float>(sizeof(float) * kMaxM * kSampChunks);
+  b.res_sums = cv.take<float>(sizeof(float) * kSampChunks);
   b.head_part = cv.take<void>(sizeof(HeadPart) * kMaxM * (size_t)kHeadParts);
   b.head_counter = cv.take<uint32_t>(sizeof(uint32_t) * kMaxM);
   b.stats = cv.take<RowStats>(sizeof(RowStats) * kMaxM);
@@ -158,6 +161,7 @@ struct ssd_ctx {
   std::vector<int> cand;
   int kmax = 0, static_l = 0, static_k = 0, q_hidden = 0, trace_T = 20, topk = 5, fixed_k = 0;
   int q_in = 3;
+  bool sampled = false;
   // graphs
   cudaGraph_t round_g = nullptr, gen_g = nullptr;
   cudaGraphExec_t round_x = nullptr, gen_x = nullptr;
@@ -283,6 +287,7 @@ cudaError_t build_walk(ssd_ctx* x, Seq& s, const std::vector<int>& cands, int j,
   if (j == 0) GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, rows(kRowsWalk), false, 0, x->cap));
   GK(enqueue_layers(x, done, cands[j], rows(kRowsWalk), 1, x->cap));
   GK(enqueue_head(x, rows(kRowsWalk), 1, x->topk, x->cap));
+  if (x->sampled) GK(launch_row_weights(x->D, x->B, rows(kRowsWalk), 1, 1, x->cap));
   GK(launch_decide(x->D, x->B, kDecideWalk, j, last ? 1 : 0, cands[j], x->final_norm,
                    x->cfg.dtype, next, 0, x->cap));
   GK(s.end());
@@ -328,6 +333,7 @@ cudaError_t build_draft_phase(ssd_ctx* x, cudaGraph_t body) {
     GK(enqueue_layers(x, 0, cands[0], rows(kRowsDraft), 1, x->cap));
   }
   GK(enqueue_head(x, rows(kRowsDraft), 1, x->topk, x->cap));
+  if (x->sampled) GK(launch_row_weights(x->D, x->B, rows(kRowsDraft), 1, 2, x->cap));
   GK(launch_decide(x->D, x->B, kDecideDraft, 0, 0, 0, x->final_norm, x->cfg.dtype, 0, hw,
                    x->cap));
   return w.end();
@@ -353,6 +359,10 @@ cudaError_t build_round(ssd_ctx* x, cudaGraph_t g, cudaGraphConditionalHandle ge
   const int mrows = spec ? std::min(x->kmax + 1, kMaxM) : 1;
   GK(enqueue_layers(x, 0, x->D.L, rows(kRowsVerify), mrows, x->cap));
   GK(enqueue_head(x, rows(kRowsVerify), mrows, x->topk, x->cap));
+  if (x->sampled) {
+    GK(launch_row_weights(x->D, x->B, rows(kRowsVerify), mrows, 0, x->cap));
+    if (spec) GK(launch_residual_weights(x->D, x->B, x->cap));
+  }
   GK(launch_accept(x->D, x->B, gen, x->cap));
   return s.end();
 }
@@ -686,12 +696,12 @@ ssd_status ssd_set_policy(ssd_ctx* x, const ssd_policy* p) {
                           cudaMemcpyHostToDevice, x->stream));
   CK(x, cudaStreamSynchronize(x->stream));
   // The graphs depend on the policy kind, the candidate (or static) exit
-  // layers, kmax and topk; everything else is read on the device from the
-  // policy just copied.
+  // layers, kmax, topk and whether tokens are sampled; everything else is
+  // read on the device from the policy just copied.
   const int kmax_new = p->kind == SSD_POLICY_AR ? 0 : p->kmax;
   const bool same_graphs = x->have_policy && x->kind == p->kind && x->cand == cand &&
                            x->kmax == kmax_new && x->static_l == p->static_l &&
-                           x->topk == dp.topk;
+                           x->topk == dp.topk && x->sampled == (dp.temp > 0.f);
   x->kind = p->kind;
   x->cand = cand;
   x->kmax = kmax_new;
@@ -702,6 +712,7 @@ ssd_status ssd_set_policy(ssd_ctx* x, const ssd_policy* p) {
   x->q_in = dp.q_in;
   x->trace_T = dp.trace_T;
   x->topk = dp.topk;
+  x->sampled = dp.temp > 0.f;
   if (same_graphs) return SSD_OK;
   cudaError_t e = build_graphs(x);
   if (e != cudaSuccess) {
@@ -724,6 +735,9 @@ ssd_status ssd_prefill(ssd_ctx* x, const int32_t* ids, int32_t n, int32_t* first
   int last_row = 0;
   ssd_status s = run_prompt(x, n, &last_row);
   if (s) return s;
+  if (x->sampled)
+    CK(x, launch_row_weights(x->D, x->B, rows_explicit(0, last_row + 1, nullptr), last_row + 1, 0,
+                             x->stream));
   CK(x, launch_set_pending(x->D, x->B, last_row, -1, n, x->stream));
   Ctl c;
   if ((s = read_ctl(x, &c))) return s;

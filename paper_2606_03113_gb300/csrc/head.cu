@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kHThreads) k_head_stats(const Dims D, const Bu
   __shared__ HeadSmem sm;
   int pos0, M;
   resolve_rows(B.ctl, sel, pos0, M);
-  const int m = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+  const int m = blockIdx.y, tid = threadIdx.x;
   if (m >= M) return;
   const float* z = B.logits + (size_t)m * D.V;
   const int nchunks = (D.V + kHChunk - 1) / kHChunk;

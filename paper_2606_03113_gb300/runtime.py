@@ -224,8 +224,9 @@ def kernels_per_round(trace: dict, n_layers: int, kind: int, bf16: bool = True) 
     """Kernel launches of one round of the round graph, from its record:
     round_begin, walk (embed; per visited segment its layers, head, decide),
     draft_begin, drafts (embed, layers 1..l*, head, decide), verify (embed,
-    all layers, head), accept.  A head counts once: its product and the
-    statistics behind it."""
+    all layers, head), accept.  A head counts once (its product, the
+    statistics and, in sampled decoding, the weight sums behind it), and so
+    does attention (its splits and their merge)."""
     n = 1  # round_begin
     if trace["kcap"] > 0:
         prev = 0
