@@ -38,7 +38,9 @@ __device__ float trace_conf(const Ctl* c, int T) {
 // k_row_weights reads the rows' logits on all SMs and leaves the weights' sums
 // over at most kSampChunks runs of the vocabulary; a draw then scans those
 // sums and walks the one run that holds it.  One block used to read whole
-// rows, each thread a run of its own: @SAMP@
+// rows, each thread a run of its own: 48 sampled tokens of the 8B widths (4
+// layers, 128256 tokens) took 43.8 ms, now 25.3 (the bf16 decode attention
+// changed in between, about 2 of the 18.5 ms).
 // Every reduction below runs in a fixed order that depends on the vocabulary
 // alone, so a draw depends only on the logits and the uniform, never on
 // scheduling.
