@@ -14,6 +14,7 @@ namespace ssd {
 
 constexpr int kMaxM = 17;          // rows of one verify pass: pending token + up to 16 drafts
 constexpr int kMaxDraft = 16;
+constexpr int kHeadRows = kMaxM + kMaxDraft;  // rows of logits and statistics (prompts)
 constexpr int kMaxCand = SSD_TRACE_MAXC;
 constexpr int kTraceCap = 64;      // C_trace window capacity
 constexpr int kSampChunks = 256;  // chunk sums of a row's sampling weights, at most
@@ -173,15 +174,16 @@ struct Bufs {
   float* attn_ml;    // [kMaxM][Hq][nsplit][2] partial (max, sum)
   uint32_t* attn_counter;  // [Hkv][kMaxM] split tickets of the attention merge
   uint32_t* chain_bar;     // [2] grid-wide phase arrivals / blocks done of the chain kernel
-  float* draft_logits;     // [kMaxDraft][V] exit logits of each draft (sampled decoding)
-  float* row_sums;         // [kMaxM][kSampChunks] sampling weights of each row's chunks
+  float* draft_logits;     // [kMaxDraft][V] exit logits of each draft (sampled decoding);
+                           // the rows behind those of logits
+  float* row_sums;         // [kHeadRows][kSampChunks] sampling weights of each row's chunks
   float* res_sums;         // [kSampChunks] the same of a rejected draft's residual
   float* attn_out;   // [kMaxM][qd]
   float* act;        // [kMaxM][F]
-  float* logits;     // [kMaxM][V] of the last exit head
-  void* head_part;   // [kMaxM][kHeadParts] statistics of a row's chunks
-  uint32_t* head_counter;  // [kMaxM] chunk tickets of the exit-head statistics
-  RowStats* stats;   // [kMaxM]
+  float* logits;     // [kMaxM][V] of the last exit head (a prompt's: [kHeadRows][V])
+  void* head_part;   // [kHeadRows][kHeadParts] statistics of a row's chunks
+  uint32_t* head_counter;  // [kHeadRows] chunk tickets of the exit-head statistics
+  RowStats* stats;   // [kHeadRows]
   float2* rope;      // [max_seq][hd/2] (cos, sin)
   void* kv;          // [L][2][Hkv][max_seq][hd]
   float* qparams;    // Q-network parameters

@@ -742,7 +742,16 @@ __global__ void k_reset_sequence(Bufs B) {
 __global__ void k_trace_push(Bufs B, int first_row, int n_rows) {
   pdl_wait();
   pdl_launch_dependents();
-  for (int i = 0; i < n_rows; ++i) trace_push(B.ctl, B.stats[first_row + i].pmax);
+  // entry i by lane i % 32 (the window keeps the last kTraceCap); then the ends
+  Ctl* c = B.ctl;
+  const int head = c->trace_head, n = c->trace_n;
+  for (int i = max(0, n_rows - kTraceCap) + (int)threadIdx.x; i < n_rows; i += 32)
+    c->trace[(head + i) % kTraceCap] = B.stats[first_row + i].pmax;
+  __syncwarp();
+  if (threadIdx.x == 0) {
+    c->trace_head = (head + n_rows) % kTraceCap;
+    c->trace_n = min(n + n_rows, kTraceCap);
+  }
 }
 
 // Pending token after a prompt: the given token, or (token < 0) the argmax
@@ -875,7 +884,7 @@ cudaError_t launch_reset_sequence(const Bufs& B, cudaStream_t st) {
 }
 
 cudaError_t launch_trace_push(const Bufs& B, int first_row, int n_rows, cudaStream_t st) {
-  return launch_ex(k_trace_push, dim3(1), dim3(1), 0, st, B, first_row, n_rows);
+  return launch_ex(k_trace_push, dim3(1), dim3(32), 0, st, B, first_row, n_rows);
 }
 
 cudaError_t launch_set_pending(const Dims& D, const Bufs& B, int stats_row, int token, int pos,

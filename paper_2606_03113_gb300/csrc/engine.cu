@@ -86,13 +86,13 @@ size_t layout(const ssd_model_cfg& c, char* base, Dims* D, Bufs* B, WideBufs* P)
   b.chain_bar = cv.take<uint32_t>(sizeof(uint32_t) * 2);
   b.attn_out = cv.take<float>(sizeof(float) * kMaxM * d.qd);
   b.act = cv.take<float>(sizeof(float) * kMaxM * d.F);
-  b.logits = cv.take<float>(sizeof(float) * kMaxM * (size_t)d.V);
-  b.draft_logits = cv.take<float>(sizeof(float) * kMaxDraft * (size_t)d.V);
-  b.row_sums = cv.take<float>(sizeof(float) * kMaxM * kSampChunks);
+  b.logits = cv.take<float>(sizeof(float) * kHeadRows * (size_t)d.V);
+  b.draft_logits = base ? b.logits + kMaxM * (size_t)d.V : nullptr;
+  b.row_sums = cv.take<float>(sizeof(float) * kHeadRows * kSampChunks);
   b.res_sums = cv.take<float>(sizeof(float) * kSampChunks);
-  b.head_part = cv.take<void>(sizeof(HeadPart) * kMaxM * (size_t)kHeadParts);
-  b.head_counter = cv.take<uint32_t>(sizeof(uint32_t) * kMaxM);
-  b.stats = cv.take<RowStats>(sizeof(RowStats) * kMaxM);
+  b.head_part = cv.take<void>(sizeof(HeadPart) * kHeadRows * (size_t)kHeadParts);
+  b.head_counter = cv.take<uint32_t>(sizeof(uint32_t) * kHeadRows);
+  b.stats = cv.take<RowStats>(sizeof(RowStats) * kHeadRows);
   b.rope = cv.take<float2>(sizeof(float2) * (size_t)d.max_seq * (d.hd / 2));
   b.kv = cv.take<void>(elt * (size_t)d.L * 2 * d.Hkv * (size_t)d.max_seq * d.hd);
   // largest network: d + 1 inputs (pooled state), kMaxQHidden hidden units
@@ -436,7 +436,7 @@ std::vector<int> wide_chunks(const ssd_ctx* x, int n) {
 
 // run_prompt for bf16 prompts longer than one decode tile: chunks of up to
 // P.cap rows through the wide kernels, then the exit head over the last
-// trace_T rows, at most kPrefillChunk at a time.
+// trace_T rows.
 ssd_status run_prompt_wide(ssd_ctx* x, int n, int* last_row) {
   const int T = x->trace_T, L = x->D.L;
   int c0 = 0;
@@ -445,12 +445,11 @@ ssd_status run_prompt_wide(ssd_ctx* x, int n, int* last_row) {
                             x->stream));
     for (int l = 0; l < L; ++l)
       CK(x, launch_layer_wide(x->D, x->B, x->P, x->xmaps, x->layers[l],
-                              l + 1 < L ? x->layers[l + 1].attn_norm : nullptr, l, M, c0, x->stream));
+                              l + 1 < L ? x->layers[l + 1].attn_norm : x->final_norm, l, M, c0, x->stream));
     for (int r = std::max(0, std::min(n - T, n - 1) - c0); r < M;) {
-      const int m = std::min(kPrefillChunk, M - r);
-      CK(x, launch_take_rows(x->D, x->B, x->P, r, m, x->stream));
-      CK(x, enqueue_head(x, rows_explicit(c0 + r, m, x->B.pre_tok + c0 + r), kPrefillChunk, x->topk,
-                         x->stream));
+      const int m = std::min(kHeadRows, M - r);
+      CK(x, launch_head_wide(x->D, x->B, x->P, x->xmaps, *lm_map(x), r, m, x->stream));
+      CK(x, launch_head_stats(x->D, x->B, x->topk, rows_explicit(c0 + r, m, nullptr), m, x->stream));
       CK(x, launch_trace_push(x->B, 0, m, x->stream));
       *last_row = m - 1;
       r += m;
@@ -612,7 +611,7 @@ ssd_status ssd_init_model(const ssd_model_cfg* cfg, const ssd_weights* w, void* 
   e = cudaMemcpyAsync(x->B.rope, rope.data(), sizeof(float2) * rope.size(), cudaMemcpyHostToDevice,
                       x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->B.ctl, 0, sizeof(Ctl), x->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(x->B.head_counter, 0, sizeof(uint32_t) * kMaxM, x->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(x->B.head_counter, 0, sizeof(uint32_t) * kHeadRows, x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->B.ss, 0, sizeof(float) * 2 * kMaxM, x->stream);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(x->B.ss_part, 0, sizeof(float) * 2 * (size_t)x->D.ss_nt * kMaxM, x->stream);

@@ -68,8 +68,10 @@ cudaError_t launch_embed_wide(const Dims& D, const Bufs& B, const WideBufs& P, c
 cudaError_t launch_layer_wide(const Dims& D, const Bufs& B, const WideBufs& P, const WideMaps& xm,
                               const LayerW& w, const void* next_norm, int layer, int M, int pos0,
                               cudaStream_t st);
-cudaError_t launch_take_rows(const Dims& D, const Bufs& B, const WideBufs& P, int row0, int M,
-                             cudaStream_t st);
+// Logits of the chunk's rows row0 .. row0 + M - 1 (at most kHeadRows) after its
+// last layer, whose next_norm was the final norm.
+cudaError_t launch_head_wide(const Dims& D, const Bufs& B, const WideBufs& P, const WideMaps& xm,
+                             const CUtensorMap& lm, int row0, int M, cudaStream_t st);
 
 // mrows is the largest number of rows a launch may see: 1 selects the
 // single-row kernels, more the multi-row ones (bf16: the tensor-core instance

@@ -25,7 +25,11 @@
 // the Llama-2-7B shape: gate/up 126.6 us (1.46 PFLOP/s with both parts), QKV
 // 83.7, down 75.0, O 35.3 us; a 512-token prompt through four layers takes
 // 1.9 ms against 18.0 ms in 32 passes of 16 rows, 2043 tokens of the 13B
-// shape 9.6 ms against 104.6 ms.
+// shape 9.6 ms against 104.6 ms.  The exit head of a prompt's last rows (20 of
+// them feed the C_trace window) is such a product too, one pass over the LM
+// head instead of one per 16 rows: a 93-token prompt of the 8B widths (4
+// layers, 128256 tokens) takes 1912 us against 2188, 512 tokens of the 7B
+// widths 2281 against 2371.
 // Attention (k_attn_wide): 64 query rows x one head per block, 64-key steps
 // with a running maximum; scores and outputs on mma.sync with the fp32
 // operand (queries, probabilities) in three bf16 parts, 24 bits, so nothing
@@ -60,7 +64,7 @@ constexpr int kWChunk = 16;           // tokens per epilogue step of a warp
 // us (94.5 us with 512 columns at a time, 76.5 us with all of K).
 constexpr int kWSeg = 16;
 
-enum WKind : int { kWQkv = 0, kWResid = 1, kWGateUp = 2 };
+enum WKind : int { kWQkv = 0, kWResid = 1, kWGateUp = 2, kWHead = 3 };
 
 template <int TT>
 struct WL {
@@ -85,6 +89,7 @@ struct WArgs {
   WideBufs P;
   int N, K, nks, nrt, ntt;     // rows, columns, stages, row tiles, token tiles
   int M, pos0, layer;
+  int row0;                    // first of the M input rows
   const float* ss_in;          // per-tile sums of squares of the input rows, or null
   float* ss_out;               // residual: the same for the rows written
   const __nv_bfloat16* gnext;  // residual: norm weights of the next product (null: none)
@@ -226,7 +231,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
             }
             weights(slot, tile, kc);
           }
-          tma_load_3d(smem + (size_t)slot * S::Stage + S::A, &xmap, kc * kWK, tt * TT, 0, &full[slot]);
+          tma_load_3d(smem + (size_t)slot * S::Stage + S::A, &xmap, kc * kWK, a.row0 + tt * TT, 0, &full[slot]);
           if (++slot == NS) {
             slot = 0;
             ph ^= 1u;
@@ -347,6 +352,11 @@ __global__ void __launch_bounds__(kWThreads, 1)
           }
           const float s = warp_sum16(sq, lane);
           if (!(lane & 1)) red[q * TT + tl + (lane >> 1)] = s;
+        } else if constexpr (KIND == kWHead) {
+          const int row = rt * kWR + 32 * q + lane;
+#pragma unroll
+          for (int j = 0; j < kWChunk; ++j)
+            if (row < a.N && j < nt) a.B.logits[(size_t)(t0 + tl + j) * D.V + row] = v[j] * srs[tl + j];
         } else {
           // swap halves: warps of rows 0-63 finish tokens 0-7 of the step,
           // warps of rows 64-127 tokens 8-15
@@ -613,7 +623,7 @@ __global__ void __launch_bounds__(kAWThreads, 2)
   }
 }
 
-// ----------------------------------------------- embedding and row hand-over
+// ------------------------------------------------------------- embedding
 
 // Row m of a chunk: h = embed[tok[m]], its split parts under the first norm's
 // weights, and its sums of squares per 128 columns.
@@ -649,27 +659,6 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// Rows row0.. of the chunk's residual stream as rows 0.. of the decode
-// buffers, with their sums of squares per 256 columns, for the exit head.
-__global__ void __launch_bounds__(256)
-    k_take_rows(const Dims D, const Bufs B, const WideBufs P, int row0) {
-  pdl_wait();
-  pdl_launch_dependents();
-  const int m = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const float* src = P.h + (size_t)(row0 + m) * D.d;
-  float* dst = B.h + (size_t)m * D.d;
-  for (int c = warp; c < D.ss_nt; c += 8) {
-    float sp = 0.f;
-    for (int i = c * 256 + lane; i < min(D.d, c * 256 + 256); i += 32) {
-      const float v = src[i];
-      dst[i] = v;
-      sp = fmaf(v, v, sp);
-    }
-    sp = warp_sum(sp);
-    if (lane == 0) B.ss_part[(size_t)c * kMaxM + m] = sp;
-  }
-}
-
 // ------------------------------------------------------------- host side
 
 namespace {
@@ -683,6 +672,7 @@ template <int TT>
 cudaError_t wide_prep_all() {
   cudaError_t e = wide_prep<TT, kWQkv>();
   if (e == cudaSuccess) e = wide_prep<TT, kWResid>();
+  if (e == cudaSuccess) e = wide_prep<TT, kWHead>();
   return e != cudaSuccess ? e : wide_prep<TT, kWGateUp>();
 }
 
@@ -761,9 +751,18 @@ cudaError_t launch_embed_wide(const Dims& D, const Bufs& B, const WideBufs& P, c
                    static_cast<const __nv_bfloat16*>(gnorm), toks);
 }
 
-cudaError_t launch_take_rows(const Dims& D, const Bufs& B, const WideBufs& P, int row0, int M,
-                             cudaStream_t st) {
-  return launch_ex(k_take_rows, dim3(M), dim3(256), 0, st, D, B, P, row0);
+cudaError_t launch_head_wide(const Dims& D, const Bufs& B, const WideBufs& P, const WideMaps& xm,
+                             const CUtensorMap& lm, int row0, int M, cudaStream_t st) {
+  WArgs a{};
+  a.D = D;
+  a.B = B;
+  a.P = P;
+  a.M = M;
+  a.row0 = row0;
+  a.N = D.V;
+  a.K = D.d;
+  a.ss_in = P.ss + row0;  // written by the last layer's down projection
+  return wide_launch<kWHead>(lm, xm.xn, a, st);
 }
 
 cudaError_t launch_layer_wide(const Dims& D, const Bufs& B, const WideBufs& P, const WideMaps& xm,
