@@ -12,7 +12,7 @@ REPO = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD_DIR = os.path.join(HERE, "_build")
 LIB_PATH = os.path.join(BUILD_DIR, "libssd.so")
-SOURCES = ["gemv.cu", "tile.cu", "wide.cu", "head.cu", "attention.cu", "control.cu", "engine.cu"]
+SOURCES = ["gemv.cu", "fp32.cu", "tile.cu", "wide.cu", "head.cu", "attention.cu", "control.cu", "engine.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
               "-Xptxas", "-warn-spills"]

@@ -19,7 +19,6 @@ constexpr int kMaxCand = SSD_TRACE_MAXC;
 constexpr int kTraceCap = 64;      // C_trace window capacity
 constexpr int kSampChunks = 256;  // chunk sums of a row's sampling weights, at most
 constexpr int kTopK = 8;           // max k of the token confidence
-constexpr int kWarps = 8;          // warps per block of the matrix-vector kernels
 constexpr int kAttnKeys = 64;      // keys per attention split (two per lane)
 constexpr int kLayerKernels = 5;   // launches per layer: qkv, attention, o, gate/up, down
 
@@ -151,7 +150,7 @@ struct LayerW {
 
 // Shapes and buffers every kernel may need.
 struct Dims {
-  int32_t L, d, Hq, Hkv, hd, F, V, max_seq, qd, kvd, nsplit, num_sms, ss_tiles, max_tiles;
+  int32_t L, d, Hq, Hkv, hd, F, V, max_seq, qd, kvd, nsplit, num_sms, max_tiles;
   int32_t attn_keys;  // keys per attention split (bf16 kernel)
   int32_t ss_nt;  // 256-row tiles of a residual row (tensor-core kernels' sum-of-squares parts)
   float eps;
@@ -160,14 +159,11 @@ struct Dims {
 struct Bufs {
   Ctl* ctl;
   float* h;          // [kMaxM][d] residual stream
-  float* ss;         // [2][kMaxM] sum of squares of h rows: [0] after down/embed, [1] after O
-  float* ss_tile;    // [2][2][max blocks][kMaxM] per-block (running, split) partials of ss
-  uint32_t* ss_counter;  // [2] block tickets of the residual kernels
   float* ss_part;    // [2][ss_nt][kMaxM] sum of squares of h rows per 256-row tile (bf16
                      // kernels): written by the tile that finishes those rows, summed in
                      // tile order by the RMSNorm that reads them
   float* gpart;      // partial tile sums of blocks sharing a tile: [num_sms][2][32][kMaxM]
-                     // (fp32 kernels) or [num_sms][2][2][kMaxM][128] (bf16 tensor-core kernels)
+                     // (gemv.cu) or [num_sms][2][2][kMaxM][128] (bf16 tensor-core kernels)
   uint32_t* tile_counter;      // [max tiles] tickets of shared tiles
   float* xq;         // [kMaxM][qd] rotated queries
   float* attn_part;  // [kMaxM][Hq][nsplit][hd] unnormalised partial outputs

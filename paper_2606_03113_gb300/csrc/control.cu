@@ -276,15 +276,14 @@ __global__ void __launch_bounds__(kSampleThreads) k_residual_weights(const Dims 
   if (threadIdx.x == 0) B.res_sums[blockIdx.x] = sm.part[kSampleThreads - 1];
 }
 
-// h[m] = embed[token_m] (fp32) and the row's sum of squares for the first
-// RMSNorm.  One block per row.  Optionally sets the drafting switch handle to
+// h[m] = embed[token_m] (fp32) and the sums of squares of its 256-element parts
+// for the first RMSNorm (bf16 models).  One block per row.  Optionally sets the drafting switch handle to
 // the chosen exit-layer index.
 template <typename T>
 __global__ void k_embed(Dims D, Bufs B, const T* __restrict__ emb, RowSel sel,
                         cudaGraphConditionalHandle sw) {
   pdl_wait();
   pdl_launch_dependents();
-  __shared__ float red[32];
   Ctl* c = B.ctl;
   int pos0, M;
   resolve_rows(c, sel, pos0, M);
@@ -316,20 +315,7 @@ __global__ void k_embed(Dims D, Bufs B, const T* __restrict__ emb, RowSel sel,
     sp = warp_sum(sp);
     if (lane == 0) B.ss_part[(size_t)c * kMaxM + m] = sp;
   }
-  float ss = 0.f;
-  for (int i = threadIdx.x; i < D.d; i += blockDim.x) {
-    const float v = Elem<T>::to_f(row[i]);
-    hr[i] = v;
-    ss = fmaf(v, v, ss);
-  }
-  ss = warp_sum(ss);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float s = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-    B.ss[m] = s;
-  }
+  for (int i = threadIdx.x; i < D.d; i += blockDim.x) hr[i] = Elem<T>::to_f(row[i]);
 }
 
 // Draft cap of the round: min(kmax, tokens still to emit - 1), the static

@@ -61,7 +61,6 @@ size_t layout(const ssd_model_cfg& c, char* base, Dims* D, Bufs* B, WideBufs* P)
   d.nsplit = (c.max_seq + kAttnKeys - 1) / kAttnKeys;
   d.eps = c.rms_eps;
   d.num_sms = kMaxBlocks;  // set to the device's SM count at init
-  d.ss_tiles = (c.d_model + 15) / 16;
   d.ss_nt = (c.d_model + 255) / 256;
   d.max_tiles = std::max(
       std::max(head_tiles(c.vocab), c.ffn_dim / 16 + 1),
@@ -71,9 +70,6 @@ size_t layout(const ssd_model_cfg& c, char* base, Dims* D, Bufs* B, WideBufs* P)
   Bufs b{};
   b.ctl = cv.take<Ctl>(sizeof(Ctl));
   b.h = cv.take<float>(sizeof(float) * kMaxM * d.d);
-  b.ss = cv.take<float>(sizeof(float) * 2 * kMaxM);
-  b.ss_tile = cv.take<float>(sizeof(float) * 2 * 2 * kMaxM * (size_t)kMaxBlocks);
-  b.ss_counter = cv.take<uint32_t>(sizeof(uint32_t) * 2);
   b.ss_part = cv.take<float>(sizeof(float) * 2 * (size_t)d.ss_nt * kMaxM);
   b.gpart = cv.take<float>(sizeof(float) * std::max((size_t)kMaxBlocks * 2 * 32 * kMaxM,
                                                       tile_part_floats(kMaxBlocks)));
@@ -612,10 +608,8 @@ ssd_status ssd_init_model(const ssd_model_cfg* cfg, const ssd_weights* w, void* 
                       x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->B.ctl, 0, sizeof(Ctl), x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->B.head_counter, 0, sizeof(uint32_t) * kHeadRows, x->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(x->B.ss, 0, sizeof(float) * 2 * kMaxM, x->stream);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(x->B.ss_part, 0, sizeof(float) * 2 * (size_t)x->D.ss_nt * kMaxM, x->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(x->B.ss_counter, 0, sizeof(uint32_t) * 2, x->stream);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(x->B.attn_counter, 0, sizeof(uint32_t) * (size_t)x->D.Hkv * kMaxM, x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->B.chain_bar, 0, sizeof(uint32_t) * 2, x->stream);

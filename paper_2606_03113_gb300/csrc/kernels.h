@@ -73,6 +73,13 @@ cudaError_t launch_layer_wide(const Dims& D, const Bufs& B, const WideBufs& P, c
 cudaError_t launch_head_wide(const Dims& D, const Bufs& B, const WideBufs& P, const WideMaps& xm,
                              const CUtensorMap& lm, int row0, int M, cudaStream_t st);
 
+// fp32 decoders (fp32.cu): the matrices of a layer (0 QKV, 2 O, 3 gate/up,
+// 4 down) and the LM head.
+cudaError_t launch_f32_part(const Dims& D, const Bufs& B, const LayerW& w, int layer, int part,
+                              RowSel sel, int mrows, cudaStream_t st);
+cudaError_t launch_f32_head(const Dims& D, const Bufs& B, const void* lm, const void* final_norm,
+                              RowSel sel, int mrows, cudaStream_t st);
+
 // mrows is the largest number of rows a launch may see: 1 selects the
 // single-row kernels, more the multi-row ones (bf16: the tensor-core instance
 // with 8, 16 or 24 token rows, the smallest that holds mrows).  big
