@@ -152,15 +152,18 @@ __global__ void __launch_bounds__(kAThreads, 3) k_attn(Dims D, Bufs B, int layer
     pw[ka] = pa;
     pw[kb2] = pb;
     __syncwarp();
+    // a row whose keys all lie in this split is finished here (its merge would
+    // be one partial with weight 1)
+    const bool whole = pos < kAK;
     const size_t pidx = ((size_t)m * D.Hq + qh) * D.nsplit + split;
-    float* part = B.attn_part + pidx * hd;
+    float* part = whole ? B.attn_out + (size_t)m * D.qd + (size_t)qh * hd : B.attn_part + pidx * hd;
     for (int dd = lane; dd < hd; dd += 32) {
       float o = 0.f;
 #pragma unroll 8
       for (int s = 0; s < nkeys; ++s) o = fmaf(pw[s], Vs[s * hd + dd], o);
-      part[dd] = o;
+      part[dd] = whole ? o / l : o;
     }
-    if (lane == 0) {
+    if (lane == 0 && !whole) {
       B.attn_ml[2 * pidx] = mx;
       B.attn_ml[2 * pidx + 1] = l;
     }
@@ -171,9 +174,10 @@ __global__ void __launch_bounds__(kAThreads, 3) k_attn(Dims D, Bufs B, int layer
   // One thread per row takes the ticket with an acquire-release add after
   // the block barrier, which publishes the block's partials and, for the
   // last split, makes every other split's visible to the whole block.
+  if (pos0 + M - 1 < kAK) return;  // every row is finished
   if (threadIdx.x == 0) s_nlast = 0;
   __syncthreads();
-  if (threadIdx.x < M && threadIdx.x >= m_first) {
+  if (threadIdx.x < M && threadIdx.x >= m_first && pos0 + (int)threadIdx.x >= kAK) {
     const int m = threadIdx.x;
     const int nsp = (pos0 + m) / kAK + 1;
     uint32_t* cnt = B.attn_counter + (size_t)g * kMaxM + m;

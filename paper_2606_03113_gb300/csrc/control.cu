@@ -15,12 +15,6 @@ __device__ __forceinline__ void set_cond(cudaGraphConditionalHandle h, unsigned 
   if (h) cudaGraphSetConditional(h, v);
 }
 
-__device__ __forceinline__ void trace_push(Ctl* c, float p) {
-  c->trace[c->trace_head] = p;
-  c->trace_head = (c->trace_head + 1) % kTraceCap;
-  if (c->trace_n < kTraceCap) ++c->trace_n;
-}
-
 // C_trace = -(1/n) sum log pmax over the n = min(T, count) most recent entries
 // (§3.1.1, average trace of token confidence).
 __device__ float trace_conf(const Ctl* c, int T) {
@@ -663,43 +657,69 @@ __global__ void k_accept(Dims D, Bufs B, cudaGraphConditionalHandle gen_while) {
       s_last = last;
       r.fix_margin = fix;
     }
+    __syncthreads();
   }
-  if (threadIdx.x != 0) return;
-  int a = 0, g;
-  if (sampled) {
-    a = s_a;
-    g = s_last;
-    if (g < 0 || g >= D.V) {
-      atomicOr(&c->err, (int)kErrToken);
-      g = 0;
+  // The record of the round, a lane per verification row: one round trip for
+  // all rows' statistics instead of one after the other.
+  __shared__ int s_round, s_keep;
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    const bool on = lane <= k && lane < kMaxM;
+    const int am = on ? B.stats[lane].argmax : 0;
+    const float mg = on ? B.stats[lane].margin : 0.f, pm = on ? B.stats[lane].pmax : 0.f;
+    const int draft = lane < k && lane < kMaxDraft ? c->tok[lane + 1] : -1;  // d_(lane + 1)
+    const int pos = c->pos, n_out = c->n_out, round = c->round_idx;
+    const int head = c->trace_head, n_trace = c->trace_n, max_new = c->max_new, lstar = c->lstar;
+    int a, g;
+    if (sampled) {
+      a = s_a;
+      g = s_last;
+      if (g < 0 || g >= D.V) {
+        if (lane == 0) atomicOr(&c->err, (int)kErrToken);
+        g = 0;
+      }
+    } else {
+      // leading rows whose argmax is the next draft
+      a = __ffs(~__ballot_sync(0xffffffffu, lane < k && am == draft)) - 1;
+      g = __shfl_sync(0xffffffffu, am, a);
     }
-  } else {
-    while (a < k && c->tok[a + 1] == B.stats[a].argmax) ++a;
-    g = B.stats[a].argmax;
+    if (on) {
+      r.verify_tok[lane] = am;
+      r.verify_margin[lane] = mg;
+      r.verify_pmax[lane] = pm;
+    }
+    if (lane <= a) {
+      const int tok = lane < a ? draft : g;
+      r.emitted[lane] = tok;
+      if (n_out + lane < D.max_seq) B.out_tok[n_out + lane] = tok;
+      c->trace[(head + lane) % kTraceCap] = pm;
+    }
+    if (lane == 0) {
+      c->trace_head = (head + a + 1) % kTraceCap;
+      c->trace_n = min(n_trace + a + 1, kTraceCap);
+      r.sampled = sampled ? 1 : 0;
+      r.lstar = lstar;
+      r.k = k;
+      r.a = a;
+      r.n_emit = a + 1;
+      if (round >= D.max_seq) atomicOr(&c->err, (int)kErrTraceFull);
+      c->n_out = n_out + a + 1;
+      c->pos = pos + a + 1;
+      c->x = g;
+      c->round_idx = round + 1;
+      s_round = round;
+      s_keep = n_out + a + 1 < max_new ? 1 : 0;
+    }
   }
-  for (int i = 0; i <= k; ++i) {
-    r.verify_tok[i] = B.stats[i].argmax;
-    r.verify_margin[i] = B.stats[i].margin;
-    r.verify_pmax[i] = B.stats[i].pmax;
+  __syncthreads();
+  if (s_round < D.max_seq) {
+    static_assert(sizeof(ssd_round_trace) % sizeof(int32_t) == 0, "copied by words");
+    const int32_t* from = reinterpret_cast<const int32_t*>(&r);
+    int32_t* to = reinterpret_cast<int32_t*>(B.traces + s_round);
+    for (int i = threadIdx.x; i < (int)(sizeof(ssd_round_trace) / sizeof(int32_t)); i += blockDim.x)
+      to[i] = from[i];
   }
-  for (int i = 0; i < a; ++i) r.emitted[i] = c->tok[i + 1];
-  r.emitted[a] = g;
-  for (int i = 0; i <= a; ++i) {
-    if (c->n_out + i < D.max_seq) B.out_tok[c->n_out + i] = r.emitted[i];
-    trace_push(c, B.stats[i].pmax);
-  }
-  r.sampled = sampled ? 1 : 0;
-  r.lstar = c->lstar;
-  r.k = k;
-  r.a = a;
-  r.n_emit = a + 1;
-  if (c->round_idx < D.max_seq) B.traces[c->round_idx] = r;
-  else atomicOr(&c->err, (int)kErrTraceFull);
-  c->n_out += a + 1;
-  c->pos += a + 1;
-  c->x = g;
-  c->round_idx += 1;
-  set_cond(gen_while, c->n_out < c->max_new ? 1u : 0u);
+  if (threadIdx.x == 0) set_cond(gen_while, (unsigned)s_keep);
 }
 
 __global__ void k_begin_call(Bufs B, int max_new) {
