@@ -604,8 +604,13 @@ __global__ void __launch_bounds__(256) k_attn_merge(const Dims D, const Bufs B, 
       O.w = fmaf(wj, p[j].w, O.w);
     }
   }
-  *reinterpret_cast<float4*>(B.attn_out + (size_t)i * kRHd + 4 * lane) =
-      make_float4(O.x / L, O.y / L, O.z / L, O.w / L);
+  // as the O projection reads it
+  uint2 hi, lo;
+  split2(O.x / L, O.y / L, hi.x, lo.x);
+  split2(O.z / L, O.w / L, hi.y, lo.y);
+  __nv_bfloat16* xo = B.xs_o + (size_t)i * kRHd + 4 * lane;
+  *reinterpret_cast<uint2*>(xo) = hi;
+  *reinterpret_cast<uint2*>(xo + (size_t)kMaxM * D.qd) = lo;
 }
 
 // Keys per split of the bf16 kernel: 64, or 128 where 64 would make more

@@ -168,14 +168,19 @@ struct Bufs {
   float* xq;         // [kMaxM][qd] rotated queries
   float* attn_part;  // [kMaxM][Hq][nsplit][hd] unnormalised partial outputs
   float* attn_ml;    // [kMaxM][Hq][nsplit][2] partial (max, sum)
+  // bf16: inputs of the products as high and low planes
+  __nv_bfloat16* xs_h;  // [2][kMaxM][d] residual rows times the norm weights of the matrix behind
+  __nv_bfloat16* xs_o;  // [2][kMaxM][qd] attention outputs
+  __nv_bfloat16* xs_a;  // [2][kMaxM][F] SwiGLU outputs
+  __nv_bfloat16* xs_x;  // [2][kMaxM][max(d, qd, F)] inputs of ssd_op_gemv
   uint32_t* attn_counter;  // [Hkv][kMaxM] split tickets of the attention merge
   uint32_t* chain_bar;     // [2] grid-wide phase arrivals / blocks done of the chain kernel
   float* draft_logits;     // [kMaxDraft][V] exit logits of each draft (sampled decoding);
                            // the rows behind those of logits
   float* row_sums;         // [kHeadRows][kSampChunks] sampling weights of each row's chunks
   float* res_sums;         // [kSampChunks] the same of a rejected draft's residual
-  float* attn_out;   // [kMaxM][qd]
-  float* act;        // [kMaxM][F]
+  float* attn_out;   // fp32: [kMaxM][qd]
+  float* act;        // fp32: [kMaxM][F]
   float* logits;     // [kMaxM][V] of the last exit head (a prompt's: [kHeadRows][V])
   void* head_part;   // [kHeadRows][kHeadParts] statistics of a row's chunks
   uint32_t* head_counter;  // [kHeadRows] chunk tickets of the exit-head statistics

@@ -274,8 +274,8 @@ __global__ void __launch_bounds__(kSampleThreads) k_residual_weights(const Dims 
 // for the first RMSNorm (bf16 models).  One block per row.  Optionally sets the drafting switch handle to
 // the chosen exit-layer index.
 template <typename T>
-__global__ void k_embed(Dims D, Bufs B, const T* __restrict__ emb, RowSel sel,
-                        cudaGraphConditionalHandle sw) {
+__global__ void k_embed(Dims D, Bufs B, const T* __restrict__ emb, const T* __restrict__ gnorm,
+                        RowSel sel, cudaGraphConditionalHandle sw) {
   pdl_wait();
   pdl_launch_dependents();
   Ctl* c = B.ctl;
@@ -309,7 +309,16 @@ __global__ void k_embed(Dims D, Bufs B, const T* __restrict__ emb, RowSel sel,
     sp = warp_sum(sp);
     if (lane == 0) B.ss_part[(size_t)c * kMaxM + m] = sp;
   }
-  for (int i = threadIdx.x; i < D.d; i += blockDim.x) hr[i] = Elem<T>::to_f(row[i]);
+  for (int i = threadIdx.x; i < D.d; i += blockDim.x) {
+    const float v = Elem<T>::to_f(row[i]);
+    hr[i] = v;
+    if constexpr (sizeof(T) == 2) {  // as the first QKV product reads it
+      const float x = v * Elem<T>::to_f(gnorm[i]);
+      const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+      B.xs_h[(size_t)m * D.d + i] = hi;
+      B.xs_h[(size_t)(kMaxM + m) * D.d + i] = __float2bfloat16_rn(x - __bfloat162float(hi));
+    }
+  }
 }
 
 // Draft cap of the round: min(kmax, tokens still to emit - 1), the static
@@ -836,14 +845,15 @@ __global__ void k_kv_to_f32(Dims D, Bufs B, int layer, int kind, int head, int p
 
 // ---------------------------------------------------------------- launchers
 
-cudaError_t launch_embed(const Dims& D, const Bufs& B, int dtype, const void* embed, RowSel sel,
-                         bool big, cudaGraphConditionalHandle sw, cudaStream_t st) {
+cudaError_t launch_embed(const Dims& D, const Bufs& B, int dtype, const void* embed,
+                         const void* gnorm, RowSel sel, bool big, cudaGraphConditionalHandle sw, cudaStream_t st) {
   const int grid = big ? kMaxM : 1;
   if (dtype == SSD_DTYPE_BF16)
       return launch_ex(k_embed<__nv_bfloat16>, dim3(grid), dim3(256), 0, st, D, B,
-                     static_cast<const __nv_bfloat16*>(embed), sel, sw);
+                     static_cast<const __nv_bfloat16*>(embed),
+                     static_cast<const __nv_bfloat16*>(gnorm), sel, sw);
   return launch_ex(k_embed<float>, dim3(grid), dim3(256), 0, st, D, B,
-                   static_cast<const float*>(embed), sel, sw);
+                   static_cast<const float*>(embed), static_cast<const float*>(gnorm), sel, sw);
 }
 
 cudaError_t launch_round_begin(const Dims& D, const Bufs& B, cudaGraphConditionalHandle draft_if,

@@ -78,10 +78,18 @@ size_t layout(const ssd_model_cfg& c, char* base, Dims* D, Bufs* B, WideBufs* P)
   b.xq = cv.take<float>(sizeof(float) * kMaxM * d.qd);
   b.attn_part = cv.take<float>(sizeof(float) * kMaxM * d.Hq * (size_t)d.nsplit * d.hd);
   b.attn_ml = cv.take<float>(sizeof(float) * kMaxM * d.Hq * (size_t)d.nsplit * 2);
+  if (c.dtype == SSD_DTYPE_BF16) {
+    b.xs_h = cv.take<__nv_bfloat16>(4 * (size_t)kMaxM * d.d);
+    b.xs_o = cv.take<__nv_bfloat16>(4 * (size_t)kMaxM * d.qd);
+    b.xs_a = cv.take<__nv_bfloat16>(4 * (size_t)kMaxM * d.F);
+    b.xs_x = cv.take<__nv_bfloat16>(4 * (size_t)kMaxM * std::max({d.d, d.qd, d.F}));
+  }
   b.attn_counter = cv.take<uint32_t>(sizeof(uint32_t) * (size_t)d.Hkv * kMaxM);
   b.chain_bar = cv.take<uint32_t>(sizeof(uint32_t) * 2);
-  b.attn_out = cv.take<float>(sizeof(float) * kMaxM * d.qd);
-  b.act = cv.take<float>(sizeof(float) * kMaxM * d.F);
+  if (c.dtype == SSD_DTYPE_F32) {
+    b.attn_out = cv.take<float>(sizeof(float) * kMaxM * d.qd);
+    b.act = cv.take<float>(sizeof(float) * kMaxM * d.F);
+  }
   b.logits = cv.take<float>(sizeof(float) * kHeadRows * (size_t)d.V);
   b.draft_logits = base ? b.logits + kMaxM * (size_t)d.V : nullptr;
   b.row_sums = cv.take<float>(sizeof(float) * kHeadRows * kSampChunks);
@@ -247,24 +255,40 @@ const CUtensorMap* lm_map(const ssd_ctx* x) {
   return x->cfg.dtype == SSD_DTYPE_BF16 ? &x->wmaps[4 * (size_t)x->cfg.n_layers] : nullptr;
 }
 
+// Norm weights of the matrix behind layer l of a pass that ends at l_to.
+const void* norm_behind(const ssd_ctx* x, int l, int l_to) {
+  return l + 1 < l_to ? x->layers[l + 1].attn_norm : x->final_norm;
+}
+
+cudaError_t enqueue_part(ssd_ctx* x, int l, int part, int l_to, RowSel sel, int mrows,
+                         cudaStream_t st) {
+  return launch_layer_part(x->D, x->B, x->cfg.dtype, x->layers[l], tile_maps(x), l, part,
+                           norm_behind(x, l, l_to), sel, mrows, st);
+}
+
 // mrows: the most rows the launches will see (1: the single-row kernels).
 cudaError_t enqueue_layers(ssd_ctx* x, int l_from, int l_to, RowSel sel, int mrows,
                            cudaStream_t st) {
+  // bf16: the rows that a pass begins with past the first layer carry the norm
+  // weights of an exit head; those of its last layer get them, since an exit
+  // head follows every pass
+  if (x->cfg.dtype == SSD_DTYPE_BF16 && l_from > 0 && l_to > l_from)
+    GK(launch_resplit(x->D, x->B, x->layers[l_from].attn_norm, sel, mrows, st));
   if (x->cfg.dtype == SSD_DTYPE_BF16 && g_chain_enabled && l_to > l_from) {
     // QKV of the first layer, then per layer: attention, and O + gate/up +
     // down + the next layer's QKV as one persistent launch
-    GK(launch_layer_part(x->D, x->B, x->cfg.dtype, x->layers[l_from], tile_maps(x), l_from, 0, sel,
-                         mrows, st));
+    GK(enqueue_part(x, l_from, 0, l_to, sel, mrows, st));
     for (int l = l_from; l < l_to; ++l) {
-      GK(launch_layer_part(x->D, x->B, x->cfg.dtype, x->layers[l], tile_maps(x), l, 1, sel, mrows,
-                           st));
+      GK(enqueue_part(x, l, 1, l_to, sel, mrows, st));
       GK(launch_tile_chain(x->D, x->B, *tile_maps(x), x->layers[l],
-                           l + 1 < l_to ? &x->layers[l + 1] : nullptr, l, sel, mrows, st));
+                           l + 1 < l_to ? &x->layers[l + 1] : nullptr, x->final_norm, l, sel, mrows,
+                           st));
     }
     return cudaSuccess;
   }
   for (int l = l_from; l < l_to; ++l)
-    GK(launch_layer(x->D, x->B, x->cfg.dtype, x->layers[l], tile_maps(x), l, sel, mrows, st));
+    GK(launch_layer(x->D, x->B, x->cfg.dtype, x->layers[l], tile_maps(x), l,
+                    norm_behind(x, l, l_to), sel, mrows, st));
   return cudaSuccess;
 }
 
@@ -280,7 +304,7 @@ cudaError_t build_walk(ssd_ctx* x, Seq& s, const std::vector<int>& cands, int j,
   cudaGraphConditionalHandle next = 0;
   if (!last) GK(cudaGraphConditionalHandleCreate(&next, s.g, 0, 0));
   GK(s.begin());
-  if (j == 0) GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, rows(kRowsWalk), false, 0, x->cap));
+  if (j == 0) GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, x->layers[0].attn_norm, rows(kRowsWalk), false, 0, x->cap));
   GK(enqueue_layers(x, done, cands[j], rows(kRowsWalk), 1, x->cap));
   GK(enqueue_head(x, rows(kRowsWalk), 1, x->topk, x->cap));
   if (x->sampled) GK(launch_row_weights(x->D, x->B, rows(kRowsWalk), 1, 1, x->cap));
@@ -312,7 +336,7 @@ cudaError_t build_draft_phase(ssd_ctx* x, cudaGraph_t body) {
     cudaGraphConditionalHandle hs;
     GK(cudaGraphConditionalHandleCreate(&hs, wbody, 0, 0));
     GK(w.begin());
-    GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, rows(kRowsDraft), false, hs, x->cap));
+    GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, x->layers[0].attn_norm, rows(kRowsDraft), false, hs, x->cap));
     GK(w.end());
     std::vector<cudaGraph_t> cases(J);
     GK(w.cond(hs, cudaGraphCondTypeSwitch, (unsigned)J, cases.data()));
@@ -325,7 +349,7 @@ cudaError_t build_draft_phase(ssd_ctx* x, cudaGraph_t body) {
     GK(w.begin());
   } else {
     GK(w.begin());
-    GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, rows(kRowsDraft), false, 0, x->cap));
+    GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, x->layers[0].attn_norm, rows(kRowsDraft), false, 0, x->cap));
     GK(enqueue_layers(x, 0, cands[0], rows(kRowsDraft), 1, x->cap));
   }
   GK(enqueue_head(x, rows(kRowsDraft), 1, x->topk, x->cap));
@@ -351,7 +375,7 @@ cudaError_t build_round(ssd_ctx* x, cudaGraph_t g, cudaGraphConditionalHandle ge
     GK(build_draft_phase(x, body));
   }
   GK(s.begin());
-  GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, rows(kRowsVerify), spec, 0, x->cap));
+  GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, x->layers[0].attn_norm, rows(kRowsVerify), spec, 0, x->cap));
   const int mrows = spec ? std::min(x->kmax + 1, kMaxM) : 1;
   GK(enqueue_layers(x, 0, x->D.L, rows(kRowsVerify), mrows, x->cap));
   GK(enqueue_head(x, rows(kRowsVerify), mrows, x->topk, x->cap));
@@ -466,7 +490,7 @@ ssd_status run_prompt(ssd_ctx* x, int n, int* last_row) {
   for (int c0 = 0; c0 < n; c0 += kPrefillChunk) {
     const int M = std::min(kPrefillChunk, n - c0);
     const RowSel sel = rows_explicit(c0, M, x->B.pre_tok + c0);
-    CK(x, launch_embed(x->D, x->B, x->cfg.dtype, x->embed, sel, true, 0, x->stream));
+    CK(x, launch_embed(x->D, x->B, x->cfg.dtype, x->embed, x->layers[0].attn_norm, sel, true, 0, x->stream));
     CK(x, enqueue_layers(x, 0, x->D.L, sel, kPrefillChunk, x->stream));
     if (c0 + M > n - T || c0 + M == n) {
       CK(x, enqueue_head(x, sel, kPrefillChunk, x->topk, x->stream));
@@ -577,9 +601,9 @@ ssd_status ssd_init_model(const ssd_model_cfg* cfg, const ssd_weights* w, void* 
       for (int k = 0; k < 4; ++k) x->layers[l].tm[k] = m + k;
     }
     ok = ok && encode_weight_map(&x->wmaps[4 * (size_t)L], w->lm_head, cfg->vocab, d) &&
-         encode_input_maps(x->tmaps.h, x->B.h, d) &&
-         encode_input_maps(x->tmaps.attn_out, x->B.attn_out, qd) &&
-         encode_input_maps(x->tmaps.act, x->B.act, F) &&
+         encode_input_maps(x->tmaps.h, x->B.xs_h, d) &&
+         encode_input_maps(x->tmaps.attn_out, x->B.xs_o, qd) &&
+         encode_input_maps(x->tmaps.act, x->B.xs_a, F) &&
          encode_wide_maps(x->xmaps.xn, x->P.xn, d, x->P.cap) &&
          encode_wide_maps(x->xmaps.xo, x->P.xo, qd, x->P.cap) &&
          encode_wide_maps(x->xmaps.xa, x->P.xa, F, x->P.cap);
@@ -888,7 +912,7 @@ ssd_status ssd_forward_exit(ssd_ctx* x, const int32_t* ids, int32_t M, int32_t p
   if (x->async_pending) return fail(x, SSD_ERR_STATE, "generation in flight");
   CK(x, cudaMemcpyAsync(x->B.pre_tok, ids, sizeof(int32_t) * M, cudaMemcpyHostToDevice, x->stream));
   const RowSel sel = rows_explicit(pos0, M, x->B.pre_tok);
-  CK(x, launch_embed(x->D, x->B, x->cfg.dtype, x->embed, sel, true, 0, x->stream));
+  CK(x, launch_embed(x->D, x->B, x->cfg.dtype, x->embed, x->layers[0].attn_norm, sel, true, 0, x->stream));
   CK(x, enqueue_layers(x, 0, l_exit, sel, M, x->stream));
   CK(x, enqueue_head(x, sel, M, topk, x->stream));
   std::vector<RowStats> st(M);
@@ -1013,11 +1037,10 @@ ssd_status ssd_op_layer(ssd_ctx* x, int32_t kernel, int32_t layer, int32_t M, in
     CK(x, enqueue_head(x, sel, M, x->topk, st));
   else if (kernel == 6)
     CK(x, launch_tile_chain(x->D, x->B, *tile_maps(x), x->layers[layer],
-                            layer + 1 < x->cfg.n_layers ? &x->layers[layer + 1] : nullptr, layer,
-                            sel, M, st));
+                            layer + 1 < x->cfg.n_layers ? &x->layers[layer + 1] : nullptr,
+                            x->final_norm, layer, sel, M, st));
   else
-    CK(x, launch_layer_part(x->D, x->B, x->cfg.dtype, x->layers[layer], tile_maps(x), layer,
-                            kernel, sel, M, st));
+    CK(x, enqueue_part(x, layer, kernel, x->cfg.n_layers, sel, M, st));
   return SSD_OK;
 }
 

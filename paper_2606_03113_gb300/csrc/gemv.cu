@@ -485,18 +485,19 @@ cudaError_t launch_attention(const Dims& D, const Bufs& B, int dtype, int layer,
                              int mrows, cudaStream_t st);
 
 cudaError_t launch_layer_part(const Dims& D, const Bufs& B, int dtype, const LayerW& w,
-                              const TileMaps* tm, int layer, int part, RowSel sel, int mrows,
-                              cudaStream_t st) {
+                              const TileMaps* tm, int layer, int part, const void* next_norm,
+                              RowSel sel, int mrows, cudaStream_t st) {
   if (part == 1) return launch_attention(D, B, dtype, layer, sel, mrows, st);
   if (dtype != SSD_DTYPE_BF16) return launch_f32_part(D, B, w, layer, part, sel, mrows, st);
   if (!tm) return cudaErrorInvalidValue;
-  return launch_tile_part(D, B, *tm, w, layer, part, sel, mrows, st);
+  return launch_tile_part(D, B, *tm, w, layer, part, next_norm, sel, mrows, st);
 }
 
 cudaError_t launch_layer(const Dims& D, const Bufs& B, int dtype, const LayerW& w,
-                         const TileMaps* tm, int layer, RowSel sel, int mrows, cudaStream_t st) {
+                         const TileMaps* tm, int layer, const void* next_norm, RowSel sel,
+                         int mrows, cudaStream_t st) {
   for (int part = 0; part < 5; ++part) {  // qkv, attention, o, gate/up, down
-    cudaError_t e = launch_layer_part(D, B, dtype, w, tm, layer, part, sel, mrows, st);
+    cudaError_t e = launch_layer_part(D, B, dtype, w, tm, layer, part, next_norm, sel, mrows, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -508,7 +509,7 @@ cudaError_t launch_head(const Dims& D, const Bufs& B, int dtype, const void* lm_
   cudaError_t e;
   if (dtype == SSD_DTYPE_BF16) {
     if (!tm || !lm_map) return cudaErrorInvalidValue;
-    e = launch_tile_head(D, B, *tm, *lm_map, final_norm, sel, mrows, st);
+    e = launch_tile_head(D, B, *tm, *lm_map, sel, mrows, st);
   } else {
     e = launch_f32_head(D, B, lm_head, final_norm, sel, mrows, st);
   }

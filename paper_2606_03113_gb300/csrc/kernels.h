@@ -21,32 +21,35 @@ constexpr int kHeadParts = 256;  // chunks of a row, at most
 constexpr int kMaxBlocks = 512;
 inline int head_tiles(int V) { return (V + 15) / 16; }
 
-// Tensor maps of the engine's fp32 input buffers ([kMaxM][K] each), read by
-// the bf16 tensor-core kernels one 64-column slice per unit.
+// Tensor maps of the split input rows (high and low planes [2][kMaxM][K]), read
+// by the bf16 tensor-core kernels one 64-column box per unit.
 struct TileMaps {
   CUtensorMap h[3], attn_out[3], act[3];  // boxes of 8, 16, 24 rows
 };
 
 // Encodes the tensor map of a bf16 weight matrix [rows][cols] (64 x 64 boxes,
-// 128-byte swizzle) or of an fp32 input [rows][cols] (64 x kMaxM boxes).
+// 128-byte swizzle) or of split input rows.
 bool encode_weight_map(CUtensorMap* m, const void* W, int rows, int cols);
-bool encode_input_map(CUtensorMap* m, const float* x, int cols, int rows, int box_rows);
-bool encode_input_maps(CUtensorMap (&m)[3], const float* x, int cols);
+bool encode_input_maps(CUtensorMap (&m)[3], const void* xs, int cols);
+// h of the rows as a matrix with norm weights gnorm reads it, where the kernel
+// that wrote h did not know them.
+cudaError_t launch_resplit(const Dims& D, const Bufs& B, const void* gnorm, RowSel sel, int mrows,
+                           cudaStream_t st);
 cudaError_t prepare_tile_kernels();
 // Resident blocks per SM of the tensor-core kernels (0: cannot be resident).
 int tile_blocks_per_sm();
 // Floats of the tensor-core kernels' split-tile partials for `num_sms` blocks.
 size_t tile_part_floats(int num_sms);
 cudaError_t launch_tile_part(const Dims& D, const Bufs& B, const TileMaps& tm, const LayerW& w,
-                             int layer, int part, RowSel sel, int mrows, cudaStream_t st);
+                             int layer, int part, const void* next_norm, RowSel sel, int mrows,
+                             cudaStream_t st);
 // One launch of a layer's O projection, gate/up and down (and, with next, the
 // next layer's QKV) as the phases of one persistent kernel.
 cudaError_t launch_tile_chain(const Dims& D, const Bufs& B, const TileMaps& tm, const LayerW& w,
-                              const LayerW* next, int layer, RowSel sel, int mrows,
-                              cudaStream_t st);
+                              const LayerW* next, const void* final_norm, int layer, RowSel sel,
+                              int mrows, cudaStream_t st);
 cudaError_t launch_tile_head(const Dims& D, const Bufs& B, const TileMaps& tm,
-                             const CUtensorMap& lm, const void* final_norm, RowSel sel, int mrows,
-                             cudaStream_t st);
+                             const CUtensorMap& lm, RowSel sel, int mrows, cudaStream_t st);
 cudaError_t launch_tile_plain(const Dims& D, const Bufs& B, const CUtensorMap& wm, int rows,
                               int cols, const float* x, int M, float* y, cudaStream_t st);
 
@@ -84,14 +87,17 @@ cudaError_t launch_f32_head(const Dims& D, const Bufs& B, const void* lm, const 
 // single-row kernels, more the multi-row ones (bf16: the tensor-core instance
 // with 8, 16 or 24 token rows, the smallest that holds mrows).  big
 // (embedding, attention) is mrows > 1.
-cudaError_t launch_embed(const Dims& D, const Bufs& B, int dtype, const void* embed, RowSel sel,
-                         bool big, cudaGraphConditionalHandle set_lstar_switch, cudaStream_t st);
+// gnorm: norm weights of the first layer.
+cudaError_t launch_embed(const Dims& D, const Bufs& B, int dtype, const void* embed,
+                         const void* gnorm, RowSel sel, bool big, cudaGraphConditionalHandle set_lstar_switch, cudaStream_t st);
+// next_norm: norm weights of the matrix behind the layer.
 cudaError_t launch_layer(const Dims& D, const Bufs& B, int dtype, const LayerW& w,
-                         const TileMaps* tm, int layer, RowSel sel, int mrows, cudaStream_t st);
+                         const TileMaps* tm, int layer, const void* next_norm, RowSel sel,
+                         int mrows, cudaStream_t st);
 // One kernel of a layer (0 qkv, 1 attention + combine, 2 o, 3 gate/up, 4 down).
 cudaError_t launch_layer_part(const Dims& D, const Bufs& B, int dtype, const LayerW& w,
-                              const TileMaps* tm, int layer, int part, RowSel sel, int mrows,
-                              cudaStream_t st);
+                              const TileMaps* tm, int layer, int part, const void* next_norm,
+                              RowSel sel, int mrows, cudaStream_t st);
 cudaError_t launch_head(const Dims& D, const Bufs& B, int dtype, const void* lm_head,
                         const CUtensorMap* lm_map, const TileMaps* tm, const void* final_norm,
                         int topk, RowSel sel, int mrows, cudaStream_t st);

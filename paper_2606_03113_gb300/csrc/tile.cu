@@ -10,15 +10,17 @@
 //    64 x 64 boxes with the 128-byte swizzle); the units, in (tile, K) order,
 //    are split evenly over a persistent grid of one block per SM
 //    ("stream-K"), so every SM streams the same bytes whatever the shape;
-//  - warp roles (320 threads): a TMA warp fills a 5-deep ring with the
-//    unit's weight boxes and its slice of the fp32 input rows (plus the
-//    RMSNorm weights); eight worker warps turn the slice into bf16 high and
-//    low operand tiles (x = hi + lo to ~16 significant bits); one MMA warp
-//    issues tcgen05.mma (M = 128 rows per half, N = 16 or 32 token columns,
-//    K = 16) for both halves and both parts into a double-buffered TMEM
-//    accumulator, and releases ring slots and operand tiles with
-//    tcgen05.commit;
-//  - at the end of a tile the workers read the accumulator from TMEM (each
+//  - the input rows come as bf16 high and low parts (x = hi + lo to ~16
+//    significant bits), written by the kernel that produced them and already
+//    multiplied by the RMSNorm weights of the product that reads them: one TMA
+//    box is a unit's operand tile.  (The workers used to split fp32 slices in
+//    shared memory, one more hand-over per unit: @PRE@)
+//  - warp roles (320 threads): a TMA warp fills a 5- or 6-deep ring with the
+//    unit's weight boxes and its input box; one MMA warp issues tcgen05.mma (M
+//    = 128 rows per half, N = 16, 32 or 48 token columns, K = 16) for both
+//    halves and both parts into a double-buffered TMEM accumulator, and
+//    releases ring slots with tcgen05.commit;
+//  - at the end of a tile eight worker warps read the accumulator from TMEM (each
 //    thread one row of each half: the rows a fused epilogue pairs, i and
 //    i + 128) and run the epilogue; a tile split between blocks is finished
 //    by its last contributor, adding the partial sums in block order;
@@ -57,27 +59,21 @@ constexpr int kMaxBlocksDev = kMaxBlocks;
 enum TMap : int { kTMapLinear = 0, kTMapQKV = 1, kTMapGateUp = 2 };
 enum TKind : int { kKPlain = 0, kKQKV = 1, kKGateUp = 2, kKResid = 3, kKHead = 4 };
 
-constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
-
 // Shared-memory layout of the instance with TP token rows (8, 16 or 24): the
 // MMA's N is 2 TP (bf16 high parts of the tokens in rows 0..TP-1, low parts
-// in rows TP..2TP-1).  Every ring slot holds a unit's weights, its operand
-// tile and its input slice, all released by the one commit of the unit's
-// MMAs.
+// in rows TP..2TP-1).  Every ring slot holds a unit's weights and its operand
+// tile, both released by the one commit of the unit's MMAs.
 template <int TP>
 struct TL {
   static constexpr int N = 2 * TP;
-  static constexpr int NS = TP == 24 ? 4 : (TP == 8 ? 6 : 5);  // ring depth
-  static constexpr int XB = TP * kKC * 4;                   // input box: TP rows x 64 fp32
-  static constexpr int XS = (int)align_up(XB + kKC * 2, 128);  // + RMSNorm weight slice
+  static constexpr int NS = TP == 24 ? 5 : 6;               // ring depth
   static constexpr int BB = N * 128;                        // operand tile (multiple of 1024)
   static constexpr uint32_t kCols = 4 * N <= 64 ? 64 : (4 * N <= 128 ? 128 : 256);
   static constexpr size_t ring = 0;
   static constexpr size_t bt = ring + (size_t)NS * kWBytes;
-  static constexpr size_t xs = bt + (size_t)NS * BB;
-  static constexpr size_t bars = align_up(xs + (size_t)NS * XS, 16);
-  // wfull[NS], xfull[NS], empty[NS], bfull[NS], accfull[2], accempty[2], drain
-  static constexpr int kNBars = 4 * NS + 5;
+  static constexpr size_t bars = bt + (size_t)NS * BB;
+  // wfull[NS], xfull[NS], empty[NS], accfull[2], accempty[2], drain
+  static constexpr int kNBars = 3 * NS + 5;
   static constexpr size_t tslot = bars + 8 * (size_t)kNBars;
   static constexpr size_t flag = tslot + 8;
   static constexpr size_t rs = flag + 8;
@@ -85,7 +81,7 @@ struct TL {
   static constexpr size_t used = red + 4 * (size_t)kWorkers * kLT;
   static constexpr size_t total = used + 1024;  // the base is aligned up to 1024 in the kernel
   static_assert(total <= 227 * 1024, "shared memory budget");
-  static_assert(BB % 1024 == 0 && XS % 128 == 0, "operand / slice alignment");
+  static_assert(BB % 1024 == 0, "operand alignment");
 };
 
 struct TGeom {
@@ -101,7 +97,7 @@ struct TArgs {
   TGeom g;
   Dims D;
   Bufs B;
-  const __nv_bfloat16* gnorm;  // RMSNorm weights of the input, or null
+  const __nv_bfloat16* gout;   // residual: norm weights of the matrix that reads the rows next
   int ss_in;                   // sum-of-squares buffer of the input scale (-1: none)
   RowSel sel;
   int layer;                   // QKV: KV-cache layer
@@ -148,23 +144,12 @@ __device__ inline int box_row(const TGeom& g, int tile, int b) {
   return tile * 256 + 64 * b;
 }
 
-__device__ __forceinline__ uint32_t swz(int m, int j) {
-  return (uint32_t)((m >> 3) * 1024 + (m & 7) * 128 + ((j ^ (m & 7)) << 4));
+// x as bf16 high and low parts into the planes of a split row buffer.
+__device__ __forceinline__ void put_split(__nv_bfloat16* p, size_t plane, float x) {
+  const __nv_bfloat16 h = __float2bfloat16_rn(x);
+  p[0] = h;
+  p[plane] = __float2bfloat16_rn(x - __bfloat162float(h));
 }
-
-__device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 a, __nv_bfloat16 b) {
-  return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
-}
-
-struct Ring {
-  uint64_t* full;
-  uint64_t* empty;
-  uint64_t* bfull;
-  uint64_t* bempty;
-  uint64_t* accfull;
-  uint64_t* accempty;
-  uint64_t* drain;
-};
 
 __device__ __forceinline__ void flag_timeout(const Bufs& B) {
   atomicOr(&B.ctl->err, (int)kErrTimeout);
@@ -175,7 +160,7 @@ __device__ __forceinline__ void flag_timeout(const Bufs& B) {
 // Adds the values of one (row pair, token) to the outputs.
 template <int KIND>
 __device__ __forceinline__ void t_pair(const TArgs& a, int tile, int s, int t, int pos0, float rs,
-                                       float v0, float v1, float& ss) {
+                                       float v0, float v1) {
   const Dims& D = a.D;
   if constexpr (KIND == kKPlain) {
     const int r0 = trow(a.g, tile, s), r1 = trow(a.g, tile, s + 128);
@@ -221,38 +206,29 @@ __device__ __forceinline__ void t_pair(const TArgs& a, int tile, int s, int t, i
     const int j = trow(a.g, tile, s);
     if (j < 0) return;
     const float gt = v0 * rs, up = v1 * rs;
-    a.B.act[(size_t)t * D.F + j] = gt / (1.0f + expf(-gt)) * up;
-  } else if constexpr (KIND == kKResid) {
-    // h[t][row] += y, and the sum of squares the next RMSNorm needs
-    const int r0 = trow(a.g, tile, s), r1 = trow(a.g, tile, s + 128);
-    float* hm = a.B.h + (size_t)t * D.d;
-    if (r0 >= 0) {
-      const float h = __ldcg(hm + r0) + v0;  // L2: rows a previous phase wrote
-      hm[r0] = h;
-      ss = fmaf(h, h, ss);
-    }
-    if (r1 >= 0) {
-      const float h = __ldcg(hm + r1) + v1;
-      hm[r1] = h;
-      ss = fmaf(h, h, ss);
-    }
+    put_split(a.B.xs_a + (size_t)t * D.F + j, (size_t)kMaxM * D.F,
+              gt / (1.0f + expf(-gt)) * up);
   }
 }
 
-// Residual add with the rows' previous values already loaded (split-tile
-// fix-ups load them together with the contributors' partial sums).
-__device__ __forceinline__ void t_resid_pre(const TArgs& a, int tile, int s, int t, float v0,
-                                            float v1, float h0, float h1, float& ss) {
-  const int r0 = trow(a.g, tile, s), r1 = trow(a.g, tile, s + 128);
+// Residual add of one (row pair, token): h[t][row] += y, the row as the next
+// matrix reads it, and the sum of squares its RMSNorm needs.  h0, h1: the rows'
+// previous values; g0, g1: the next norm's weights.
+__device__ __forceinline__ void t_resid(const TArgs& a, int r0, int r1, int t, float v0, float v1,
+                                        float h0, float h1, float g0, float g1, float& ss) {
   float* hm = a.B.h + (size_t)t * a.D.d;
+  __nv_bfloat16* xs = a.B.xs_h + (size_t)t * a.D.d;
+  const size_t plane = (size_t)kMaxM * a.D.d;
   if (r0 >= 0) {
     const float h = h0 + v0;
     hm[r0] = h;
+    put_split(xs + r0, plane, h * g0);
     ss = fmaf(h, h, ss);
   }
   if (r1 >= 0) {
     const float h = h1 + v1;
     hm[r1] = h;
+    put_split(xs + r1, plane, h * g1);
     ss = fmaf(h, h, ss);
   }
 }
@@ -278,7 +254,7 @@ template <int TP>
 struct Blk {
   using S = TL<TP>;
   unsigned char* smem;
-  uint64_t *full, *xfull, *empty, *bfull, *accfull, *accempty, *drain;
+  uint64_t *full, *xfull, *empty, *accfull, *accempty, *drain;
   uint32_t* tslot;
   int* sflag;
   float *srs, *red;
@@ -287,10 +263,9 @@ struct Blk {
     smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(raw) + 1023) &
                                             ~static_cast<uintptr_t>(1023));
     full = reinterpret_cast<uint64_t*>(smem + S::bars);  // weights landed
-    xfull = full + S::NS;                                // input slice landed
+    xfull = full + S::NS;                                // operand tile landed
     empty = xfull + S::NS;                               // slot released by the MMAs
-    bfull = empty + S::NS;                               // operand tile written
-    accfull = bfull + S::NS;
+    accfull = empty + S::NS;
     accempty = accfull + 2;
     drain = accempty + 2;
     tslot = reinterpret_cast<uint32_t*>(smem + S::tslot);
@@ -305,8 +280,7 @@ struct Blk {
       for (int i = 0; i < S::NS; ++i) {
         mbar_init(&full[i], 1);
         mbar_init(&xfull[i], 1);
-        mbar_init(&empty[i], 1);         // MMA commit
-        mbar_init(&bfull[i], kWorkers);  // operand tile written
+        mbar_init(&empty[i], 1);  // MMA commit
       }
       for (int i = 0; i < 2; ++i) {
         mbar_init(&accfull[i], 1);
@@ -320,14 +294,6 @@ struct Blk {
     __syncthreads();
     tc_fence_after();
     return *tslot;
-  }
-
-  // workers: zeroed operand tiles (rows past M stay zero)
-  __device__ void clear_operands(int tid) {
-    uint4* z = reinterpret_cast<uint4*>(smem + S::bt);
-    for (int i = tid; i < S::NS * S::BB / 16; i += kWThreads) z[i] = make_uint4(0, 0, 0, 0);
-    fence_proxy_async_smem();
-    named_sync(1, kWThreads);
   }
 };
 
@@ -353,7 +319,7 @@ __device__ bool mma_units(const Blk<TP>& k, const TGeom& g, int u_begin, int n, 
       ++tc;
       if (!mbar_wait(&k.accempty[tc & 1], ((uint32_t)(tc >> 1) & 1u) ^ 1u)) return false;
     }
-    if (!mbar_wait(&k.full[slot], ph) || !mbar_wait(&k.bfull[slot], ph)) return false;
+    if (!mbar_wait(&k.full[slot], ph) || !mbar_wait(&k.xfull[slot], ph)) return false;
     tc_fence_after();
     const uint32_t abase = smem_u32(k.smem + S::ring + (size_t)slot * kWBytes);
     const uint32_t bbase = smem_u32(k.smem + S::bt + (size_t)slot * S::BB);
@@ -370,14 +336,13 @@ __device__ bool mma_units(const Blk<TP>& k, const TGeom& g, int u_begin, int n, 
   return true;
 }
 
-// Workers (eight warps) for the block's units of one matrix: operand tiles
-// from the input slices, then the fused epilogue of every tile.  The RMSNorm
-// scale of the input rows is read first (from the sum-of-squares parts).
-template <int TP, int KIND, bool NORM>
+// Workers (eight warps) for the block's units of one matrix: the fused epilogue
+// of every tile.  The RMSNorm scale of the input rows is read first (from the
+// sum-of-squares parts).
+template <int TP, int KIND>
 __device__ void worker_units(const TArgs& a, const Blk<TP>& k, uint32_t tmem,
-                             int u_begin, int n, int gi0, int& tc, bool& ok, int pos0, int M) {
-  using S = TL<TP>;
-  constexpr int NS = S::NS, N = S::N;
+                             int u_begin, int n, int& tc, bool& ok, int pos0, int M) {
+  constexpr int N = TL<TP>::N;
   constexpr int LTN = TP / 2;                 // tokens per parity group read back
   constexpr int LTR = LTN < kLT ? LTN : kLT;  // ... of which can be rows (t < kMaxM)
   const TGeom& g = a.g;
@@ -428,6 +393,15 @@ __device__ void worker_units(const TArgs& a, const Blk<TP>& k, uint32_t tmem,
   // per-tile epilogue: TMEM -> registers (high + low parts) -> fused epilogue
   auto epilogue = [&](int tile, int tcv) {
     const int buf = tcv & 1;
+    // residual: the thread's rows and the next norm's weights there
+    int rr0 = -1, rr1 = -1;
+    float gn0 = 0.f, gn1 = 0.f;
+    if constexpr (KIND == kKResid) {
+      rr0 = trow(g, tile, srow);
+      rr1 = trow(g, tile, srow + 128);
+      if (rr0 >= 0) gn0 = __bfloat162float(a.gout[rr0]);
+      if (rr1 >= 0) gn1 = __bfloat162float(a.gout[rr1]);
+    }
     if (ok) {
       const bool w = __all_sync(0xffffffffu, mbar_wait(&k.accfull[buf], (uint32_t)(tcv >> 1) & 1u));
       if (!w) {
@@ -468,7 +442,11 @@ __device__ void worker_units(const TArgs& a, const Blk<TP>& k, uint32_t tmem,
         if (t >= M) break;
         const float v0 = grp ? v[0][2 * lt + 1] : v[0][2 * lt];
         const float v1 = grp ? v[1][2 * lt + 1] : v[1][2 * lt];
-        t_pair<KIND>(a, tile, srow, t, pos0, rs_t[lt], v0, v1, ssv[lt]);
+        if constexpr (KIND == kKResid)
+          t_resid(a, rr0, rr1, t, v0, v1, rr0 >= 0 ? __ldcg(a.B.h + (size_t)t * a.D.d + rr0) : 0.f,
+                  rr1 >= 0 ? __ldcg(a.B.h + (size_t)t * a.D.d + rr1) : 0.f, gn0, gn1, ssv[lt]);
+        else
+          t_pair<KIND>(a, tile, srow, t, pos0, rs_t[lt], v0, v1);
       }
       if constexpr (KIND == kKResid) tile_ss(ssv, tile);
       return;
@@ -497,13 +475,12 @@ __device__ void worker_units(const TArgs& a, const Blk<TP>& k, uint32_t tmem,
     // phase or kernel), loaded while the contributors are counted in
     float hp0[LTN], hp1[LTN];
     if constexpr (KIND == kKResid) {
-      const int r0 = trow(g, tile, srow), r1 = trow(g, tile, srow + 128);
 #pragma unroll
       for (int lt = 0; lt < LTN; ++lt) {
         const int t = 2 * lt + grp;
         const float* hm = a.B.h + (size_t)(t < M ? t : 0) * a.D.d;
-        hp0[lt] = (t < M && r0 >= 0) ? __ldcg(hm + r0) : 0.f;
-        hp1[lt] = (t < M && r1 >= 0) ? __ldcg(hm + r1) : 0.f;
+        hp0[lt] = (t < M && rr0 >= 0) ? __ldcg(hm + rr0) : 0.f;
+        hp1[lt] = (t < M && rr1 >= 0) ? __ldcg(hm + rr1) : 0.f;
       }
     }
     if (tid == 0) {
@@ -593,74 +570,19 @@ __device__ void worker_units(const TArgs& a, const Blk<TP>& k, uint32_t tmem,
       const int t = 2 * lt + grp;
       if (t >= M) break;
       if constexpr (KIND == kKResid)
-        t_resid_pre(a, tile, srow, t, u0[lt], u1[lt], hp0[lt], hp1[lt], ss_sp[lt]);
+        t_resid(a, rr0, rr1, t, u0[lt], u1[lt], hp0[lt], hp1[lt], gn0, gn1, ss_sp[lt]);
       else
-        t_pair<KIND>(a, tile, srow, t, pos0, rs_t[lt], u0[lt], u1[lt], ss_sp[lt]);
+        t_pair<KIND>(a, tile, srow, t, pos0, rs_t[lt], u0[lt], u1[lt]);
     }
     // the split tile's sums of squares are the tile's part
     if constexpr (KIND == kKResid) tile_ss(ss_sp, tile);
   };
 
-  int prev_tile = -1;
-  for (int i = 0; i < n; ++i) {
-    const int gi = gi0 + i;
-    const int u = u_begin + i;
-    const int slot = gi % NS;
-    const int tile = u / g.nks, kc = u - tile * g.nks;
-    if (i == 0 || kc == 0) ++tc;
-    // operand tile of unit i, built while its weights are still in flight:
-    // the slot's previous use was released before its copies were issued,
-    // so only the input slice's arrival is waited for
-    if (ok) {
-      const bool w = __all_sync(0xffffffffu, mbar_wait(&k.xfull[slot], (uint32_t)(gi / NS) & 1u));
-      if (!w) {
-        if (lane == 0) flag_timeout(a.B);
-        ok = false;
-      }
-    }
-    if (ok) {
-      const unsigned char* xs = k.smem + S::xs + (size_t)slot * S::XS;
-      unsigned char* bt = k.smem + S::bt + (size_t)slot * S::BB;
-      const int kvalid = g.K - kc * kKC;
-      for (int task = tid; task < M * 8; task += kWThreads) {
-        const int m = task >> 3, j = task & 7;
-        const float4 x0 = *reinterpret_cast<const float4*>(xs + m * (kKC * 4) + j * 32);
-        const float4 x1 = *reinterpret_cast<const float4*>(xs + m * (kKC * 4) + j * 32 + 16);
-        float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-        if (NORM) {
-          const uint4 gq = *reinterpret_cast<const uint4*>(xs + S::XB + j * 16);
-          float gv[8];
-          Elem<__nv_bfloat16>::unpack(gq, gv);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) xv[e] *= gv[e];
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          if (j * 8 + e >= kvalid) xv[e] = 0.f;
-        uint32_t hi[4], lo[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const __nv_bfloat16 h0 = __float2bfloat16_rn(xv[2 * e]);
-          const __nv_bfloat16 h1 = __float2bfloat16_rn(xv[2 * e + 1]);
-          hi[e] = pack_bf16(h0, h1);
-          lo[e] = pack_bf16(__float2bfloat16_rn(xv[2 * e] - __bfloat162float(h0)),
-                            __float2bfloat16_rn(xv[2 * e + 1] - __bfloat162float(h1)));
-        }
-        *reinterpret_cast<uint4*>(bt + swz(m, j)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *reinterpret_cast<uint4*>(bt + swz(TP + m, j)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-      }
-      fence_proxy_async_smem();
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&k.bfull[slot]);
-    // epilogue of the tile the previous unit completed
-    if (i > 0 && kc == 0) epilogue(prev_tile, tc - 1);
-    prev_tile = tile;
-  }
-  if (n > 0) epilogue(prev_tile, tc);
+  const int last_tile = n > 0 ? (u_end - 1) / g.nks : first_tile - 1;
+  for (int tile = first_tile; tile <= last_tile; ++tile) epilogue(tile, ++tc);
 }
 
-template <int TP, int KIND, bool NORM>
+template <int TP, int KIND>
 __global__ void __launch_bounds__(kTThreads, 1)
     k_tile(const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap,
            const TArgs a) {
@@ -670,7 +592,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
   Blk<TP> k(smem_raw);
   unsigned char* smem = k.smem;
   const TGeom& g = a.g;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int u_begin = t_start(g, blockIdx.x), u_end = t_start(g, blockIdx.x + 1);
   const int n = u_end - u_begin;
   const uint32_t tmem = k.setup(warp, kMmaWarp);
@@ -699,18 +621,15 @@ __global__ void __launch_bounds__(kTThreads, 1)
       bool ok = true;
       for (int i = 0; i < npre && ok; ++i) ok = issue_w(i);
       pdl_wait();
-      const int K = g.K;
+      // inputs written by the previous kernel's generic stores, read by TMA
+      asm volatile("fence.proxy.async.global;" ::: "memory");
       for (int i = 0; i < n && ok; ++i) {
         if (i >= npre) ok = issue_w(i);
         if (!ok) break;
         const int slot = i % NS;
         const int kc = (u_begin + i) % g.nks;
-        unsigned char* xdst = smem + S::xs + (size_t)slot * S::XS;
-        const int cols = min(kKC, K - kc * kKC);
-        const uint32_t gbytes = NORM ? (uint32_t)cols * 2u : 0u;
-        mbar_arrive_expect_tx(&k.xfull[slot], (uint32_t)S::XB + gbytes);
-        tma_load_2d(xdst, &xmap, kc * kKC, 0, &k.xfull[slot], pol);
-        if (NORM) bulk_g2s(xdst + S::XB, a.gnorm + (size_t)kc * kKC, gbytes, &k.xfull[slot], pol);
+        mbar_arrive_expect_tx(&k.xfull[slot], (uint32_t)S::BB);
+        tma_load_3d(smem + S::bt + (size_t)slot * S::BB, &xmap, kc * kKC, 0, 0, &k.xfull[slot]);
       }
       if (!ok) flag_timeout(a.B);
       // every copy has landed before the block exits
@@ -729,15 +648,14 @@ __global__ void __launch_bounds__(kTThreads, 1)
       if (!mbar_wait(k.drain, 0)) flag_timeout(a.B);
     }
   } else {
-    // ---------------- workers: operand tiles and epilogues
+    // ---------------- workers: epilogues
     pdl_wait();
     int pos0, M;
     resolve_rows(a.B.ctl, a.sel, pos0, M);
     if (M > TP) M = TP;  // the launcher picks TP >= M
-    k.clear_operands(tid);
     int tc = -1;
     bool ok = true;
-    worker_units<TP, KIND, NORM>(a, k, tmem, u_begin, n, 0, tc, ok, pos0, M);
+    worker_units<TP, KIND>(a, k, tmem, u_begin, n, tc, ok, pos0, M);
   }
 
   // TMEM is released once every MMA has completed and every read is done
@@ -821,7 +739,6 @@ __global__ void __launch_bounds__(kCThreads, 1)
   } else if (warp == kXWarp) {
     // ---------------- input slices: phase p after every block finished p - 1
     if (lane == 0) {
-      const uint64_t pol = evict_first_policy();
       for (int p = 0; p < NPH; ++p) tma_prefetch_desc(&maps.x[p]);
       pdl_wait();
       bool ok = true;
@@ -829,13 +746,11 @@ __global__ void __launch_bounds__(kCThreads, 1)
       for (int p = 0; p < NPH; ++p) {
         const TArgs& a = ca.ph[p];
         const TGeom& g = a.g;
-        if (p > 0) {
-          if (!counter_wait(ca.bar, (uint32_t)(p * P))) ok = false;
-          // inputs written by other blocks' generic stores, read by TMA
-          asm volatile("fence.proxy.async.global;" ::: "memory");
-        }
+        if (p > 0 && !counter_wait(ca.bar, (uint32_t)(p * P))) ok = false;
+        // inputs written by generic stores (other blocks', the previous
+        // kernel's), read by TMA
+        asm volatile("fence.proxy.async.global;" ::: "memory");
         const int u_begin = t_start(g, blockIdx.x), n = t_start(g, blockIdx.x + 1) - u_begin;
-        const bool norm = a.gnorm != nullptr;
         for (int i = 0; i < n && ok; ++i, ++gi) {
           const int slot = gi % NS;
           if (!mbar_wait(&k.empty[slot], ((uint32_t)(gi / NS) & 1u) ^ 1u)) {
@@ -843,12 +758,9 @@ __global__ void __launch_bounds__(kCThreads, 1)
             break;
           }
           const int kc = (u_begin + i) % g.nks;
-          unsigned char* xdst = smem + S::xs + (size_t)slot * S::XS;
-          const int cols = min(kKC, g.K - kc * kKC);
-          const uint32_t gbytes = norm ? (uint32_t)cols * 2u : 0u;
-          mbar_arrive_expect_tx(&k.xfull[slot], (uint32_t)S::XB + gbytes);
-          tma_load_2d(xdst, &maps.x[p], kc * kKC, 0, &k.xfull[slot], pol);
-          if (norm) bulk_g2s(xdst + S::XB, a.gnorm + (size_t)kc * kKC, gbytes, &k.xfull[slot], pol);
+          mbar_arrive_expect_tx(&k.xfull[slot], (uint32_t)S::BB);
+          tma_load_3d(smem + S::bt + (size_t)slot * S::BB, &maps.x[p], kc * kKC, 0, 0,
+                      &k.xfull[slot]);
         }
         if (!ok) break;
       }
@@ -876,12 +788,10 @@ __global__ void __launch_bounds__(kCThreads, 1)
     int pos0, M;
     resolve_rows(ca.ph[0].B.ctl, ca.ph[0].sel, pos0, M);
     if (M > TP) M = TP;
-    k.clear_operands(tid);
-    int tc = -1, gi = 0;
+    int tc = -1;
     bool ok = true;
-    auto phase = [&](auto kind, auto norm, int p) {
+    auto phase = [&](auto kind, int p) {
       constexpr int KIND = decltype(kind)::value;
-      constexpr bool NORM = decltype(norm)::value;
       const TArgs& a = ca.ph[p];
       if (p > 0) {
         // every block finished phase p - 1: one thread acquires, the CTA
@@ -893,16 +803,15 @@ __global__ void __launch_bounds__(kCThreads, 1)
         named_sync(1, kWThreads);
       }
       const int u_begin = t_start(a.g, blockIdx.x), n = t_start(a.g, blockIdx.x + 1) - u_begin;
-      worker_units<TP, KIND, NORM>(a, k, tmem, u_begin, n, gi, tc, ok, pos0, M);
-      gi += n;
+      worker_units<TP, KIND>(a, k, tmem, u_begin, n, tc, ok, pos0, M);
       // this block's outputs of phase p are written: arrive
       named_sync(1, kWThreads);
       if (tid == 0) red_release_gpu(ca.bar, 1u);
     };
-    phase(std::integral_constant<int, kKResid>{}, std::false_type{}, 0);
-    phase(std::integral_constant<int, kKGateUp>{}, std::true_type{}, 1);
-    phase(std::integral_constant<int, kKResid>{}, std::false_type{}, 2);
-    if constexpr (QKV4) phase(std::integral_constant<int, kKQKV>{}, std::true_type{}, 3);
+    phase(std::integral_constant<int, kKResid>{}, 0);
+    phase(std::integral_constant<int, kKGateUp>{}, 1);
+    phase(std::integral_constant<int, kKResid>{}, 2);
+    if constexpr (QKV4) phase(std::integral_constant<int, kKQKV>{}, 3);
     // the last block out resets the counters for the next launch (every
     // block has passed all of its waits by now)
     if (tid == 0 && atomicAdd(ca.bar + 1, 1u) == (uint32_t)(P - 1)) {
@@ -952,32 +861,32 @@ TGeom make_tgeom(const Dims& D, int N, int K, int map) {
   return g;
 }
 
-template <int TP, int KIND, bool NORM>
+template <int TP, int KIND>
 cudaError_t tile_launch(const CUtensorMap& wm, const CUtensorMap& xm, const TArgs& a,
                         cudaStream_t st) {
   // unit indices are 32-bit: T * blocks must stay below 2^31
   if (a.g.T < 1 || a.g.T > (1 << 22) || a.g.P < 1 || a.g.P > kMaxBlocksDev)
     return cudaErrorInvalidValue;
-  return launch_ex(k_tile<TP, KIND, NORM>, dim3(a.g.P), dim3(kTThreads),
+  return launch_ex(k_tile<TP, KIND>, dim3(a.g.P), dim3(kTThreads),
                    TL<TP>::total, st, wm, xm, a);
 }
 
 // Token rows of the instance for launches of up to mrows rows.
 int tp_index(int mrows) { return mrows <= 8 ? 0 : (mrows <= 16 ? 1 : 2); }
 
-template <int KIND, bool NORM>
+template <int KIND>
 cudaError_t tile_dispatch(const CUtensorMap& wm, const CUtensorMap* xm3, const TArgs& a, int mrows,
                           cudaStream_t st) {
   switch (tp_index(mrows)) {
-    case 0: return tile_launch<8, KIND, NORM>(wm, xm3[0], a, st);
-    case 1: return tile_launch<16, KIND, NORM>(wm, xm3[1], a, st);
-    default: return tile_launch<24, KIND, NORM>(wm, xm3[2], a, st);
+    case 0: return tile_launch<8, KIND>(wm, xm3[0], a, st);
+    case 1: return tile_launch<16, KIND>(wm, xm3[1], a, st);
+    default: return tile_launch<24, KIND>(wm, xm3[2], a, st);
   }
 }
 
-template <int TP, int KIND, bool NORM>
+template <int TP, int KIND>
 cudaError_t prep_one() {
-  return cudaFuncSetAttribute(k_tile<TP, KIND, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(k_tile<TP, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)TL<TP>::total);
 }
 
@@ -996,11 +905,11 @@ cudaError_t prep_chain() {
                               (int)TL<TP>::total);
 }
 
-template <int KIND, bool NORM>
+template <int KIND>
 cudaError_t prep_kind() {
-  cudaError_t e = prep_one<8, KIND, NORM>();
-  if (e == cudaSuccess) e = prep_one<16, KIND, NORM>();
-  return e != cudaSuccess ? e : prep_one<24, KIND, NORM>();
+  cudaError_t e = prep_one<8, KIND>();
+  if (e == cudaSuccess) e = prep_one<16, KIND>();
+  return e != cudaSuccess ? e : prep_one<24, KIND>();
 }
 
 }  // namespace
@@ -1015,19 +924,6 @@ bool encode_weight_map(CUtensorMap* m, const void* W, int rows, int cols) {
                   es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-bool encode_input_map(CUtensorMap* m, const float* x, int cols, int rows, int box_rows) {
-  if (!get_encoder() || !x || ((uintptr_t)x & 15u) || ((size_t)cols * 4) % 16 || rows < 1 ||
-      rows > kMaxM || box_rows < 1 || box_rows > 256)
-    return false;
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)cols * 4};
-  cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
-  cuuint32_t es[2] = {1, 1};
-  return g_encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(x), dims, strides, box,
-                  es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 bool encode_split_map(CUtensorMap* m, const void* x, int cols, int cap, int box_rows) {
@@ -1046,14 +942,14 @@ bool encode_split_map(CUtensorMap* m, const void* x, int cols, int cap, int box_
 
 cudaError_t prepare_tile_kernels() {
   cudaError_t e;
-  if ((e = prep_kind<kKPlain, false>()) != cudaSuccess) return e;
-  if ((e = prep_kind<kKQKV, true>()) != cudaSuccess) return e;
-  if ((e = prep_kind<kKGateUp, true>()) != cudaSuccess) return e;
-  if ((e = prep_kind<kKResid, false>()) != cudaSuccess) return e;
+  if ((e = prep_kind<kKPlain>()) != cudaSuccess) return e;
+  if ((e = prep_kind<kKQKV>()) != cudaSuccess) return e;
+  if ((e = prep_kind<kKGateUp>()) != cudaSuccess) return e;
+  if ((e = prep_kind<kKResid>()) != cudaSuccess) return e;
   if ((e = prep_chain<8>()) != cudaSuccess) return e;
   if ((e = prep_chain<16>()) != cudaSuccess) return e;
   if ((e = prep_chain<24>()) != cudaSuccess) return e;
-  return prep_kind<kKHead, true>();
+  return prep_kind<kKHead>();
 }
 
 // Blocks of the tensor-core kernels that can be resident on one SM at once
@@ -1070,20 +966,49 @@ int tile_blocks_per_sm() {
   occ((const void*)k_chain<8, true>, kCThreads, TL<8>::total);
   occ((const void*)k_chain<16, true>, kCThreads, TL<16>::total);
   occ((const void*)k_chain<24, true>, kCThreads, TL<24>::total);
-  occ((const void*)k_tile<8, kKHead, true>, kTThreads, TL<8>::total);
-  occ((const void*)k_tile<24, kKQKV, true>, kTThreads, TL<24>::total);
+  occ((const void*)k_tile<8, kKHead>, kTThreads, TL<8>::total);
+  occ((const void*)k_tile<24, kKQKV>, kTThreads, TL<24>::total);
   return lo;
 }
 
 size_t tile_part_floats(int num_sms) { return (size_t)num_sms * 2 * 2 * kMaxM * 128; }
 
-bool encode_input_maps(CUtensorMap (&m)[3], const float* x, int cols) {
-  return encode_input_map(&m[0], x, cols, kMaxM, 8) && encode_input_map(&m[1], x, cols, kMaxM, 16) &&
-         encode_input_map(&m[2], x, cols, kMaxM, 24);
+bool encode_input_maps(CUtensorMap (&m)[3], const void* xs, int cols) {
+  return encode_split_map(&m[0], xs, cols, kMaxM, 8) && encode_split_map(&m[1], xs, cols, kMaxM, 16) &&
+         encode_split_map(&m[2], xs, cols, kMaxM, 24);
+}
+
+// fp32 rows as split rows, times norm weights if there are any: for the
+// products whose inputs no kernel of this file wrote (a walk that goes on past
+// an exit, whose rows carry the final norm; ssd_op_gemv).
+__global__ void __launch_bounds__(256)
+    k_split_rows(const Bufs B, RowSel sel, const float* __restrict__ x,
+                 const __nv_bfloat16* __restrict__ gnorm, __nv_bfloat16* xs, int K) {
+  pdl_wait();
+  pdl_launch_dependents();
+  int pos0, M;
+  resolve_rows(B.ctl, sel, pos0, M);
+  const int m = blockIdx.y, i = blockIdx.x * 256 + threadIdx.x;
+  if (m >= M || i >= K) return;
+  float v = x[(size_t)m * K + i];
+  if (gnorm) v *= __bfloat162float(gnorm[i]);
+  put_split(xs + (size_t)m * K + i, (size_t)kMaxM * K, v);
+}
+
+static cudaError_t split_rows(const Bufs& B, RowSel sel, const float* x, const void* gnorm,
+                              __nv_bfloat16* xs, int K, int mrows, cudaStream_t st) {
+  return launch_ex(k_split_rows, dim3((K + 255) / 256, mrows), dim3(256), 0, st, B, sel, x,
+                   static_cast<const __nv_bfloat16*>(gnorm), xs, K);
+}
+
+cudaError_t launch_resplit(const Dims& D, const Bufs& B, const void* gnorm, RowSel sel, int mrows,
+                           cudaStream_t st) {
+  return split_rows(B, sel, B.h, gnorm, B.xs_h, D.d, mrows, st);
 }
 
 cudaError_t launch_tile_part(const Dims& D, const Bufs& B, const TileMaps& tm, const LayerW& w,
-                             int layer, int part, RowSel sel, int mrows, cudaStream_t st) {
+                             int layer, int part, const void* next_norm, RowSel sel, int mrows,
+                             cudaStream_t st) {
   TArgs a{};
   a.D = D;
   a.B = B;
@@ -1092,32 +1017,32 @@ cudaError_t launch_tile_part(const Dims& D, const Bufs& B, const TileMaps& tm, c
   switch (part) {
     case 0:
       a.g = make_tgeom(D, (D.Hq + 2 * D.Hkv) * D.hd, D.d, kTMapQKV);
-      a.gnorm = static_cast<const __nv_bfloat16*>(w.attn_norm);
       a.ss_in = 0;
-      return tile_dispatch<kKQKV, true>(*w.tm[0], tm.h, a, mrows, st);
+      return tile_dispatch<kKQKV>(*w.tm[0], tm.h, a, mrows, st);
     case 2:
       a.g = make_tgeom(D, D.d, D.qd, kTMapLinear);
       a.ss_in = -1;
       a.which = 1;
-      return tile_dispatch<kKResid, false>(*w.tm[1], tm.attn_out, a, mrows, st);
+      a.gout = static_cast<const __nv_bfloat16*>(w.ffn_norm);
+      return tile_dispatch<kKResid>(*w.tm[1], tm.attn_out, a, mrows, st);
     case 3:
       a.g = make_tgeom(D, 2 * D.F, D.d, kTMapGateUp);
-      a.gnorm = static_cast<const __nv_bfloat16*>(w.ffn_norm);
       a.ss_in = 1;
-      return tile_dispatch<kKGateUp, true>(*w.tm[2], tm.h, a, mrows, st);
+      return tile_dispatch<kKGateUp>(*w.tm[2], tm.h, a, mrows, st);
     case 4:
       a.g = make_tgeom(D, D.d, D.F, kTMapLinear);
       a.ss_in = -1;
       a.which = 0;
-      return tile_dispatch<kKResid, false>(*w.tm[3], tm.act, a, mrows, st);
+      a.gout = static_cast<const __nv_bfloat16*>(next_norm);
+      return tile_dispatch<kKResid>(*w.tm[3], tm.act, a, mrows, st);
     default:
       return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t launch_tile_chain(const Dims& D, const Bufs& B, const TileMaps& tm, const LayerW& w,
-                              const LayerW* next, int layer, RowSel sel, int mrows,
-                              cudaStream_t st) {
+                              const LayerW* next, const void* final_norm, int layer, RowSel sel,
+                              int mrows, cudaStream_t st) {
   const int tp = tp_index(mrows);
   ChainArgs ca{};
   ChainMaps cm{};
@@ -1131,23 +1056,23 @@ cudaError_t launch_tile_chain(const Dims& D, const Bufs& B, const TileMaps& tm, 
   // O projection + residual
   ca.ph[0].g = make_tgeom(D, D.d, D.qd, kTMapLinear);
   ca.ph[0].which = 1;
+  ca.ph[0].gout = static_cast<const __nv_bfloat16*>(w.ffn_norm);
   cm.w[0] = *w.tm[1];
   cm.x[0] = tm.attn_out[tp];
   // RMSNorm + gate/up + SwiGLU
   ca.ph[1].g = make_tgeom(D, 2 * D.F, D.d, kTMapGateUp);
-  ca.ph[1].gnorm = static_cast<const __nv_bfloat16*>(w.ffn_norm);
   ca.ph[1].ss_in = 1;
   cm.w[1] = *w.tm[2];
   cm.x[1] = tm.h[tp];
   // down projection + residual
   ca.ph[2].g = make_tgeom(D, D.d, D.F, kTMapLinear);
   ca.ph[2].which = 0;
+  ca.ph[2].gout = static_cast<const __nv_bfloat16*>(next ? next->attn_norm : final_norm);
   cm.w[2] = *w.tm[3];
   cm.x[2] = tm.act[tp];
   ca.nph = 3;
   if (next) {  // the next layer's RMSNorm + QKV + RoPE + KV append
     ca.ph[3].g = make_tgeom(D, (D.Hq + 2 * D.Hkv) * D.hd, D.d, kTMapQKV);
-    ca.ph[3].gnorm = static_cast<const __nv_bfloat16*>(next->attn_norm);
     ca.ph[3].ss_in = 0;
     ca.ph[3].layer = layer + 1;
     cm.w[3] = *next->tm[0];
@@ -1167,32 +1092,30 @@ cudaError_t launch_tile_chain(const Dims& D, const Bufs& B, const TileMaps& tm, 
 }
 
 cudaError_t launch_tile_head(const Dims& D, const Bufs& B, const TileMaps& tm,
-                             const CUtensorMap& lm, const void* final_norm, RowSel sel, int mrows,
-                             cudaStream_t st) {
+                             const CUtensorMap& lm, RowSel sel, int mrows, cudaStream_t st) {
   TArgs a{};
   a.D = D;
   a.B = B;
   a.sel = sel;
   a.g = make_tgeom(D, D.V, D.d, kTMapLinear);
-  a.gnorm = static_cast<const __nv_bfloat16*>(final_norm);
   a.ss_in = 0;
-  return tile_dispatch<kKHead, true>(lm, tm.h, a, mrows, st);
+  return tile_dispatch<kKHead>(lm, tm.h, a, mrows, st);
 }
 
 cudaError_t launch_tile_plain(const Dims& D, const Bufs& B, const CUtensorMap& wm, int rows,
                               int cols, const float* x, int M, float* y, cudaStream_t st) {
   CUtensorMap xm[3];
-  const int tp = tp_index(M);
-  if (!encode_input_map(&xm[tp], x, cols, M, tp == 0 ? 8 : (tp == 1 ? 16 : 24)))
-    return cudaErrorInvalidValue;
+  if (!encode_input_maps(xm, B.xs_x, cols)) return cudaErrorInvalidValue;
   TArgs a{};
   a.D = D;
   a.B = B;
   a.sel = RowSel{kRowsExplicit, 0, M, nullptr};
+  const cudaError_t e = split_rows(B, a.sel, x, nullptr, B.xs_x, cols, M, st);
+  if (e != cudaSuccess) return e;
   a.g = make_tgeom(D, rows, cols, kTMapLinear);
   a.ss_in = -1;
   a.y = y;
-  return tile_dispatch<kKPlain, false>(wm, xm, a, M, st);
+  return tile_dispatch<kKPlain>(wm, xm, a, M, st);
 }
 
 }  // namespace ssd

@@ -97,16 +97,6 @@ struct WArgs {
 
 __device__ __forceinline__ void w_flag(const Bufs& B) { atomicOr(&B.ctl->err, (int)kErrTimeout); }
 
-// 3-D tiled load (columns, rows, part).
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int c0, int r0,
-                                            int z0, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(r0), "r"(z0), "r"(smem_u32(bar))
-      : "memory");
-}
-
 __device__ __forceinline__ void tma_load_2d_plain(void* dst, const CUtensorMap* map, int c0, int r0,
                                                   uint64_t* bar) {
   asm volatile(
