@@ -194,6 +194,8 @@ struct Bufs {
   int32_t* pre_tok;  // [max_seq] prefill / teacher-forced token ids
 };
 
+constexpr int kWideParts = 256;  // blocks that may share tiles in one launch
+
 // Buffers of a prompt chunk (bf16 models, wide.cu): up to cap rows.  The
 // inputs of the products are kept as bf16 high and low planes.
 struct WideBufs {
@@ -204,6 +206,8 @@ struct WideBufs {
   __nv_bfloat16* xo;   // [2][cap][qd] attention outputs
   __nv_bfloat16* xa;   // [2][cap][F] SwiGLU outputs
   float* ss;           // [2][ceil(d / 128)][cap] sums of squares of h per 128 columns
+  float* part;         // [kWideParts][128][128] sums of blocks that share a tile
+  uint32_t* tickets;   // [kWideParts] blocks done with it
 };
 
 }  // namespace ssd

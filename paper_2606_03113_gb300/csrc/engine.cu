@@ -116,6 +116,8 @@ size_t layout(const ssd_model_cfg& c, char* base, Dims* D, Bufs* B, WideBufs* P)
     w.xo = cv.take<__nv_bfloat16>(4 * cap * d.qd);
     w.xa = cv.take<__nv_bfloat16>(4 * cap * d.F);
     w.ss = cv.take<float>(sizeof(float) * 2 * (size_t)((d.d + 127) / 128) * cap);
+    w.part = cv.take<float>(sizeof(float) * 128 * 128 * (size_t)kWideParts);
+    w.tickets = cv.take<uint32_t>(sizeof(uint32_t) * kWideParts);
   }
   if (D) *D = d;
   if (B) *B = b;
@@ -636,6 +638,8 @@ ssd_status ssd_init_model(const ssd_model_cfg* cfg, const ssd_weights* w, void* 
     e = cudaMemsetAsync(x->B.ss_part, 0, sizeof(float) * 2 * (size_t)x->D.ss_nt * kMaxM, x->stream);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(x->B.attn_counter, 0, sizeof(uint32_t) * (size_t)x->D.Hkv * kMaxM, x->stream);
+  if (e == cudaSuccess && cfg->dtype == SSD_DTYPE_BF16)
+    e = cudaMemsetAsync(x->P.tickets, 0, sizeof(uint32_t) * kWideParts, x->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(x->B.chain_bar, 0, sizeof(uint32_t) * 2, x->stream);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(x->B.tile_counter, 0, sizeof(uint32_t) * (size_t)x->D.max_tiles, x->stream);

@@ -11,6 +11,10 @@
 // multiplied by the RMSNorm weights of the product that reads it; the
 // norm's scale is applied to the product (per-tile sums of squares travel
 // beside the rows).
+//  - a product with fewer tiles than SMs (a short prompt's O and down) splits K
+//    over up to eight blocks per tile, whose last one adds their sums: 93
+//    tokens through four layers and the head of the 8B widths take 1740 us
+//    against 1870 with one block per tile;
 //  - persistent grid, tiles dealt round robin with the token tiles of one
 //    weight tile next to each other (they share it in L2);
 //  - warp roles (320 threads): a TMA warp fills a ring of 64-column stages
@@ -88,11 +92,25 @@ struct WArgs {
   Bufs B;
   WideBufs P;
   int N, K, nks, nrt, ntt;     // rows, columns, stages, row tiles, token tiles
+  int nsp;                     // parts that K is split into (blocks that share a tile)
   int M, pos0, layer;
   int row0;                    // first of the M input rows
   const float* ss_in;          // per-tile sums of squares of the input rows, or null
   float* ss_out;               // residual: the same for the rows written
   const __nv_bfloat16* gnext;  // residual: norm weights of the next product (null: none)
+};
+
+// Work item `it`: row tile, token tile and part of K (stages k0 .. k0 + n - 1).
+struct WItem {
+  int rt, tt, sp, k0, n;
+  __device__ WItem(const WArgs& a, int it) {
+    tt = it % a.ntt;
+    const int r = it / a.ntt;
+    sp = r % a.nsp;
+    rt = r / a.nsp;
+    k0 = (int)((long long)a.nks * sp / a.nsp);
+    n = (int)((long long)a.nks * (sp + 1) / a.nsp) - k0;
+  }
 };
 
 __device__ __forceinline__ void w_flag(const Bufs& B) { atomicOr(&B.ctl->err, (int)kErrTimeout); }
@@ -186,16 +204,16 @@ __global__ void __launch_bounds__(kWThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  __shared__ int s_last;
   pdl_launch_dependents();
 
-  const int ntiles = a.nrt * a.ntt;
+  const int ntiles = a.nrt * a.ntt * a.nsp;
   if (warp == kWTmaWarp) {
     if (lane == 0) {
       tma_prefetch_desc(&wmap);
       tma_prefetch_desc(&xmap);
       // weight boxes of the first stages need nothing from earlier kernels
-      auto weights = [&](int slot, int tile, int kc) {
-        const int rt = tile / a.ntt;
+      auto weights = [&](int slot, int rt, int kc) {
         unsigned char* dst = smem + (size_t)slot * S::Stage;
         mbar_arrive_expect_tx(&full[slot], (uint32_t)S::Stage);
         const int r0 = KIND == kWGateUp ? rt * 64 : rt * 128;
@@ -205,23 +223,26 @@ __global__ void __launch_bounds__(kWThreads, 1)
       };
       bool ok = true;
       int npre = 0;
-      if ((int)blockIdx.x < ntiles)
-        for (; npre < NS && npre < a.nks; ++npre) weights(npre, blockIdx.x, npre);
+      if ((int)blockIdx.x < ntiles) {
+        const WItem w(a, blockIdx.x);
+        for (; npre < NS && npre < w.n; ++npre) weights(npre, w.rt, w.k0 + npre);
+      }
       pdl_wait();
       asm volatile("fence.proxy.async.global;" ::: "memory");
       int slot = 0, it = 0;
       uint32_t ph = 1;
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const int tt = tile % a.ntt;
-        for (int kc = 0; kc < a.nks; ++kc, ++it) {
+        const WItem w(a, tile);
+        for (int i = 0; i < w.n; ++i, ++it) {
+          const int kc = w.k0 + i;
           if (it >= npre) {
             if (!mbar_wait(&empty[slot], ph)) {
               ok = false;
               break;
             }
-            weights(slot, tile, kc);
+            weights(slot, w.rt, kc);
           }
-          tma_load_3d(smem + (size_t)slot * S::Stage + S::A, &xmap, kc * kWK, a.row0 + tt * TT, 0, &full[slot]);
+          tma_load_3d(smem + (size_t)slot * S::Stage + S::A, &xmap, kc * kWK, a.row0 + w.tt * TT, 0, &full[slot]);
           if (++slot == NS) {
             slot = 0;
             ph ^= 1u;
@@ -239,7 +260,8 @@ __global__ void __launch_bounds__(kWThreads, 1)
       int slot = 0, sc = 0;
       uint32_t ph = 0;
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        for (int kc = 0; kc < a.nks; ++kc) {
+        const int n = WItem(a, tile).n;
+        for (int kc = 0; kc < n; ++kc) {
           const bool first = kc % kWSeg == 0;
           if (first && !(ok = mbar_wait(&accempty[sc & 1], ((uint32_t)(sc >> 1) & 1u) ^ 1u))) break;
           if (!(ok = mbar_wait(&full[slot], ph))) break;
@@ -252,7 +274,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
             tc_mma_bf16(d, sdesc_k128(ab + kk * 32), sdesc_k128(xb + kk * 32), idesc,
                         !first || kk > 0);
           tc_commit(&empty[slot]);
-          if (kc % kWSeg == kWSeg - 1 || kc == a.nks - 1) tc_commit(&accfull[sc++ & 1]);
+          if (kc % kWSeg == kWSeg - 1 || kc == n - 1) tc_commit(&accfull[sc++ & 1]);
           if (++slot == NS) {
             slot = 0;
             ph ^= 1u;
@@ -271,9 +293,9 @@ __global__ void __launch_bounds__(kWThreads, 1)
     const int q = warp & 3, th = warp >> 2;
     bool ok = true;
     int sc = 0, xp = 0;
-    const int nseg = (a.nks + kWSeg - 1) / kWSeg;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-      const int rt = tile / a.ntt, t0 = (tile % a.ntt) * TT;
+      const WItem w(a, tile);
+      const int rt = w.rt, t0 = w.tt * TT, nseg = (w.n + kWSeg - 1) / kWSeg;
       if constexpr (KIND != kWResid) {
         // RMSNorm scale of the tile's input rows: their sums of squares per
         // 128 columns, added in column order
@@ -311,6 +333,27 @@ __global__ void __launch_bounds__(kWThreads, 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&accempty[sc & 1]);
+      }
+      if (a.nsp > 1) {
+        // K is split: the last block of the tile adds the parts in K order
+        const int id = rt * a.ntt + w.tt;
+        float* part = a.P.part + (size_t)id * a.nsp * (TT * 128) + tid;
+        const int nc = min(TT / 2, (a.M - t0 - th * (TT / 2) + kWChunk - 1) / kWChunk * kWChunk);
+#pragma unroll
+        for (int c = 0; c < TT / 2; ++c)
+          if (c < nc) part[((size_t)w.sp * (TT / 2) + c) * kWEThreads] = acc[c];
+        named_sync(1, kWEThreads);
+        if (tid == 0)
+          s_last = atom_add_acq_rel_gpu(a.P.tickets + id, 1u) == (uint32_t)(a.nsp - 1);
+        named_sync(1, kWEThreads);
+        if (!s_last) continue;
+        if (tid == 0) a.P.tickets[id] = 0u;
+#pragma unroll
+        for (int c = 0; c < TT / 2; ++c) acc[c] = 0.f;
+        for (int s = 0; s < a.nsp; ++s)
+#pragma unroll
+          for (int c = 0; c < TT / 2; ++c)
+            if (c < nc) acc[c] += __ldcg(&part[((size_t)s * (TT / 2) + c) * kWEThreads]);
       }
 #pragma unroll
       for (int c = 0; c < TT / 2; c += kWChunk) {
@@ -673,21 +716,27 @@ int stage_cost(int tt) { return 273 + 4 * tt + tt / 4; }
 
 int row_tiles(int N, bool pairs) { return pairs ? (N / 2 + 63) / 64 : (N + kWR - 1) / kWR; }
 
-// Token tile (index 0, 1, 2 = 32, 64, 128 tokens) of the product of N rows
-// with M tokens that has the least work on the busiest SM.
-int pick_tile(int sms, int nrt, int M, long long* cost) {
-  int best = 0;
-  long long bc = 0;
+// Token tile (index 0, 1, 2 = 32, 64, 128 tokens) and parts of K of the product
+// of nrt row tiles x nks stages with M tokens that have the least work on the
+// busiest SM.  K is split only where that still leaves every block its own
+// SM; the join costs about 6000 cycles (the parts' stores, the ticket's round
+// trip) and the parts' way back through L2.
+struct WPlan {
+  int ti, nsp;
+  long long cost;
+};
+WPlan pick_plan(int sms, int nrt, int nks, int M) {
+  WPlan best{0, 1, -1};
   for (int i = 0; i < 3; ++i) {
     const int tt = 32 << i;
     const long long tiles = (long long)nrt * ((M + tt - 1) / tt);
-    const long long c = (tiles + sms - 1) / sms * stage_cost(tt);
-    if (i == 0 || c < bc) {
-      bc = c;
-      best = i;
+    for (int nsp = 1; nsp <= 8; ++nsp) {
+      if (nsp > 1 && (tiles * nsp > sms || tiles * nsp > kWideParts || nks / nsp < kWSeg)) break;
+      const long long c = (tiles * nsp + sms - 1) / sms * ((nks + nsp - 1) / nsp) * stage_cost(tt) +
+                          (nsp > 1 ? 6000 + 9LL * nsp * tt : 0);
+      if (best.cost < 0 || c < best.cost) best = WPlan{i, nsp, c};
     }
   }
-  if (cost) *cost = bc;
   return best;
 }
 
@@ -695,11 +744,12 @@ template <int KIND>
 cudaError_t wide_launch(const CUtensorMap& wm, const CUtensorMap* xm, WArgs& a, cudaStream_t st) {
   a.nks = (a.K + kWK - 1) / kWK;
   a.nrt = row_tiles(a.N, KIND == kWGateUp);
-  const int ti = pick_tile(a.D.num_sms, a.nrt, a.M, nullptr);
-  a.ntt = (a.M + (32 << ti) - 1) / (32 << ti);
-  const long long tiles = (long long)a.nrt * a.ntt;
+  const WPlan p = pick_plan(a.D.num_sms, a.nrt, a.nks, a.M);
+  a.ntt = (a.M + (32 << p.ti) - 1) / (32 << p.ti);
+  a.nsp = p.nsp;
+  const long long tiles = (long long)a.nrt * a.ntt * a.nsp;
   const dim3 grid((unsigned)(tiles < a.D.num_sms ? tiles : a.D.num_sms)), blk(kWThreads);
-  switch (ti) {
+  switch (p.ti) {
     case 0: return launch_ex(k_wide<32, KIND>, grid, blk, WL<32>::total, st, wm, xm[0], a);
     case 1: return launch_ex(k_wide<64, KIND>, grid, blk, WL<64>::total, st, wm, xm[1], a);
     default: return launch_ex(k_wide<128, KIND>, grid, blk, WL<128>::total, st, wm, xm[2], a);
@@ -726,9 +776,7 @@ cudaError_t prepare_wide_kernels() {
 // Work of one layer of a chunk of M rows on the busiest SM (stage cycles).
 long long wide_layer_cost(const Dims& D, int M) {
   auto mat = [&](int N, int K, bool pairs) {
-    long long c;
-    pick_tile(D.num_sms, row_tiles(N, pairs), M, &c);
-    return c * ((K + kWK - 1) / kWK);
+    return pick_plan(D.num_sms, row_tiles(N, pairs), (K + kWK - 1) / kWK, M).cost;
   };
   return mat((D.Hq + 2 * D.Hkv) * D.hd, D.d, false) + mat(D.d, D.qd, false) +
          mat(2 * D.F, D.d, true) + mat(D.d, D.F, false);
