@@ -38,7 +38,7 @@
 // with a running maximum; scores and outputs on mma.sync with the fp32
 // operand (queries, probabilities) in three bf16 parts, 24 bits, so nothing
 // is rounded below fp32.  Bound by mma.sync: 512 rows of the Llama-2-7B shape
-// take 42 us a layer, rows 1024-1919 of the 13B shape 262 us (315 TFLOP/s with
+// take 41 us a layer, rows 1024-1919 of the 13B shape 252 us (328 TFLOP/s with
 // the three parts).
 #include <math.h>
 
@@ -559,18 +559,19 @@ __global__ void __launch_bounds__(kAWThreads, 2)
 #pragma unroll
         for (int p = 0; p < np; ++p)
           ldsm4(sq + (uint32_t)((pass ? 0 : 2 - p) * kAQ * 256) + sw256(lrow, 2 * kk + lch), qa[p]);
+        // keys 16 n2 .. + 15 x 16 columns: two n-tiles
+        uint32_t kf[4][4];
 #pragma unroll
-        for (int n2 = 0; n2 < 4; ++n2) {
-          // keys 16 n2 .. + 15 x 16 columns: two n-tiles
-          uint32_t kf[4];
+        for (int n2 = 0; n2 < 4; ++n2)
           ldsm4(kd + sw256(16 * n2 + (lane & 7) + ((lane >> 4) << 3), 2 * kk + ((lane >> 3) & 1)),
-                kf);
+                kf[n2]);
 #pragma unroll
-          for (int p = 0; p < np; ++p) {
-            mma16816(s[2 * n2], qa[p], kf[0], kf[1]);
-            mma16816(s[2 * n2 + 1], qa[p], kf[2], kf[3]);
+        for (int p = 0; p < np; ++p)
+#pragma unroll
+          for (int n2 = 0; n2 < 4; ++n2) {
+            mma16816(s[2 * n2], qa[p], kf[n2][0], kf[n2][1]);
+            mma16816(s[2 * n2 + 1], qa[p], kf[n2][2], kf[n2][3]);
           }
-        }
       }
     // scale, causal mask, running maximum
     const int kbase = b * kAKB + 2 * (lane & 3);
@@ -608,28 +609,34 @@ __global__ void __launch_bounds__(kAWThreads, 2)
         split3(s[2 * ks + (e >> 1)][2 * (e & 1)], s[2 * ks + (e >> 1)][2 * (e & 1) + 1],
                pa[ks][0][e], pa[ks][1][e], pa[ks][2][e]);
 #pragma unroll
-    for (int n2 = 0; n2 < 8; ++n2) {
-      // this step's share of 16 columns in sums of its own, then one rounded
-      // fused multiply-add into the running output
-      float t[2][4];
+    for (int n4 = 0; n4 < 4; ++n4) {
+      // this step's share of 32 columns in sums of its own (four chains, to
+      // cover the latency of mma.sync), then one rounded fused multiply-add
+      // into the running output
+      float t[4][4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) t[0][e] = t[1][e] = 0.f;
-      uint32_t vf[4][4];
+      for (int n = 0; n < 4; ++n)
 #pragma unroll
-      for (int ks = 0; ks < 4; ++ks)
-        ldsm4t(vd + sw256(16 * ks + (lane & 15), 2 * n2 + (lane >> 4)), vf[ks]);
+        for (int e = 0; e < 4; ++e) t[n][e] = 0.f;
+      uint32_t vf[2][4][4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+          ldsm4t(vd + sw256(16 * ks + (lane & 15), 4 * n4 + 2 * h + (lane >> 4)), vf[h][ks]);
 #pragma unroll
       for (int p = 2; p >= 0; --p)
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-          mma16816(t[0], pa[ks][p], vf[ks][0], vf[ks][1]);
-          mma16816(t[1], pa[ks][p], vf[ks][2], vf[ks][3]);
-        }
+        for (int ks = 0; ks < 4; ++ks)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        o[2 * n2][e] = fmaf(o[2 * n2][e], f[e >> 1], t[0][e]);
-        o[2 * n2 + 1][e] = fmaf(o[2 * n2 + 1][e], f[e >> 1], t[1][e]);
-      }
+          for (int h = 0; h < 2; ++h) {
+            mma16816(t[2 * h], pa[ks][p], vf[h][ks][0], vf[h][ks][1]);
+            mma16816(t[2 * h + 1], pa[ks][p], vf[h][ks][2], vf[h][ks][3]);
+          }
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[4 * n4 + n][e] = fmaf(o[4 * n4 + n][e], f[e >> 1], t[n][e]);
     }
     __syncthreads();  // the buffer is staged again two steps on
   }
