@@ -613,8 +613,12 @@ __global__ void __launch_bounds__(256) k_attn_merge(const Dims D, const Bufs B, 
   *reinterpret_cast<uint2*>(xo + (size_t)kMaxM * D.qd) = lo;
 }
 
-// Keys per split of the bf16 kernel: 64, or 128 where 64 would make more
-// blocks than the SMs hold at once (three each) with a full cache.
+// Keys per split of the bf16 kernel: 64, or 128 where 64 would make more blocks
+// than three per SM with a full cache: fewer partials to store and merge, for
+// two key steps in a row.  Live with the merge, one row, a cache of 2304
+// positions, 128 against 64 keys: 32 KV heads at context 640 9.5 against 10.3
+// us, at 2048 17.7 against 18.6; 40 KV heads at 1000 12.4 both, at 2176 22.3
+// against 21.2.
 int attn_split_keys(int n_kv_heads, int max_seq, int sms) {
   const int n = (max_seq + kRStep - 1) / kRStep;
   return n_kv_heads * n > 3 * sms ? 2 * kRStep : kRStep;

@@ -137,6 +137,13 @@ struct Elem<__nv_bfloat16> {
   __device__ static __forceinline__ __nv_bfloat16 from_f(float v) { return __float2bfloat16_rn(v); }
 };
 
+// x as bf16 high and low parts into the planes of a split row buffer.
+__device__ __forceinline__ void put_split(__nv_bfloat16* p, size_t plane, float x) {
+  const __nv_bfloat16 h = __float2bfloat16_rn(x);
+  p[0] = h;
+  p[plane] = __float2bfloat16_rn(x - __bfloat162float(h));
+}
+
 // Per-layer weights (device pointers, model dtype).
 struct LayerW {
   const void* attn_norm;

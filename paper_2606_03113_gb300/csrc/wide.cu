@@ -164,13 +164,6 @@ __device__ __forceinline__ float warp_sum16(float (&v)[16], int lane) {
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-// x as bf16 high and low parts into the two planes of an operand buffer.
-__device__ __forceinline__ void put_split(__nv_bfloat16* p, size_t plane, float x) {
-  const __nv_bfloat16 h = __float2bfloat16_rn(x);
-  p[0] = h;
-  p[plane] = __float2bfloat16_rn(x - __bfloat162float(h));
-}
-
 }  // namespace
 
 template <int TT, int KIND>
