@@ -105,7 +105,7 @@ __device__ __forceinline__ float warp_row_total(const float* sums, int nch) {
 // Inverse-CDF draw from non-negative weights w(v) whose chunk sums are given:
 // with W their total and C_v = w(0) + ... + w(v) in token order, the token is
 // the first v with C_v > u W; *margin = min(u W - C_{v-1}, C_v - u W) / W.
-// Returns -1 when W is not positive; when rounding leaves u W at or beyond
+// Returns -1 when W is not positive and finite; when rounding leaves u W at or beyond
 // the total (of the vocabulary or of the chunk), the last token of positive
 // weight before it (margin 0).  Every thread of the block calls it.
 template <typename W>
@@ -125,7 +125,7 @@ __device__ int block_draw(int V, const W& w, const float* sums, float u, float* 
   if (tid < nch && sm.part[tid] > T) atomicMin(&sm.first, tid);
   __syncthreads();
   int c = sm.first;
-  if (!(S > 0.f)) return -1;
+  if (!(S > 0.f && S < INFINITY)) return -1;
   const bool beyond = c >= nch;
   if (beyond) c = nch - 1;
   const float base = c > 0 ? sm.part[c - 1] : 0.f;

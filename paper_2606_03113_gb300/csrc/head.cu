@@ -12,7 +12,9 @@
 // barriers and the round trips of the row's ticket.
 //
 // Every sum has a fixed order that depends on the vocabulary alone, so a
-// row's statistics are the same whatever the number of rows.
+// row's statistics are the same whatever the number of rows.  A NaN or -inf
+// logit takes part in nothing; a +inf one is the maximum, and the sums (lse,
+// entropy, pmax, C_k) are NaN, so that no draw is made from such a row.
 #include <math.h>
 
 #include "kernels.h"
@@ -161,12 +163,13 @@ __global__ void __launch_bounds__(kHThreads) k_head_stats(const Dims D, const Bu
       }
     s = block_sum(s, sm);
     t = block_sum(t, sm);
-    if (S > 0.f && s > 0.f) {
+    // (a sum that is not a number, from an infinite logit, stays one)
+    if (S != 0.f && s != 0.f) {
       const float nm = fmaxf(mx, cm), ea = expf(mx - nm), eb = expf(cm - nm);
       T = ea * (T + (mx - nm) * S) + eb * (t + (cm - nm) * s);
       S = S * ea + s * eb;
       mx = nm;
-    } else if (s > 0.f) {
+    } else if (s != 0.f) {
       mx = cm;
       S = s;
       T = t;
@@ -206,10 +209,10 @@ __global__ void __launch_bounds__(kHThreads) k_head_stats(const Dims D, const Bu
       const HeadPart* p = parts + (i >> 3);
       k[j] = i < np * kTopK ? make_key(__ldcg(&p->tv[i & 7]), __ldcg(&p->ti[i & 7])) : Key{0u, 0u};
     }
-    mx = block_max(ps > 0.f ? pm : -INFINITY, sm);
-    const float d = pm - mx, e = ps > 0.f ? expf(d) : 0.f;
-    S = block_sum(ps > 0.f ? ps * e : 0.f, sm);
-    T = block_sum(ps > 0.f ? e * (pt + d * ps) : 0.f, sm);
+    mx = block_max(ps != 0.f ? pm : -INFINITY, sm);
+    const float d = pm - mx, e = ps != 0.f ? expf(d) : 0.f;
+    S = block_sum(ps != 0.f ? ps * e : 0.f, sm);
+    T = block_sum(ps != 0.f ? e * (pt + d * ps) : 0.f, sm);
     block_topk(k, sm);
     if (tid == 0) B.head_counter[m] = 0u;
   }
