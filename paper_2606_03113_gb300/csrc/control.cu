@@ -55,7 +55,7 @@ struct SampleSmem {
   float red[kSampleThreads / 32];
   float rows[kMaxM];           // row totals
   float pd[kMaxDraft], qd[kMaxDraft];
-  int first, tok;
+  int first, end, tok;
   float margin;
 };
 
@@ -105,9 +105,12 @@ __device__ __forceinline__ float warp_row_total(const float* sums, int nch) {
 // Inverse-CDF draw from non-negative weights w(v) whose chunk sums are given:
 // with W their total and C_v = w(0) + ... + w(v) in token order, the token is
 // the first v with C_v > u W; *margin = min(u W - C_{v-1}, C_v - u W) / W.
-// Returns -1 when W is not positive and finite; when rounding leaves u W at or beyond
-// the total (of the vocabulary or of the chunk), the last token of positive
-// weight before it (margin 0).  Every thread of the block calls it.
+// Returns -1 when W is not positive and finite.  The chunk and, in it, the
+// thread's run that hold u W are the first whose prefix sums exceed it; a run is
+// walked by its own thread alone, from the prefix before it.  Where rounding
+// leaves u W at or beyond the total, or beyond the sum that the walk reaches, the
+// token is the last one of positive weight up to there (margin 0): never one
+// of weight 0.  Every thread of the block calls it.
 template <typename W>
 __device__ int block_draw(int V, const W& w, const float* sums, float u, float* margin,
                           SampleSmem& sm) {
@@ -116,42 +119,49 @@ __device__ int block_draw(int V, const W& w, const float* sums, float u, float* 
   static_assert(kSampChunks <= kSampleThreads, "a chunk per thread");
   if (tid == 0) {
     sm.first = kSampChunks;
-    sm.tok = 0x7fffffff;
+    sm.tok = -1;
     sm.margin = 0.f;
   }
   block_prefix(tid < nch ? __ldcg(sums + tid) : 0.f, sm);
   const float S = sm.part[kSampleThreads - 1];
+  if (!(S > 0.f && S < INFINITY)) return -1;
   const float T = u * S;
   if (tid < nch && sm.part[tid] > T) atomicMin(&sm.first, tid);
   __syncthreads();
   int c = sm.first;
-  if (!(S > 0.f && S < INFINITY)) return -1;
   const bool beyond = c >= nch;
   if (beyond) c = nch - 1;
   const float base = c > 0 ? sm.part[c - 1] : 0.f;
   __syncthreads();
   int v0, v1;
   thread_run(V, c, v0, v1);
+  if (tid == 0) {
+    sm.first = kSampleThreads;
+    sm.end = min(V, (c + 1) * samp_chunk(V));
+  }
   if (!beyond) {
     block_prefix(run_sum(v0, v1, w), sm);
-    float cum = base + (tid > 0 ? sm.part[tid - 1] : 0.f), mg = 0.f;
-    int found = 0x7fffffff;
-    for (int v = v0; v < v1; ++v) {
-      const float nx = cum + w(v);
-      if (nx > T) {
-        found = v;
-        mg = fmaxf(fminf(T - cum, nx - T), 0.f) / S;
-        break;
-      }
-      cum = nx;
-    }
-    if (found != 0x7fffffff) atomicMin(&sm.tok, found);
+    if (base + sm.part[tid] > T) atomicMin(&sm.first, tid);
     __syncthreads();
-    if (sm.tok == found && found != 0x7fffffff) sm.margin = mg;
+    if (tid == sm.first) {
+      float cum = base + (tid > 0 ? sm.part[tid - 1] : 0.f);
+      sm.end = v0;  // where nothing in the run has weight
+      for (int v = v0; v < v1; ++v) {
+        const float wv = w(v);
+        if (!(wv > 0.f)) continue;
+        sm.tok = v;
+        const float nx = cum + wv;
+        if (nx > T) {
+          sm.margin = fmaxf(fminf(T - cum, nx - T), 0.f) / S;
+          break;
+        }
+        cum = nx;
+      }
+    }
     __syncthreads();
   }
-  if (tid == 0 && sm.tok == 0x7fffffff) {
-    int v = min(V, (c + 1) * samp_chunk(V)) - 1;
+  if (tid == 0 && sm.tok < 0) {
+    int v = sm.end - 1;
     while (v > 0 && !(w(v) > 0.f)) --v;
     sm.tok = v;
   }

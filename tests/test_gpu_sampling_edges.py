@@ -1,4 +1,5 @@
-"""Draws from hand-set logits: rows whose logits are not finite.
+"""Draws from hand-set logits: weights of exactly zero with u S in the rounding
+gap between two threads' runs, and rows whose logits are not finite.
 
 The model's layers add nothing (wo = w_down = 0), every embedding is a row of
 ones and eps is 0, so the normed row is ones and a logit is the sum of its
@@ -8,6 +9,7 @@ import dataclasses
 import numpy as np
 import pytest
 
+import synth
 from parity import has_gpu
 from synth.workloads import TINY, scaled_down
 from paper_2606_03113_gb300 import ssd as S
@@ -29,6 +31,37 @@ def engine(V, z):
     dm.lm_head[:, 0] = torch.from_numpy(np.asarray(z, dtype=np.float32)).cuda()
     torch.cuda.synchronize()
     return dm, Engine(dm, 128)
+
+
+def test_token_of_zero_weight_is_never_drawn():
+    # Token 1 has weight 1; the first token of each 8-token run has weight 0,
+    # the others 0.9 x 2^-25, which a running sum above 1 cannot take up (half
+    # its last place is 2^-24) but the sums of runs and chunks do.  Every u S
+    # above 1 then lies between the end of a run's sequential sum and the prefix
+    # that the next run starts from.
+    V = 32768
+    z = np.full(V, np.log(0.9 * 2.0 ** -25), dtype=np.float32)
+    z[::8] = -200.0
+    z[1] = 0.0
+    wgt = np.exp(z.astype(np.float64))
+    wgt[::8] = 0.0
+    cdf = np.cumsum(wgt) / wgt.sum()
+    ids = np.arange(5, dtype=np.int32)
+    above = [(s, u) for s in range(40000)
+             for u in [float(synth.sample_uniforms(s, len(ids) - 1, 2, 1)[0])] if u > cdf[7]][:12]
+    assert len(above) == 12
+    dm, eng = engine(V, z)
+    try:
+        zg, _ = eng.forward_exit(ids, 0, 1)
+        assert np.array_equal(zg[0], z)
+        for seed, u in above:
+            eng.set_ar(temperature=1.0, sample_seed=seed)
+            t = eng.prefill(ids)
+            assert z[t] > -200.0, (seed, u, t)
+            # fp32 sums of at most 8 + 256 + 16 terms, all below 2: 2^-23 each
+            assert abs(cdf[t] - u) < 280 * 2.0 ** -23
+    finally:
+        eng.close()
 
 
 @pytest.mark.parametrize("V", [1024, 8192])
