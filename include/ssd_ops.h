@@ -51,23 +51,29 @@ ssd_status ssd_read_kv(ssd_ctx* ctx, int32_t layer, int32_t kind, int32_t head, 
 ssd_status ssd_read_state(ssd_ctx* ctx, int32_t* x, int32_t* pos, float* trace, int32_t cap,
                           int32_t* n_trace);
 
-/* One launch of the weight-streaming matrix-vector kernel on the weights of
- * layer `layer`: which = 0 wqkv, 1 wo, 2 w_gate_up, 3 w_down, 4 lm_head
- * (layer ignored).  y[m][r] = sum_c W[r][c] x[m][c] for m < M (1 <= M <= 17),
- * x_dev [M][cols] and y_dev [M][rows] fp32 device buffers.  Enqueued on
- * `stream` (NULL = the context's stream); no synchronisation. */
+/* The weight-streaming matrix-vector kernel on the weights of layer `layer`:
+ * which = 0 wqkv, 1 wo, 2 w_gate_up, 3 w_down, 4 lm_head (layer ignored).
+ * y[m][r] = sum_c W[r][c] x[m][c] for m < M (1 <= M <= 17), x_dev [M][cols] and
+ * y_dev [M][rows] fp32 device buffers.  fp32: one launch; bf16: a short launch
+ * splits x into two bf16 parts in front of it.  Enqueued on `stream` (NULL =
+ * the context's stream); no synchronisation. */
 ssd_status ssd_op_gemv(ssd_ctx* ctx, int32_t which, int32_t layer, int32_t M, const float* x_dev,
                        float* y_dev, void* stream);
 
-/* One launch of one hot-path kernel of layer `layer` exactly as the round
- * graphs launch it, on M rows at positions pos0..pos0+M-1 of the context's
- * own buffers: kernel = 0 QKV (+RoPE, KV append), 1 attention (split-K with
- * the split merge in the same kernel), 2 O projection (+residual), 3 gate/up (+RMSNorm, SwiGLU),
- * 4 down projection (+residual), 5 exit head (final RMSNorm, LM head,
- * statistics; layer ignored), 6 (bf16) the chained launch the layer passes
- * use: O projection, gate/up and down of `layer` and the QKV of layer + 1
- * (when there is one) as the phases of one persistent kernel.  It overwrites the activations and the KV rows
- * at those positions: for timing and profiling, not inside a generation.
+/* One hot-path kernel of layer `layer`, on M rows at positions
+ * pos0..pos0+M-1 of the context's own buffers: kernel = 0 QKV (+RMSNorm, RoPE,
+ * KV append), 1 attention (bf16: the splits and, in a second launch, their
+ * merge; fp32: one launch), 2 O projection (+residual), 3 gate/up (+RMSNorm,
+ * SwiGLU), 4 down projection (+residual), 5 exit head (final RMSNorm and LM
+ * head, then the statistics in a launch of their own; layer ignored), 6 (bf16)
+ * the chained launch the layer passes use: O projection, gate/up and down of
+ * `layer` and the QKV of layer + 1 (when there is one) as the phases of one
+ * persistent kernel.  The kernels are the ones the passes launch.  Each reads
+ * what the kernel before it in a layer wrote; 0, 3 and 5 read the residual rows
+ * under their own norm weights, whatever wrote them last (bf16: a short launch
+ * in front multiplies the rows, which in a pass the kernel that writes them
+ * does).  It overwrites the activations and the KV rows at those positions: for
+ * timing and profiling, not inside a generation.
  * Needs pos0 + M <= max_seq.  Enqueued on `stream` (NULL = the context's). */
 ssd_status ssd_op_layer(ssd_ctx* ctx, int32_t kernel, int32_t layer, int32_t M, int32_t pos0,
                         void* stream);

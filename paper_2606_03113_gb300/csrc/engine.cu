@@ -1037,6 +1037,14 @@ ssd_status ssd_op_layer(ssd_ctx* x, int32_t kernel, int32_t layer, int32_t M, in
     return fail(x, SSD_ERR_INVALID_ARG, "the chained kernel is a bf16 kernel");
   cudaStream_t st = stream ? static_cast<cudaStream_t>(stream) : x->stream;
   const RowSel sel = rows_explicit(pos0, M, x->B.pre_tok);
+  // bf16: the rows' split parts carry the norm weights that their last writer
+  // expected behind it; a kernel asked for on its own reads them under its own
+  if (x->cfg.dtype == SSD_DTYPE_BF16 && (kernel == 0 || kernel == 3 || kernel == 5))
+    CK(x, launch_resplit(x->D, x->B,
+                         kernel == 0   ? x->layers[layer].attn_norm
+                         : kernel == 3 ? x->layers[layer].ffn_norm
+                                       : x->final_norm,
+                         sel, M, st));
   if (kernel == 5)
     CK(x, enqueue_head(x, sel, M, x->topk, st));
   else if (kernel == 6)
