@@ -624,29 +624,42 @@ int attn_split_keys(int n_kv_heads, int max_seq, int sms) {
   return n_kv_heads * n > 3 * sms ? 2 * kRStep : kRStep;
 }
 
+static size_t rows_smem(int keys, int groups) {
+  return (size_t)(keys / kRStep) * 2 * kRKeyBytes + groups * kRGroupBytes;
+}
+
+// The limits of dynamic shared memory, once and the same for every context: a
+// function's attributes are shared by all threads, and a launch's own size
+// depends on the model and on the number of rows.
+cudaError_t prepare_attention_kernels() {
+  cudaError_t e = cudaFuncSetAttribute(k_attn_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)rows_smem(2 * kRStep, kRMaxGroups));
+  if (e != cudaSuccess) return e;
+  // fp32: what the device has (the merge of a long cache takes more than a split's keys)
+  int dev = 0, most = 0;
+  cudaFuncAttributes fa;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
+    return e;
+  if ((e = cudaFuncGetAttributes(&fa, k_attn<float>)) != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_attn<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              most - (int)fa.sharedSizeBytes);
+}
+
 static cudaError_t attn_bf16(const Dims& D, const Bufs& B, int layer, RowSel sel, int mrows,
                              cudaStream_t st) {
   const int rows = mrows * (D.Hq / D.Hkv);
   const int groups = rows <= 16 ? 1 : (rows <= 32 ? 2 : kRMaxGroups);
-  const size_t smem = (size_t)(D.attn_keys / kRStep) * 2 * kRKeyBytes + groups * kRGroupBytes;
-  cudaError_t e =
-      cudaFuncSetAttribute(k_attn_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  const size_t smem = rows_smem(D.attn_keys, groups);
   const dim3 grid((D.max_seq + D.attn_keys - 1) / D.attn_keys, D.Hkv);
-  e = launch_ex(k_attn_rows, grid, dim3(groups * kRGThreads), smem, st, D, B, layer, sel);
+  cudaError_t e = launch_ex(k_attn_rows, grid, dim3(groups * kRGThreads), smem, st, D, B, layer, sel);
   if (e != cudaSuccess) return e;
   return launch_ex(k_attn_merge, dim3((mrows * D.Hq + 7) / 8), dim3(256), 0, st, D, B, sel);
 }
 
 static cudaError_t attn_f32(const Dims& D, const Bufs& B, int layer, RowSel sel, cudaStream_t st) {
   dim3 grid(D.nsplit, D.Hkv);
-  const size_t smem = attn_smem(D);
-  if (smem > 48 * 1024) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_attn<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  return launch_ex(k_attn<float>, grid, dim3(kAThreads), smem, st, D, B, layer, sel);
+  return launch_ex(k_attn<float>, grid, dim3(kAThreads), attn_smem(D), st, D, B, layer, sel);
 }
 
 cudaError_t launch_attention(const Dims& D, const Bufs& B, int dtype, int layer, RowSel sel,
