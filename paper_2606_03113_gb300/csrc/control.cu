@@ -710,6 +710,7 @@ __global__ void k_accept(Dims D, Bufs B, cudaGraphConditionalHandle gen_while) {
       if (n_out + lane < D.max_seq) B.out_tok[n_out + lane] = tok;
       c->trace[(head + lane) % kTraceCap] = pm;
     }
+    __syncwarp();  // every lane has read the control block
     if (lane == 0) {
       c->trace_head = (head + a + 1) % kTraceCap;
       c->trace_n = min(n_trace + a + 1, kTraceCap);
