@@ -191,11 +191,19 @@ ssd_status ssd_set_policy(ssd_ctx* ctx, const ssd_policy* policy);
  * positions, and returns the next token, which becomes the pending token:
  * the greedy one, or with a policy temperature > 0 (set before this call) a
  * draw from the full model's distribution at that temperature, its uniform
- * keyed by (sample_seed, n - 1).  Needs n + 1 <= max_seq.  Synchronises the stream once. */
+ * keyed by (sample_seed, n - 1).  Needs n + 1 <= max_seq.  Synchronises the stream once.
+ * bf16 models run more than 16 tokens through kernels of their own, whose sums
+ * are in another order than decoding's: the KV rows agree with those that
+ * decoding the same tokens leaves to rounding, not bit for bit.  A row's bits
+ * do not depend on the tokens after it: prompts of more than 16 tokens agree
+ * bit for bit on their common beginning. */
 ssd_status ssd_prefill(ssd_ctx* ctx, const int32_t* ids, int32_t n, int32_t* first_token);
 
 /* Like ssd_prefill over ids[0..n-1) but takes ids[n-1] as the pending token
- * (resumes a sequence whose last token is already chosen).  n >= 2. */
+ * (resumes a sequence whose last token is already chosen).  n >= 2.  With a
+ * bf16 model the rows that decoding wrote are recomputed as ssd_prefill does
+ * it, so a resumed sequence can go another way than the uninterrupted one where
+ * a decision is nearly a tie; fp32 rows are the same bit for bit. */
 ssd_status ssd_resume(ssd_ctx* ctx, const int32_t* ids, int32_t n);
 
 /* One speculation round, emitting 1..cap tokens into out_ids (host).  The

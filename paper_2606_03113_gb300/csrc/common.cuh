@@ -201,7 +201,7 @@ struct Bufs {
   int32_t* pre_tok;  // [max_seq] prefill / teacher-forced token ids
 };
 
-constexpr int kWideParts = 256;  // blocks that may share tiles in one launch
+constexpr int kWideParts = 512;  // partial sums of tiles that blocks share, in one launch
 
 // Buffers of a prompt chunk (bf16 models, wide.cu): up to cap rows.  The
 // inputs of the products are kept as bf16 high and low planes.
@@ -213,8 +213,8 @@ struct WideBufs {
   __nv_bfloat16* xo;   // [2][cap][qd] attention outputs
   __nv_bfloat16* xa;   // [2][cap][F] SwiGLU outputs
   float* ss;           // [2][ceil(d / 128)][cap] sums of squares of h per 128 columns
-  float* part;         // [kWideParts][128][128] sums of blocks that share a tile
-  uint32_t* tickets;   // [kWideParts] blocks done with it
+  float* part;         // [kWideParts][128][128] partial sums of tiles that blocks share
+  uint32_t* tickets;   // [kWideParts] blocks done with a tile
 };
 
 }  // namespace ssd

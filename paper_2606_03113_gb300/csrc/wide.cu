@@ -12,9 +12,11 @@
 // norm's scale is applied to the product (per-tile sums of squares travel
 // beside the rows).
 //  - a product with fewer tiles than SMs (a short prompt's O and down) splits K
-//    over up to eight blocks per tile, whose last one adds their sums: 93
-//    tokens through four layers and the head of the 8B widths take 1740 us
-//    against 1870 with one block per tile;
+//    over up to eight blocks per tile, whose last one adds their sums.  The
+//    segments of K that are added, and their order, depend on the matrix alone,
+//    so a row's bits do not depend on the length of the prompt.  (Parts that add
+//    their own segments first leave less to join, down of the 8B shape with 89
+//    rows 41.5 us against 48.4, but then the order follows the split.)
 //  - persistent grid, tiles dealt round robin with the token tiles of one
 //    weight tile next to each other (they share it in L2);
 //  - warp roles (320 threads): a TMA warp fills a ring of 64-column stages
@@ -42,6 +44,8 @@
 // the three parts).
 #include <math.h>
 
+#include <algorithm>
+
 #include "kernels.h"
 #include "mma.cuh"
 #include "pipe.cuh"
@@ -58,14 +62,15 @@ constexpr int kWEThreads = kWEpi * 32;
 constexpr int kWTmaWarp = kWEpi, kWMmaWarp = kWEpi + 1;
 constexpr int kWThreads = (kWEpi + 2) * 32;
 constexpr int kWChunk = 16;           // tokens per epilogue step of a warp
-// Stages summed in one TMEM accumulator before the epilogue warps add it to
-// their registers: the tensor core's running sum is cut and not rounded at
-// each 16-column step, so a sum over all of K in TMEM would be off by up to
-// K / 16 units in the last place, to one side.  1024 columns at a time keep
-// that at 64, as in the decode kernels, whose blocks sum 450 to 2300 columns
-// of a row each.  The drain is hidden by the other accumulator but for its
-// own tensor-memory reads: 512 tokens of the 12288 x 4096 product take 83.7
-// us (94.5 us with 512 columns at a time, 76.5 us with all of K).
+// K is summed in segments of at most this many stages, one TMEM accumulator
+// each, which the epilogue warps add in their registers: the tensor core's
+// running sum is cut and not rounded at each 16-column step, so a sum over all
+// of K in TMEM would be off by up to K / 16 units in the last place, to one
+// side.  1024 columns at a time keep that at 64, as in the decode kernels, whose
+// blocks sum 450 to 2300 columns of a row each.  The drain is hidden by the
+// other accumulator but for its own tensor-memory reads: 512 tokens of the
+// 12288 x 4096 product take 83.7 us (94.5 us with 512 columns at a time, 76.5 us
+// with all of K).
 constexpr int kWSeg = 16;
 
 enum WKind : int { kWQkv = 0, kWResid = 1, kWGateUp = 2, kWHead = 3 };
@@ -92,6 +97,7 @@ struct WArgs {
   Bufs B;
   WideBufs P;
   int N, K, nks, nrt, ntt;     // rows, columns, stages, row tiles, token tiles
+  int nseg, seg_q, seg_r;      // segments of K; stages of each, and the first ones that have one more
   int nsp;                     // parts that K is split into (blocks that share a tile)
   int M, pos0, layer;
   int row0;                    // first of the M input rows
@@ -100,18 +106,31 @@ struct WArgs {
   const __nv_bfloat16* gnext;  // residual: norm weights of the next product (null: none)
 };
 
-// Work item `it`: row tile, token tile and part of K (stages k0 .. k0 + n - 1).
+// First stage of segment g of K.
+__device__ __forceinline__ int w_seg_start(const WArgs& a, int g) {
+  return g * a.seg_q + min(g, a.seg_r);
+}
+
+// Work item `it`: row tile, token tile and part of K (segments g0 .. g1 - 1,
+// stages k0 .. k0 + n - 1).
 struct WItem {
-  int rt, tt, sp, k0, n;
+  int rt, tt, sp, g0, g1, k0, n;
   __device__ WItem(const WArgs& a, int it) {
     tt = it % a.ntt;
     const int r = it / a.ntt;
     sp = r % a.nsp;
     rt = r / a.nsp;
-    k0 = (int)((long long)a.nks * sp / a.nsp);
-    n = (int)((long long)a.nks * (sp + 1) / a.nsp) - k0;
+    g0 = a.nseg * sp / a.nsp;
+    g1 = a.nseg * (sp + 1) / a.nsp;
+    k0 = w_seg_start(a, g0);
+    n = w_seg_start(a, g1) - k0;
   }
 };
+
+// Partial sums that the parts of a tile leave: one of the first part's
+// segments, which are the first terms of the sum over K, and one of each
+// later segment.
+__host__ __device__ inline int w_slots(int nseg, int nsp) { return nseg - nseg / nsp + 1; }
 
 __device__ __forceinline__ void w_flag(const Bufs& B) { atomicOr(&B.ctl->err, (int)kErrTimeout); }
 
@@ -253,9 +272,10 @@ __global__ void __launch_bounds__(kWThreads, 1)
       int slot = 0, sc = 0;
       uint32_t ph = 0;
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const int n = WItem(a, tile).n;
-        for (int kc = 0; kc < n; ++kc) {
-          const bool first = kc % kWSeg == 0;
+        const WItem w(a, tile);
+        int g = w.g0, seg_end = w_seg_start(a, g + 1);
+        bool first = true;
+        for (int kc = w.k0; kc < w.k0 + w.n; ++kc) {
           if (first && !(ok = mbar_wait(&accempty[sc & 1], ((uint32_t)(sc >> 1) & 1u) ^ 1u))) break;
           if (!(ok = mbar_wait(&full[slot], ph))) break;
           tc_fence_after();
@@ -267,7 +287,11 @@ __global__ void __launch_bounds__(kWThreads, 1)
             tc_mma_bf16(d, sdesc_k128(ab + kk * 32), sdesc_k128(xb + kk * 32), idesc,
                         !first || kk > 0);
           tc_commit(&empty[slot]);
-          if (kc % kWSeg == kWSeg - 1 || kc == n - 1) tc_commit(&accfull[sc++ & 1]);
+          first = kc + 1 == seg_end;
+          if (first) {
+            tc_commit(&accfull[sc++ & 1]);
+            seg_end = w_seg_start(a, ++g + 1);
+          }
           if (++slot == NS) {
             slot = 0;
             ph ^= 1u;
@@ -288,7 +312,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
     int sc = 0, xp = 0;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
       const WItem w(a, tile);
-      const int rt = w.rt, t0 = w.tt * TT, nseg = (w.n + kWSeg - 1) / kWSeg;
+      const int rt = w.rt, t0 = w.tt * TT;
       if constexpr (KIND != kWResid) {
         // RMSNorm scale of the tile's input rows: their sums of squares per
         // 128 columns, added in column order
@@ -304,11 +328,15 @@ __global__ void __launch_bounds__(kWThreads, 1)
         }
         named_sync(1, kWEThreads);
       }
-      // the tile's sums: segments added in K order, high plus low parts
+      // the tile's sums: segments added in K order, high plus low parts; a later
+      // part of a split K hands its segments on one by one, so that the order
+      // is the same whatever the split
+      const int id = rt * a.ntt + w.tt, nslot = w_slots(a.nseg, a.nsp), first_later = a.nseg / a.nsp;
+      float4* part = reinterpret_cast<float4*>(a.P.part) + (size_t)id * nslot * (TT * 32) + tid;
       float acc[TT / 2];
 #pragma unroll
       for (int c = 0; c < TT / 2; ++c) acc[c] = 0.f;
-      for (int g = 0; g < nseg; ++g, ++sc) {
+      for (int g = w.g0; g < w.g1; ++g, ++sc) {
         if (ok) {
           ok = __all_sync(0xffffffffu, mbar_wait(&accfull[sc & 1], (uint32_t)(sc >> 1) & 1u));
           if (!ok && lane == 0) w_flag(a.B);
@@ -320,21 +348,30 @@ __global__ void __launch_bounds__(kWThreads, 1)
           if (ok && t0 + th * (TT / 2) + c < a.M) {
             float v[kWChunk];
             tc_ld16_sum(src + c, src + TT + c, v);
+            if (w.sp == 0) {
 #pragma unroll
-            for (int j = 0; j < kWChunk; ++j) acc[c + j] += v[j];
+              for (int j = 0; j < kWChunk; ++j) acc[c + j] += v[j];
+            } else {
+              float4* to = part + ((size_t)(g - first_later + 1) * (TT / 8) + c / 4) * kWEThreads;
+#pragma unroll
+              for (int j = 0; j < kWChunk; j += 4)
+                to[(size_t)(j / 4) * kWEThreads] = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            }
           }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&accempty[sc & 1]);
       }
       if (a.nsp > 1) {
-        // K is split: the last block of the tile adds the parts in K order
-        const int id = rt * a.ntt + w.tt;
-        float* part = a.P.part + (size_t)id * a.nsp * (TT * 128) + tid;
+        // K is split: the last block of the tile adds the partial sums in K order
         const int nc = min(TT / 2, (a.M - t0 - th * (TT / 2) + kWChunk - 1) / kWChunk * kWChunk);
+        if (w.sp == 0) {
 #pragma unroll
-        for (int c = 0; c < TT / 2; ++c)
-          if (c < nc) part[((size_t)w.sp * (TT / 2) + c) * kWEThreads] = acc[c];
+          for (int c = 0; c < TT / 2; c += 4)
+            if (c < nc)
+              part[(size_t)(c / 4) * kWEThreads] =
+                  make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
+        }
         named_sync(1, kWEThreads);
         if (tid == 0)
           s_last = atom_add_acq_rel_gpu(a.P.tickets + id, 1u) == (uint32_t)(a.nsp - 1);
@@ -343,10 +380,20 @@ __global__ void __launch_bounds__(kWThreads, 1)
         if (tid == 0) a.P.tickets[id] = 0u;
 #pragma unroll
         for (int c = 0; c < TT / 2; ++c) acc[c] = 0.f;
-        for (int s = 0; s < a.nsp; ++s)
+        for (int s = 0; s < nslot; ++s) {
+          float4 u[TT / 8];  // in flight together
 #pragma unroll
-          for (int c = 0; c < TT / 2; ++c)
-            if (c < nc) acc[c] += __ldcg(&part[((size_t)s * (TT / 2) + c) * kWEThreads]);
+          for (int i = 0; i < TT / 8; ++i)
+            u[i] = 4 * i < nc ? __ldcg(&part[((size_t)s * (TT / 8) + i) * kWEThreads])
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int i = 0; i < TT / 8; ++i) {
+            acc[4 * i] += u[i].x;
+            acc[4 * i + 1] += u[i].y;
+            acc[4 * i + 2] += u[i].z;
+            acc[4 * i + 3] += u[i].w;
+          }
+        }
       }
 #pragma unroll
       for (int c = 0; c < TT / 2; c += kWChunk) {
@@ -716,6 +763,15 @@ int stage_cost(int tt) { return 273 + 4 * tt + tt / 4; }
 
 int row_tiles(int N, bool pairs) { return pairs ? (N / 2 + 63) / 64 : (N + kWR - 1) / kWR; }
 
+// Segments of K, by the matrix and the device alone: as many equal groups of
+// them as one token tile's row tiles leave SMs for (at most eight, and no group
+// shorter than kWSeg stages), so that a short prompt's parts come out even, and
+// in a group as few as kWSeg allows.
+int segments(int sms, int nrt, int nks) {
+  const int groups = std::max(1, std::min({8, sms / nrt, nks / kWSeg}));
+  return groups * ((nks + groups * kWSeg - 1) / (groups * kWSeg));
+}
+
 // Token tile (index 0, 1, 2 = 32, 64, 128 tokens) and parts of K of the product
 // of nrt row tiles x nks stages with M tokens that have the least work on the
 // busiest SM.  K is split only where that still leaves every block its own
@@ -727,13 +783,17 @@ struct WPlan {
 };
 WPlan pick_plan(int sms, int nrt, int nks, int M) {
   WPlan best{0, 1, -1};
+  const int nseg = segments(sms, nrt, nks);
   for (int i = 0; i < 3; ++i) {
     const int tt = 32 << i;
     const long long tiles = (long long)nrt * ((M + tt - 1) / tt);
     for (int nsp = 1; nsp <= 8; ++nsp) {
-      if (nsp > 1 && (tiles * nsp > sms || tiles * nsp > kWideParts || nks / nsp < kWSeg)) break;
-      const long long c = (tiles * nsp + sms - 1) / sms * ((nks + nsp - 1) / nsp) * stage_cost(tt) +
-                          (nsp > 1 ? 6000 + 9LL * nsp * tt : 0);
+      if (nsp > 1 && (nsp > nseg || tiles * nsp > sms ||
+                      tiles * w_slots(nseg, nsp) * tt > (long long)kWideParts * 128))
+        break;
+      const int most = nsp > 1 ? (nseg + nsp - 1) / nsp * ((nks + nseg - 1) / nseg) : nks;
+      const long long c = (tiles * nsp + sms - 1) / sms * most * stage_cost(tt) +
+                          (nsp > 1 ? 6000 + 9LL * w_slots(nseg, nsp) * tt : 0);
       if (best.cost < 0 || c < best.cost) best = WPlan{i, nsp, c};
     }
   }
@@ -746,6 +806,9 @@ cudaError_t wide_launch(const CUtensorMap& wm, const CUtensorMap* xm, WArgs& a, 
   a.nrt = row_tiles(a.N, KIND == kWGateUp);
   const WPlan p = pick_plan(a.D.num_sms, a.nrt, a.nks, a.M);
   a.ntt = (a.M + (32 << p.ti) - 1) / (32 << p.ti);
+  a.nseg = segments(a.D.num_sms, a.nrt, a.nks);
+  a.seg_q = a.nks / a.nseg;
+  a.seg_r = a.nks % a.nseg;
   a.nsp = p.nsp;
   const long long tiles = (long long)a.nrt * a.ntt * a.nsp;
   const dim3 grid((unsigned)(tiles < a.D.num_sms ? tiles : a.D.num_sms)), blk(kWThreads);
