@@ -185,19 +185,19 @@ struct Residual {
   __device__ float operator()(int v) const { return fmaxf(p(v) / sp - q(v) / sq, 0.f); }
 };
 
-// Weight sums of the logits rows `sel` (the statistics kernel has left their
-// maxima), one chunk per block; keep >= 0: also stores the row as draft 0
+// Weight sums of the logits rows `sel` from row0 on (the statistics kernel has
+// left their maxima), one chunk per block; keep > 0: also stores the row as draft 0
 // (kKeepWalk) or draft k of the round (kKeepDraft) for the acceptance test.
 enum KeepMode : int { kKeepNone = 0, kKeepWalk = 1, kKeepDraft = 2 };
 __global__ void __launch_bounds__(kSampleThreads)
-    k_row_weights(const Dims D, const Bufs B, RowSel sel, int keep) {
+    k_row_weights(const Dims D, const Bufs B, RowSel sel, int row0, int keep) {
   pdl_wait();
   pdl_launch_dependents();
   __shared__ SampleSmem sm;
   const Ctl* c = B.ctl;
   int pos0, M;
   resolve_rows(c, sel, pos0, M);
-  const int m = blockIdx.y;
+  const int m = row0 + blockIdx.y;
   if (m >= M) return;
   const float* z = B.logits + (size_t)m * D.V;
   const Tempered w{z, B.stats[m].zmax, c->pol.temp};
@@ -887,11 +887,11 @@ cudaError_t launch_accept(const Dims& D, const Bufs& B, cudaGraphConditionalHand
   return launch_ex(k_accept, dim3(1), dim3(kSampleThreads), 0, st, D, B, gen_while);
 }
 
-cudaError_t launch_row_weights(const Dims& D, const Bufs& B, RowSel sel, int mrows, int keep_mode,
-                               cudaStream_t st) {
+cudaError_t launch_row_weights(const Dims& D, const Bufs& B, RowSel sel, int row0, int mrows,
+                               int keep_mode, cudaStream_t st) {
   const int C = samp_chunk(D.V);
-  return launch_ex(k_row_weights, dim3((D.V + C - 1) / C, mrows), dim3(kSampleThreads), 0, st, D, B,
-                   sel, keep_mode);
+  return launch_ex(k_row_weights, dim3((D.V + C - 1) / C, mrows - row0), dim3(kSampleThreads), 0, st,
+                   D, B, sel, row0, keep_mode);
 }
 
 cudaError_t launch_residual_weights(const Dims& D, const Bufs& B, cudaStream_t st) {

@@ -309,7 +309,7 @@ cudaError_t build_walk(ssd_ctx* x, Seq& s, const std::vector<int>& cands, int j,
   if (j == 0) GK(launch_embed(x->D, x->B, x->cfg.dtype, x->embed, x->layers[0].attn_norm, rows(kRowsWalk), false, 0, x->cap));
   GK(enqueue_layers(x, done, cands[j], rows(kRowsWalk), 1, x->cap));
   GK(enqueue_head(x, rows(kRowsWalk), 1, x->topk, x->cap));
-  if (x->sampled) GK(launch_row_weights(x->D, x->B, rows(kRowsWalk), 1, 1, x->cap));
+  if (x->sampled) GK(launch_row_weights(x->D, x->B, rows(kRowsWalk), 0, 1, 1, x->cap));
   GK(launch_decide(x->D, x->B, kDecideWalk, j, last ? 1 : 0, cands[j], x->final_norm,
                    x->cfg.dtype, next, 0, x->cap));
   GK(s.end());
@@ -355,7 +355,7 @@ cudaError_t build_draft_phase(ssd_ctx* x, cudaGraph_t body) {
     GK(enqueue_layers(x, 0, cands[0], rows(kRowsDraft), 1, x->cap));
   }
   GK(enqueue_head(x, rows(kRowsDraft), 1, x->topk, x->cap));
-  if (x->sampled) GK(launch_row_weights(x->D, x->B, rows(kRowsDraft), 1, 2, x->cap));
+  if (x->sampled) GK(launch_row_weights(x->D, x->B, rows(kRowsDraft), 0, 1, 2, x->cap));
   GK(launch_decide(x->D, x->B, kDecideDraft, 0, 0, 0, x->final_norm, x->cfg.dtype, 0, hw,
                    x->cap));
   return w.end();
@@ -382,7 +382,7 @@ cudaError_t build_round(ssd_ctx* x, cudaGraph_t g, cudaGraphConditionalHandle ge
   GK(enqueue_layers(x, 0, x->D.L, rows(kRowsVerify), mrows, x->cap));
   GK(enqueue_head(x, rows(kRowsVerify), mrows, x->topk, x->cap));
   if (x->sampled) {
-    GK(launch_row_weights(x->D, x->B, rows(kRowsVerify), mrows, 0, x->cap));
+    GK(launch_row_weights(x->D, x->B, rows(kRowsVerify), 0, mrows, 0, x->cap));
     if (spec) GK(launch_residual_weights(x->D, x->B, x->cap));
   }
   GK(launch_accept(x->D, x->B, gen, x->cap));
@@ -758,8 +758,8 @@ ssd_status ssd_prefill(ssd_ctx* x, const int32_t* ids, int32_t n, int32_t* first
   ssd_status s = run_prompt(x, n, &last_row);
   if (s) return s;
   if (x->sampled)
-    CK(x, launch_row_weights(x->D, x->B, rows_explicit(0, last_row + 1, nullptr), last_row + 1, 0,
-                             x->stream));
+    CK(x, launch_row_weights(x->D, x->B, rows_explicit(0, last_row + 1, nullptr), last_row,
+                             last_row + 1, 0, x->stream));
   CK(x, launch_set_pending(x->D, x->B, last_row, -1, n, x->stream));
   Ctl c;
   if ((s = read_ctl(x, &c))) return s;

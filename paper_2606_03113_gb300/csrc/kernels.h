@@ -116,10 +116,11 @@ cudaError_t launch_draft_begin(const Bufs& B, cudaGraphConditionalHandle draft_w
                                cudaStream_t st);
 cudaError_t launch_accept(const Dims& D, const Bufs& B, cudaGraphConditionalHandle gen_while,
                           cudaStream_t st);
-// Sampled decoding: weight sums of logits rows (keep_mode 1, 2: also the row as
-// the round's draft 0 or k), then those of the first rejected draft's residual.
-cudaError_t launch_row_weights(const Dims& D, const Bufs& B, RowSel sel, int mrows, int keep_mode,
-                               cudaStream_t st);
+// Sampled decoding: weight sums of the logits rows row0 .. mrows - 1 (keep_mode 1,
+// 2: also the row as the round's draft 0 or k), then those of the first rejected
+// draft's residual.
+cudaError_t launch_row_weights(const Dims& D, const Bufs& B, RowSel sel, int row0, int mrows,
+                               int keep_mode, cudaStream_t st);
 cudaError_t launch_residual_weights(const Dims& D, const Bufs& B, cudaStream_t st);
 cudaError_t launch_begin_call(const Bufs& B, int max_new, cudaStream_t st);
 cudaError_t launch_reset_sequence(const Bufs& B, cudaStream_t st);

@@ -64,6 +64,26 @@ def test_token_of_zero_weight_is_never_drawn():
         eng.close()
 
 
+@pytest.mark.parametrize("n", [1, 5, 16, 17, 40])
+def test_draw_after_the_prompt_reads_its_last_row(n):
+    # the last token's row gives 2048 tokens equal weights, so that u decides; the
+    # rows before it (of opposite sign) would give them none
+    V = 4096
+    z = np.zeros(V)
+    z[V // 2:] = -200.0
+    dm, eng = engine(V, z)
+    try:
+        dm.embed[1:] = -1.0
+        ids = np.array([1] * (n - 1) + [0], dtype=np.int32)
+        for seed in range(4):
+            eng.set_ar(temperature=0.7, sample_seed=seed)
+            t = eng.prefill(ids)
+            u = float(synth.sample_uniforms(seed, n - 1, 2, 1)[0])
+            assert t == int(u * 2048)  # sums of ones up to 2048 are exact in fp32
+    finally:
+        eng.close()
+
+
 @pytest.mark.parametrize("V", [1024, 8192])
 @pytest.mark.parametrize("bad", [np.inf, np.nan])
 def test_rows_without_a_finite_sum_are_refused(V, bad):
