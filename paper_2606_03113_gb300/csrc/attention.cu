@@ -38,40 +38,39 @@ constexpr int kMergeBatch = 40;  // split partials loaded per round of the merge
 constexpr int kMergeBatch4 = 8;  // ... four dimensions each, when merging many rows
 constexpr int kAWarps = kAThreads / 32;
 
-// Stages keys [k0, k1) of the split (relative to s0) into shared memory:
-// all global loads are issued before any is converted.
-template <typename T>
-__device__ __forceinline__ void stage_keys(const T* kb, const T* vb, int hd, int k0, int k1,
+// Stages keys [k0, k1) of the split (relative to s0) into shared memory: the
+// loads of a thread's kUnroll chunks are issued before any is stored.
+__device__ __forceinline__ void stage_keys(const float* kb, const float* vb, int hd, int k0, int k1,
                                            float* Ks, float* Vs) {
-  using E = Elem<T>;
-  constexpr int EPC = E::kPerChunk;
-  const int cpr = hd / EPC;  // 16-byte chunks per key row
+  const int cpr = hd / 4;  // 16-byte chunks per key row
   const int n = (k1 - k0) * cpr;
   constexpr int kUnroll = 4;
   for (int c0 = threadIdx.x; c0 < n; c0 += kAThreads * kUnroll) {
-    uint4 ku[kUnroll], vu[kUnroll];
+    float4 ku[kUnroll], vu[kUnroll];
 #pragma unroll
     for (int j = 0; j < kUnroll; ++j) {
       const int c = c0 + j * kAThreads;
       if (c < n) {
-        const int key = k0 + c / cpr, off = (c % cpr) * EPC;
-        ku[j] = __ldg(reinterpret_cast<const uint4*>(kb + (size_t)key * hd + off));
-        vu[j] = __ldg(reinterpret_cast<const uint4*>(vb + (size_t)key * hd + off));
+        const int key = k0 + c / cpr, off = (c % cpr) * 4;
+        ku[j] = __ldg(reinterpret_cast<const float4*>(kb + (size_t)key * hd + off));
+        vu[j] = __ldg(reinterpret_cast<const float4*>(vb + (size_t)key * hd + off));
       }
     }
 #pragma unroll
     for (int j = 0; j < kUnroll; ++j) {
       const int c = c0 + j * kAThreads;
       if (c < n) {
-        const int key = k0 + c / cpr, off = (c % cpr) * EPC;
-        float kf[EPC], vf[EPC];
-        E::unpack(ku[j], kf);
-        E::unpack(vu[j], vf);
-#pragma unroll
-        for (int e = 0; e < EPC; ++e) {
-          Ks[key * (hd + 1) + off + e] = kf[e];
-          Vs[key * hd + off + e] = vf[e];
-        }
+        const int key = k0 + c / cpr, off = (c % cpr) * 4;
+        float* kr = Ks + key * (hd + 1) + off;
+        kr[0] = ku[j].x;
+        kr[1] = ku[j].y;
+        kr[2] = ku[j].z;
+        kr[3] = ku[j].w;
+        float* vr = Vs + key * hd + off;
+        vr[0] = vu[j].x;
+        vr[1] = vu[j].y;
+        vr[2] = vu[j].z;
+        vr[3] = vu[j].w;
       }
     }
   }
@@ -79,7 +78,6 @@ __device__ __forceinline__ void stage_keys(const T* kb, const T* vb, int hd, int
 
 }  // namespace
 
-template <typename T>
 // Three blocks per SM (the shared memory of a split allows three).
 __global__ void __launch_bounds__(kAThreads, 3) k_attn(Dims D, Bufs B, int layer, RowSel sel) {
   extern __shared__ float sm[];
@@ -93,16 +91,16 @@ __global__ void __launch_bounds__(kAThreads, 3) k_attn(Dims D, Bufs B, int layer
   int* last_rows = reinterpret_cast<int*>(Ps + kAWarps * kAK);  // [kMaxM] rows this block merges
   __shared__ int s_nlast;
 
-  const T* kv = static_cast<const T*>(B.kv) + (size_t)layer * 2 * D.Hkv * D.max_seq * hd;
+  const float* kv = static_cast<const float*>(B.kv) + (size_t)layer * 2 * D.Hkv * D.max_seq * hd;
   const int s0 = split * kAK;
-  const T* kb = kv + ((size_t)g * D.max_seq + s0) * hd;
-  const T* vb = kv + ((size_t)(D.Hkv + g) * D.max_seq + s0) * hd;
+  const float* kb = kv + ((size_t)g * D.max_seq + s0) * hd;
+  const float* vb = kv + ((size_t)(D.Hkv + g) * D.max_seq + s0) * hd;
 
   // keys written by earlier passes: loaded before the wait
   int pos0, M;
   resolve_rows(B.ctl, sel, pos0, M);
   int nold = min(max(min(pos0, D.max_seq) - s0, 0), kAK);  // clamped: never past the cache
-  if (pos0 + M > s0 && nold > 0) stage_keys<T>(kb, vb, hd, 0, nold, Ks, Vs);
+  if (pos0 + M > s0 && nold > 0) stage_keys(kb, vb, hd, 0, nold, Ks, Vs);
   pdl_wait();
   pdl_launch_dependents();
   {
@@ -117,7 +115,7 @@ __global__ void __launch_bounds__(kAThreads, 3) k_attn(Dims D, Bufs B, int layer
   }
   if (s0 > pos0 + M - 1) return;  // beyond every row's causal window
   const int nkeys = min(kAK, pos0 + M - s0);
-  if (nkeys > nold) stage_keys<T>(kb, vb, hd, nold, nkeys, Ks, Vs);
+  if (nkeys > nold) stage_keys(kb, vb, hd, nold, nkeys, Ks, Vs);
   __syncthreads();
 
   // partial attention of every (row, head) pair of the group over this split
@@ -641,8 +639,8 @@ cudaError_t prepare_attention_kernels() {
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
     return e;
-  if ((e = cudaFuncGetAttributes(&fa, k_attn<float>)) != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_attn<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if ((e = cudaFuncGetAttributes(&fa, k_attn)) != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_attn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               most - (int)fa.sharedSizeBytes);
 }
 
@@ -659,7 +657,7 @@ static cudaError_t attn_bf16(const Dims& D, const Bufs& B, int layer, RowSel sel
 
 static cudaError_t attn_f32(const Dims& D, const Bufs& B, int layer, RowSel sel, cudaStream_t st) {
   dim3 grid(D.nsplit, D.Hkv);
-  return launch_ex(k_attn<float>, grid, dim3(kAThreads), attn_smem(D), st, D, B, layer, sel);
+  return launch_ex(k_attn, grid, dim3(kAThreads), attn_smem(D), st, D, B, layer, sel);
 }
 
 cudaError_t launch_attention(const Dims& D, const Bufs& B, int dtype, int layer, RowSel sel,

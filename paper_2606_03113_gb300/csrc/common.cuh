@@ -20,7 +20,6 @@ constexpr int kTraceCap = 64;      // C_trace window capacity
 constexpr int kSampChunks = 256;  // chunk sums of a row's sampling weights, at most
 constexpr int kTopK = 8;           // max k of the token confidence
 constexpr int kAttnKeys = 64;      // keys per attention split (two per lane)
-constexpr int kLayerKernels = 5;   // launches per layer: qkv, attention, o, gate/up, down
 
 // Which rows a kernel works on.  Inside the round graphs they follow the
 // device control block; prefill and the op entry points pass them directly.

@@ -249,23 +249,22 @@ struct Seq {
     if (e_ != cudaSuccess) return e_;           \
   } while (0)
 
-const TileMaps* tile_maps(const ssd_ctx* x) {
-  return x->cfg.dtype == SSD_DTYPE_BF16 ? &x->tmaps : nullptr;
-}
-
-const CUtensorMap* lm_map(const ssd_ctx* x) {
-  return x->cfg.dtype == SSD_DTYPE_BF16 ? &x->wmaps[4 * (size_t)x->cfg.n_layers] : nullptr;
-}
+const CUtensorMap& lm_map(const ssd_ctx* x) { return x->wmaps[4 * (size_t)x->cfg.n_layers]; }
 
 // Norm weights of the matrix behind layer l of a pass that ends at l_to.
 const void* norm_behind(const ssd_ctx* x, int l, int l_to) {
   return l + 1 < l_to ? x->layers[l + 1].attn_norm : x->final_norm;
 }
 
+// One kernel of a layer (0 qkv, 1 attention, 2 o, 3 gate/up, 4 down) on up to
+// mrows rows; the pass ends at layer l_to.
 cudaError_t enqueue_part(ssd_ctx* x, int l, int part, int l_to, RowSel sel, int mrows,
                          cudaStream_t st) {
-  return launch_layer_part(x->D, x->B, x->cfg.dtype, x->layers[l], tile_maps(x), l, part,
-                           norm_behind(x, l, l_to), sel, mrows, st);
+  if (part == 1) return launch_attention(x->D, x->B, x->cfg.dtype, l, sel, mrows, st);
+  if (x->cfg.dtype != SSD_DTYPE_BF16)
+    return launch_f32_part(x->D, x->B, x->layers[l], l, part, sel, mrows, st);
+  return launch_tile_part(x->D, x->B, x->tmaps, x->layers[l], l, part,
+                          norm_behind(x, l, l_to), sel, mrows, st);
 }
 
 // mrows: the most rows the launches will see (1: the single-row kernels).
@@ -282,21 +281,23 @@ cudaError_t enqueue_layers(ssd_ctx* x, int l_from, int l_to, RowSel sel, int mro
     GK(enqueue_part(x, l_from, 0, l_to, sel, mrows, st));
     for (int l = l_from; l < l_to; ++l) {
       GK(enqueue_part(x, l, 1, l_to, sel, mrows, st));
-      GK(launch_tile_chain(x->D, x->B, *tile_maps(x), x->layers[l],
+      GK(launch_tile_chain(x->D, x->B, x->tmaps, x->layers[l],
                            l + 1 < l_to ? &x->layers[l + 1] : nullptr, x->final_norm, l, sel, mrows,
                            st));
     }
     return cudaSuccess;
   }
   for (int l = l_from; l < l_to; ++l)
-    GK(launch_layer(x->D, x->B, x->cfg.dtype, x->layers[l], tile_maps(x), l,
-                    norm_behind(x, l, l_to), sel, mrows, st));
+    for (int part = 0; part < 5; ++part) GK(enqueue_part(x, l, part, l_to, sel, mrows, st));
   return cudaSuccess;
 }
 
 cudaError_t enqueue_head(ssd_ctx* x, RowSel sel, int mrows, int topk, cudaStream_t st) {
-  return launch_head(x->D, x->B, x->cfg.dtype, x->lm_head, lm_map(x), tile_maps(x), x->final_norm,
-                     topk, sel, mrows, st);
+  if (x->cfg.dtype == SSD_DTYPE_BF16)
+    GK(launch_tile_head(x->D, x->B, x->tmaps, lm_map(x), sel, mrows, st));
+  else
+    GK(launch_f32_head(x->D, x->B, x->lm_head, x->final_norm, sel, mrows, st));
+  return launch_head_stats(x->D, x->B, topk, sel, mrows, st);
 }
 
 // Walk segment j: layers (done, c_j], exit head, decision; nested IF for j+1.
@@ -470,7 +471,7 @@ ssd_status run_prompt_wide(ssd_ctx* x, int n, int* last_row) {
                               l + 1 < L ? x->layers[l + 1].attn_norm : x->final_norm, l, M, c0, x->stream));
     for (int r = std::max(0, std::min(n - T, n - 1) - c0); r < M;) {
       const int m = std::min(kHeadRows, M - r);
-      CK(x, launch_head_wide(x->D, x->B, x->P, x->xmaps, *lm_map(x), r, m, x->stream));
+      CK(x, launch_head_wide(x->D, x->B, x->P, x->xmaps, lm_map(x), r, m, x->stream));
       CK(x, launch_head_stats(x->D, x->B, x->topk, rows_explicit(c0 + r, m, nullptr), m, x->stream));
       CK(x, launch_trace_push(x->B, 0, m, x->stream));
       *last_row = m - 1;
@@ -1049,7 +1050,7 @@ ssd_status ssd_op_layer(ssd_ctx* x, int32_t kernel, int32_t layer, int32_t M, in
   if (kernel == 5)
     CK(x, enqueue_head(x, sel, M, x->topk, st));
   else if (kernel == 6)
-    CK(x, launch_tile_chain(x->D, x->B, *tile_maps(x), x->layers[layer],
+    CK(x, launch_tile_chain(x->D, x->B, x->tmaps, x->layers[layer],
                             layer + 1 < x->cfg.n_layers ? &x->layers[layer + 1] : nullptr,
                             x->final_norm, layer, sel, M, st));
   else

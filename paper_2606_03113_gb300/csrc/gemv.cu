@@ -480,42 +480,6 @@ cudaError_t prepare_gemv_kernels() {
   return prepare_one<__nv_bfloat16, kMaxM>();
 }
 
-// Attention launchers live in attention.cu.
-cudaError_t launch_attention(const Dims& D, const Bufs& B, int dtype, int layer, RowSel sel,
-                             int mrows, cudaStream_t st);
-
-cudaError_t launch_layer_part(const Dims& D, const Bufs& B, int dtype, const LayerW& w,
-                              const TileMaps* tm, int layer, int part, const void* next_norm,
-                              RowSel sel, int mrows, cudaStream_t st) {
-  if (part == 1) return launch_attention(D, B, dtype, layer, sel, mrows, st);
-  if (dtype != SSD_DTYPE_BF16) return launch_f32_part(D, B, w, layer, part, sel, mrows, st);
-  if (!tm) return cudaErrorInvalidValue;
-  return launch_tile_part(D, B, *tm, w, layer, part, next_norm, sel, mrows, st);
-}
-
-cudaError_t launch_layer(const Dims& D, const Bufs& B, int dtype, const LayerW& w,
-                         const TileMaps* tm, int layer, const void* next_norm, RowSel sel,
-                         int mrows, cudaStream_t st) {
-  for (int part = 0; part < 5; ++part) {  // qkv, attention, o, gate/up, down
-    cudaError_t e = launch_layer_part(D, B, dtype, w, tm, layer, part, next_norm, sel, mrows, st);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-cudaError_t launch_head(const Dims& D, const Bufs& B, int dtype, const void* lm_head,
-                        const CUtensorMap* lm_map, const TileMaps* tm, const void* final_norm,
-                        int topk, RowSel sel, int mrows, cudaStream_t st) {
-  cudaError_t e;
-  if (dtype == SSD_DTYPE_BF16) {
-    if (!tm || !lm_map) return cudaErrorInvalidValue;
-    e = launch_tile_head(D, B, *tm, *lm_map, sel, mrows, st);
-  } else {
-    e = launch_f32_head(D, B, lm_head, final_norm, sel, mrows, st);
-  }
-  return e != cudaSuccess ? e : launch_head_stats(D, B, topk, sel, mrows, st);
-}
-
 template <typename T, int MM>
 static cudaError_t plain_t(const Dims& D, const Bufs& B, const void* W, int rows, int cols,
                            const float* x, int M, float* y, cudaStream_t st) {

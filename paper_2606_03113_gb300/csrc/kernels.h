@@ -83,24 +83,16 @@ cudaError_t launch_f32_part(const Dims& D, const Bufs& B, const LayerW& w, int l
 cudaError_t launch_f32_head(const Dims& D, const Bufs& B, const void* lm, const void* final_norm,
                               RowSel sel, int mrows, cudaStream_t st);
 
-// mrows is the largest number of rows a launch may see: 1 selects the
-// single-row kernels, more the multi-row ones (bf16: the tensor-core instance
-// with 8, 16 or 24 token rows, the smallest that holds mrows).  big
-// (embedding, attention) is mrows > 1.
-// gnorm: norm weights of the first layer.
+// mrows is the largest number of rows a launch may see.  It picks the instance:
+// fp32 matrices 1, 8 or 17 input rows, bf16 products 8, 16 or 24 token rows
+// (the smallest that holds mrows), bf16 attention the row groups of a block.
+// gnorm: norm weights of the first layer.  big: a block for each of kMaxM rows,
+// else for one.
 cudaError_t launch_embed(const Dims& D, const Bufs& B, int dtype, const void* embed,
-                         const void* gnorm, RowSel sel, bool big, cudaGraphConditionalHandle set_lstar_switch, cudaStream_t st);
-// next_norm: norm weights of the matrix behind the layer.
-cudaError_t launch_layer(const Dims& D, const Bufs& B, int dtype, const LayerW& w,
-                         const TileMaps* tm, int layer, const void* next_norm, RowSel sel,
-                         int mrows, cudaStream_t st);
-// One kernel of a layer (0 qkv, 1 attention + combine, 2 o, 3 gate/up, 4 down).
-cudaError_t launch_layer_part(const Dims& D, const Bufs& B, int dtype, const LayerW& w,
-                              const TileMaps* tm, int layer, int part, const void* next_norm,
-                              RowSel sel, int mrows, cudaStream_t st);
-cudaError_t launch_head(const Dims& D, const Bufs& B, int dtype, const void* lm_head,
-                        const CUtensorMap* lm_map, const TileMaps* tm, const void* final_norm,
-                        int topk, RowSel sel, int mrows, cudaStream_t st);
+                         const void* gnorm, RowSel sel, bool big,
+                         cudaGraphConditionalHandle set_lstar_switch, cudaStream_t st);
+cudaError_t launch_attention(const Dims& D, const Bufs& B, int dtype, int layer, RowSel sel,
+                             int mrows, cudaStream_t st);
 cudaError_t launch_head_stats(const Dims& D, const Bufs& B, int topk, RowSel sel, int mrows,
                               cudaStream_t st);
 cudaError_t prepare_attention_kernels();

@@ -679,7 +679,6 @@ constexpr int kCThreads = (kWorkers + 3) * 32;
 
 struct ChainArgs {
   TArgs ph[4];
-  int nph;
   uint32_t* bar;  // [0] arrivals of finished phases, [1] blocks done (self-resetting)
 };
 
@@ -1065,16 +1064,14 @@ cudaError_t launch_tile_chain(const Dims& D, const Bufs& B, const TileMaps& tm, 
   ca.ph[2].gout = static_cast<const __nv_bfloat16*>(next ? next->attn_norm : final_norm);
   cm.w[2] = *w.tm[3];
   cm.x[2] = tm.act[tp];
-  ca.nph = 3;
   if (next) {  // the next layer's RMSNorm + QKV + RoPE + KV append
     ca.ph[3].g = make_tgeom(D, (D.Hq + 2 * D.Hkv) * D.hd, D.d, kTMapQKV);
     ca.ph[3].ss_in = 0;
     ca.ph[3].layer = layer + 1;
     cm.w[3] = *next->tm[0];
     cm.x[3] = tm.h[tp];
-    ca.nph = 4;
   }
-  for (int p = 0; p < ca.nph; ++p)
+  for (int p = 0; p < (next ? 4 : 3); ++p)
     if (ca.ph[p].g.T < 1 || ca.ph[p].g.T > (1 << 22) || ca.ph[p].g.P < 1 ||
         ca.ph[p].g.P > kMaxBlocksDev)
       return cudaErrorInvalidValue;
