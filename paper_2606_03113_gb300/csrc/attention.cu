@@ -629,17 +629,18 @@ static size_t rows_smem(int keys, int groups) {
 // The limits of dynamic shared memory, once and the same for every context: a
 // function's attributes are shared by all threads, and a launch's own size
 // depends on the model and on the number of rows.
-cudaError_t prepare_attention_kernels() {
-  cudaError_t e = cudaFuncSetAttribute(k_attn_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)rows_smem(2 * kRStep, kRMaxGroups));
-  if (e != cudaSuccess) return e;
-  // fp32: what the device has (the merge of a long cache takes more than a split's keys)
+cudaError_t prepare_attention_kernels(int dtype) {
+  if (dtype == SSD_DTYPE_BF16)
+    return cudaFuncSetAttribute(k_attn_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)rows_smem(2 * kRStep, kRMaxGroups));
+  // what the device has: the merge of a long cache takes more than a split's keys
   int dev = 0, most = 0;
   cudaFuncAttributes fa;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncGetAttributes(&fa, k_attn)) != cudaSuccess) return e;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_attn);
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_attn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               most - (int)fa.sharedSizeBytes);
 }

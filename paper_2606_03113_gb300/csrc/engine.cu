@@ -562,7 +562,7 @@ ssd_status ssd_init_model(const ssd_model_cfg* cfg, const ssd_weights* w, void* 
   cudaError_t e0 = cudaGetDevice(&dev);
   if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e0 == cudaSuccess) e0 = prepare_gemv_kernels();
-  if (e0 == cudaSuccess) e0 = prepare_attention_kernels();
+  if (e0 == cudaSuccess) e0 = prepare_attention_kernels(cfg->dtype);
   if (e0 == cudaSuccess && cfg->dtype == SSD_DTYPE_BF16) e0 = prepare_tile_kernels();
   if (e0 == cudaSuccess && cfg->dtype == SSD_DTYPE_BF16) e0 = prepare_wide_kernels();
   if (e0 != cudaSuccess) return cuda_fail(nullptr, "ssd_init_model device query", e0);

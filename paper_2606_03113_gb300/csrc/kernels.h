@@ -95,7 +95,7 @@ cudaError_t launch_attention(const Dims& D, const Bufs& B, int dtype, int layer,
                              int mrows, cudaStream_t st);
 cudaError_t launch_head_stats(const Dims& D, const Bufs& B, int topk, RowSel sel, int mrows,
                               cudaStream_t st);
-cudaError_t prepare_attention_kernels();
+cudaError_t prepare_attention_kernels(int dtype);
 // Keys per split of the bf16 decode attention.
 int attn_split_keys(int n_kv_heads, int max_seq, int sms);
 cudaError_t launch_round_begin(const Dims& D, const Bufs& B, cudaGraphConditionalHandle draft_if,
