@@ -200,7 +200,7 @@ struct Bufs {
   int32_t* pre_tok;  // [max_seq] prefill / teacher-forced token ids
 };
 
-constexpr int kWideParts = 512;  // partial sums of tiles that blocks share, in one launch
+constexpr int kWideParts = 256;  // partial sums of tiles that blocks share, in one launch
 
 // Buffers of a prompt chunk (bf16 models, wide.cu): up to cap rows.  The
 // inputs of the products are kept as bf16 high and low planes.

@@ -12,11 +12,10 @@
 // norm's scale is applied to the product (per-tile sums of squares travel
 // beside the rows).
 //  - a product with fewer tiles than SMs (a short prompt's O and down) splits K
-//    over up to eight blocks per tile, whose last one adds their sums.  The
-//    segments of K that are added, and their order, depend on the matrix alone,
-//    so a row's bits do not depend on the length of the prompt.  (Parts that add
-//    their own segments first leave less to join, down of the 8B shape with 89
-//    rows 41.5 us against 48.4, but then the order follows the split.)
+//    over up to eight blocks per tile, whose last one adds their sums.  How K
+//    is cut into groups and segments, and the order of their sums, depends on the
+//    matrix and the device alone, so a row's bits do not depend on the length of
+//    the prompt;
 //  - persistent grid, tiles dealt round robin with the token tiles of one
 //    weight tile next to each other (they share it in L2);
 //  - warp roles (320 threads): a TMA warp fills a ring of 64-column stages
@@ -74,6 +73,11 @@ constexpr int kWChunk = 16;           // tokens per epilogue step of a warp
 constexpr int kWSeg = 16;
 
 enum WKind : int { kWQkv = 0, kWResid = 1, kWGateUp = 2, kWHead = 3 };
+// O and down are the products that short prompts split most and over the longest
+// K: their segments are added in groups first, so that a split leaves few sums to
+// join (down of the 8B shape, 89 rows: 4 a tile instead of 13, 41.5 us against
+// 48.4; a second accumulator costs the others 1 % of a long prompt).
+constexpr bool w_grouped(int kind) { return kind == kWResid; }
 
 template <int TT>
 struct WL {
@@ -97,7 +101,8 @@ struct WArgs {
   Bufs B;
   WideBufs P;
   int N, K, nks, nrt, ntt;     // rows, columns, stages, row tiles, token tiles
-  int nseg, seg_q, seg_r;      // segments of K; stages of each, and the first ones that have one more
+  int ngrp, spg;               // groups of K, segments of a group (1 but for grouped kinds)
+  int seg_q, seg_r;            // stages of a segment; the first seg_r have one more
   int nsp;                     // parts that K is split into (blocks that share a tile)
   int M, pos0, layer;
   int row0;                    // first of the M input rows
@@ -111,7 +116,7 @@ __device__ __forceinline__ int w_seg_start(const WArgs& a, int g) {
   return g * a.seg_q + min(g, a.seg_r);
 }
 
-// Work item `it`: row tile, token tile and part of K (segments g0 .. g1 - 1,
+// Work item `it`: row tile, token tile and part of K (groups g0 .. g1 - 1,
 // stages k0 .. k0 + n - 1).
 struct WItem {
   int rt, tt, sp, g0, g1, k0, n;
@@ -120,17 +125,16 @@ struct WItem {
     const int r = it / a.ntt;
     sp = r % a.nsp;
     rt = r / a.nsp;
-    g0 = a.nseg * sp / a.nsp;
-    g1 = a.nseg * (sp + 1) / a.nsp;
-    k0 = w_seg_start(a, g0);
-    n = w_seg_start(a, g1) - k0;
+    g0 = a.ngrp * sp / a.nsp;
+    g1 = a.ngrp * (sp + 1) / a.nsp;
+    k0 = w_seg_start(a, g0 * a.spg);
+    n = w_seg_start(a, g1 * a.spg) - k0;
   }
 };
 
-// Partial sums that the parts of a tile leave: one of the first part's
-// segments, which are the first terms of the sum over K, and one of each
-// later segment.
-__host__ __device__ inline int w_slots(int nseg, int nsp) { return nseg - nseg / nsp + 1; }
+// Partial sums that the parts of a tile leave: one of the first part, whose
+// groups are the first terms of the sum over K, and one of each later group.
+__host__ __device__ inline int w_slots(int ngrp, int nsp) { return ngrp - ngrp / nsp + 1; }
 
 __device__ __forceinline__ void w_flag(const Bufs& B) { atomicOr(&B.ctl->err, (int)kErrTimeout); }
 
@@ -143,8 +147,25 @@ __device__ __forceinline__ void tma_load_2d_plain(void* dst, const CUtensorMap* 
       : "memory");
 }
 
-// 16 columns of the warp's TMEM lanes from two places (high and low parts), added.
-__device__ __forceinline__ void tc_ld16_sum(uint32_t hi, uint32_t lo, float (&v)[16]) {
+// 8 or 16 columns of the warp's TMEM lanes from two places (high and low parts),
+// added.
+__device__ __forceinline__ void tc_ld_sum(uint32_t hi, uint32_t lo, float (&v)[8]) {
+  uint32_t a[8], b[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]),
+                 "=r"(a[7])
+               : "r"(hi)
+               : "memory");
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]),
+                 "=r"(b[7])
+               : "r"(lo)
+               : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(a[i]) + __uint_as_float(b[i]);
+}
+__device__ __forceinline__ void tc_ld_sum(uint32_t hi, uint32_t lo, float (&v)[16]) {
   uint32_t a[16], b[16];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
@@ -273,7 +294,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
       uint32_t ph = 0;
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
         const WItem w(a, tile);
-        int g = w.g0, seg_end = w_seg_start(a, g + 1);
+        int sg = w.g0 * a.spg, seg_end = w_seg_start(a, sg + 1);
         bool first = true;
         for (int kc = w.k0; kc < w.k0 + w.n; ++kc) {
           if (first && !(ok = mbar_wait(&accempty[sc & 1], ((uint32_t)(sc >> 1) & 1u) ^ 1u))) break;
@@ -290,7 +311,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
           first = kc + 1 == seg_end;
           if (first) {
             tc_commit(&accfull[sc++ & 1]);
-            seg_end = w_seg_start(a, ++g + 1);
+            seg_end = w_seg_start(a, ++sg + 1);
           }
           if (++slot == NS) {
             slot = 0;
@@ -328,49 +349,70 @@ __global__ void __launch_bounds__(kWThreads, 1)
         }
         named_sync(1, kWEThreads);
       }
-      // the tile's sums: segments added in K order, high plus low parts; a later
-      // part of a split K hands its segments on one by one, so that the order
-      // is the same whatever the split
-      const int id = rt * a.ntt + w.tt, nslot = w_slots(a.nseg, a.nsp), first_later = a.nseg / a.nsp;
+      // the tile's sums: the segments (high plus low parts) of a group added in
+      // K order, then the groups.  A later part of a split K hands its groups on
+      // one by one, so the order is the same whatever the split.
+      constexpr bool kGrp = w_grouped(KIND);
+      const int id = rt * a.ntt + w.tt, nslot = w_slots(a.ngrp, a.nsp), later = a.ngrp / a.nsp;
+      const int nc = min(TT / 2, (a.M - t0 - th * (TT / 2) + kWChunk - 1) / kWChunk * kWChunk);
       float4* part = reinterpret_cast<float4*>(a.P.part) + (size_t)id * nslot * (TT * 32) + tid;
-      float acc[TT / 2];
+      auto hand_on = [&](int slot, int c, const float* v) {  // columns c .. c + 3
+        part[((size_t)slot * (TT / 8) + c / 4) * kWEThreads] = make_float4(v[0], v[1], v[2], v[3]);
+      };
+      float tot[TT / 2];
 #pragma unroll
-      for (int c = 0; c < TT / 2; ++c) acc[c] = 0.f;
-      for (int g = w.g0; g < w.g1; ++g, ++sc) {
-        if (ok) {
-          ok = __all_sync(0xffffffffu, mbar_wait(&accfull[sc & 1], (uint32_t)(sc >> 1) & 1u));
-          if (!ok && lane == 0) w_flag(a.B);
+      for (int c = 0; c < TT / 2; ++c) tot[c] = 0.f;
+      for (int g = w.g0; g < w.g1; ++g) {
+        float acc[kGrp ? TT / 2 : 1];
+        if constexpr (kGrp) {
+#pragma unroll
+          for (int c = 0; c < TT / 2; ++c) acc[c] = 0.f;
         }
-        tc_fence_after();
-        const uint32_t src = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((sc & 1) * N + th * (TT / 2));
-#pragma unroll
-        for (int c = 0; c < TT / 2; c += kWChunk)
-          if (ok && t0 + th * (TT / 2) + c < a.M) {
-            float v[kWChunk];
-            tc_ld16_sum(src + c, src + TT + c, v);
-            if (w.sp == 0) {
-#pragma unroll
-              for (int j = 0; j < kWChunk; ++j) acc[c + j] += v[j];
-            } else {
-              float4* to = part + ((size_t)(g - first_later + 1) * (TT / 8) + c / 4) * kWEThreads;
-#pragma unroll
-              for (int j = 0; j < kWChunk; j += 4)
-                to[(size_t)(j / 4) * kWEThreads] = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-            }
+        for (int i = 0; i < (kGrp ? a.spg : 1); ++i, ++sc) {
+          if (ok) {
+            ok = __all_sync(0xffffffffu, mbar_wait(&accfull[sc & 1], (uint32_t)(sc >> 1) & 1u));
+            if (!ok && lane == 0) w_flag(a.B);
           }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&accempty[sc & 1]);
+          tc_fence_after();
+          const uint32_t src =
+              tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)((sc & 1) * N + th * (TT / 2));
+          constexpr int kDrain = kGrp ? 8 : 16;  // (16 with two accumulators would spill)
+#pragma unroll
+          for (int c = 0; c < TT / 2; c += kDrain)
+            if (ok && c < nc) {
+              float v[kDrain];
+              tc_ld_sum(src + c, src + TT + c, v);
+              if constexpr (kGrp) {
+#pragma unroll
+                for (int j = 0; j < kDrain; ++j) acc[c + j] += v[j];
+              } else if (w.sp == 0) {
+#pragma unroll
+                for (int j = 0; j < kDrain; ++j) tot[c + j] += v[j];
+              } else {
+#pragma unroll
+                for (int j = 0; j < kDrain; j += 4) hand_on(g - later + 1, c + j, v + j);
+              }
+            }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&accempty[sc & 1]);
+        }
+        if constexpr (kGrp) {
+#pragma unroll
+          for (int c = 0; c < TT / 2; ++c) tot[c] += acc[c];
+          if (w.sp > 0) {
+#pragma unroll
+            for (int c = 0; c < TT / 2; c += 4)
+              if (c < nc) hand_on(g - later + 1, c, acc + c);
+          }
+        }
       }
       if (a.nsp > 1) {
         // K is split: the last block of the tile adds the partial sums in K order
-        const int nc = min(TT / 2, (a.M - t0 - th * (TT / 2) + kWChunk - 1) / kWChunk * kWChunk);
         if (w.sp == 0) {
 #pragma unroll
           for (int c = 0; c < TT / 2; c += 4)
-            if (c < nc)
-              part[(size_t)(c / 4) * kWEThreads] =
-                  make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
+            if (c < nc) hand_on(0, c, tot + c);
         }
         named_sync(1, kWEThreads);
         if (tid == 0)
@@ -379,7 +421,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
         if (!s_last) continue;
         if (tid == 0) a.P.tickets[id] = 0u;
 #pragma unroll
-        for (int c = 0; c < TT / 2; ++c) acc[c] = 0.f;
+        for (int c = 0; c < TT / 2; ++c) tot[c] = 0.f;
         for (int s = 0; s < nslot; ++s) {
           float4 u[TT / 8];  // in flight together
 #pragma unroll
@@ -388,10 +430,10 @@ __global__ void __launch_bounds__(kWThreads, 1)
                               : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
           for (int i = 0; i < TT / 8; ++i) {
-            acc[4 * i] += u[i].x;
-            acc[4 * i + 1] += u[i].y;
-            acc[4 * i + 2] += u[i].z;
-            acc[4 * i + 3] += u[i].w;
+            tot[4 * i] += u[i].x;
+            tot[4 * i + 1] += u[i].y;
+            tot[4 * i + 2] += u[i].z;
+            tot[4 * i + 3] += u[i].w;
           }
         }
       }
@@ -401,7 +443,7 @@ __global__ void __launch_bounds__(kWThreads, 1)
         if (t0 + tl >= a.M) break;
         float v[kWChunk];
 #pragma unroll
-        for (int j = 0; j < kWChunk; ++j) v[j] = acc[c + j];
+        for (int j = 0; j < kWChunk; ++j) v[j] = tot[c + j];
         const int nt = min(kWChunk, a.M - t0 - tl);
         if constexpr (KIND == kWResid) {
           const int row = rt * kWR + 32 * q + lane;
@@ -763,13 +805,18 @@ int stage_cost(int tt) { return 273 + 4 * tt + tt / 4; }
 
 int row_tiles(int N, bool pairs) { return pairs ? (N / 2 + 63) / 64 : (N + kWR - 1) / kWR; }
 
-// Segments of K, by the matrix and the device alone: as many equal groups of
-// them as one token tile's row tiles leave SMs for (at most eight, and no group
-// shorter than kWSeg stages), so that a short prompt's parts come out even, and
-// in a group as few as kWSeg allows.
-int segments(int sms, int nrt, int nks) {
+// How K is cut, by the matrix and the device alone: into as many equal groups as
+// one token tile's row tiles leave SMs for (at most eight, none shorter than
+// kWSeg stages), which are the parts of a short prompt, and a group into as few
+// segments as kWSeg allows.  Where segments are not added in groups each is a
+// group of its own.
+struct KCut {
+  int ngrp, spg;
+};
+KCut cut_k(int sms, int nrt, int nks, bool grouped) {
   const int groups = std::max(1, std::min({8, sms / nrt, nks / kWSeg}));
-  return groups * ((nks + groups * kWSeg - 1) / (groups * kWSeg));
+  const int spg = (nks + groups * kWSeg - 1) / (groups * kWSeg);
+  return grouped ? KCut{groups, spg} : KCut{groups * spg, 1};
 }
 
 // Token tile (index 0, 1, 2 = 32, 64, 128 tokens) and parts of K of the product
@@ -781,19 +828,19 @@ struct WPlan {
   int ti, nsp;
   long long cost;
 };
-WPlan pick_plan(int sms, int nrt, int nks, int M) {
+WPlan pick_plan(int sms, int nrt, int nks, int M, bool grouped) {
   WPlan best{0, 1, -1};
-  const int nseg = segments(sms, nrt, nks);
+  const int groups = cut_k(sms, nrt, nks, grouped).ngrp;
   for (int i = 0; i < 3; ++i) {
     const int tt = 32 << i;
     const long long tiles = (long long)nrt * ((M + tt - 1) / tt);
     for (int nsp = 1; nsp <= 8; ++nsp) {
-      if (nsp > 1 && (nsp > nseg || tiles * nsp > sms ||
-                      tiles * w_slots(nseg, nsp) * tt > (long long)kWideParts * 128))
+      if (nsp > 1 && (nsp > groups || tiles * nsp > sms ||
+                      tiles * w_slots(groups, nsp) * tt > (long long)kWideParts * 128))
         break;
-      const int most = nsp > 1 ? (nseg + nsp - 1) / nsp * ((nks + nseg - 1) / nseg) : nks;
+      const int most = ((groups + nsp - 1) / nsp * nks + groups - 1) / groups;
       const long long c = (tiles * nsp + sms - 1) / sms * most * stage_cost(tt) +
-                          (nsp > 1 ? 6000 + 9LL * w_slots(nseg, nsp) * tt : 0);
+                          (nsp > 1 ? 6000 + 9LL * w_slots(groups, nsp) * tt : 0);
       if (best.cost < 0 || c < best.cost) best = WPlan{i, nsp, c};
     }
   }
@@ -804,11 +851,13 @@ template <int KIND>
 cudaError_t wide_launch(const CUtensorMap& wm, const CUtensorMap* xm, WArgs& a, cudaStream_t st) {
   a.nks = (a.K + kWK - 1) / kWK;
   a.nrt = row_tiles(a.N, KIND == kWGateUp);
-  const WPlan p = pick_plan(a.D.num_sms, a.nrt, a.nks, a.M);
+  const WPlan p = pick_plan(a.D.num_sms, a.nrt, a.nks, a.M, w_grouped(KIND));
+  const KCut cut = cut_k(a.D.num_sms, a.nrt, a.nks, w_grouped(KIND));
   a.ntt = (a.M + (32 << p.ti) - 1) / (32 << p.ti);
-  a.nseg = segments(a.D.num_sms, a.nrt, a.nks);
-  a.seg_q = a.nks / a.nseg;
-  a.seg_r = a.nks % a.nseg;
+  a.ngrp = cut.ngrp;
+  a.spg = cut.spg;
+  a.seg_q = a.nks / (a.ngrp * a.spg);
+  a.seg_r = a.nks % (a.ngrp * a.spg);
   a.nsp = p.nsp;
   const long long tiles = (long long)a.nrt * a.ntt * a.nsp;
   const dim3 grid((unsigned)(tiles < a.D.num_sms ? tiles : a.D.num_sms)), blk(kWThreads);
@@ -838,11 +887,11 @@ cudaError_t prepare_wide_kernels() {
 
 // Work of one layer of a chunk of M rows on the busiest SM (stage cycles).
 long long wide_layer_cost(const Dims& D, int M) {
-  auto mat = [&](int N, int K, bool pairs) {
-    return pick_plan(D.num_sms, row_tiles(N, pairs), (K + kWK - 1) / kWK, M).cost;
+  auto mat = [&](int kind, int N, int K) {
+    return pick_plan(D.num_sms, row_tiles(N, kind == kWGateUp), (K + kWK - 1) / kWK, M, w_grouped(kind)).cost;
   };
-  return mat((D.Hq + 2 * D.Hkv) * D.hd, D.d, false) + mat(D.d, D.qd, false) +
-         mat(2 * D.F, D.d, true) + mat(D.d, D.F, false);
+  return mat(kWQkv, (D.Hq + 2 * D.Hkv) * D.hd, D.d) + mat(kWResid, D.d, D.qd) +
+         mat(kWGateUp, 2 * D.F, D.d) + mat(kWResid, D.d, D.F);
 }
 
 cudaError_t launch_embed_wide(const Dims& D, const Bufs& B, const WideBufs& P, const void* embed,
