@@ -613,10 +613,18 @@ __global__ void __launch_bounds__(256) k_attn_merge(const Dims D, const Bufs B, 
 
 // Keys per split of the bf16 kernel: 64, or 128 where 64 would make more blocks
 // than three per SM with a full cache: fewer partials to store and merge, for
-// two key steps in a row.  Live with the merge, one row, a cache of 2304
-// positions, 128 against 64 keys: 32 KV heads at context 640 9.5 against 10.3
-// us, at 2048 17.7 against 18.6; 40 KV heads at 1000 12.4 both, at 2176 22.3
-// against 21.2.
+// two key steps in a row.  One value for a model's whole cache, since a row's
+// sums have to be the same in drafting and in verification.  Live with the merge,
+// a cache of 2304 positions, us a layer for 1 / 17 rows with 128 and 64 keys:
+//   context             100                     1000                    2176
+//   32 KV heads   7.5/10.3, 7.0/9.4       9.2/13.1, 10.6/16.2    17.1/23.1, 18.2/27.9
+//   40 KV heads   7.8/10.9, 7.2/10.1     11.3/16.4, 12.0/18.9    21.2/28.5, 20.3/32.8
+//    8 (of 64)    6.2/20.5, 6.0/15.4      6.4/21.3,  7.3/18.7     8.8/24.5, 10.7/33.3
+// So 128 loses 5 to 10 % at the beginning of a long cache and 4 % for one row
+// of 40 heads behind 2048 positions, and wins up to 20 % elsewhere.  With few
+// KV heads (the last line, which the rule gives 64) a wide verification is a
+// third faster with 64 up to some 640 positions and as much slower from 1500
+// on; there the rule keeps the shorter contexts' choice.
 int attn_split_keys(int n_kv_heads, int max_seq, int sms) {
   const int n = (max_seq + kRStep - 1) / kRStep;
   return n_kv_heads * n > 3 * sms ? 2 * kRStep : kRStep;

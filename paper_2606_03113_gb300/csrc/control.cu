@@ -31,10 +31,10 @@ __device__ float trace_conf(const Ctl* c, int T) {
 // P(v) = exp((z_v - max z) / T) / sum_w exp((z_w - max z) / T).
 // k_row_weights reads the rows' logits on all SMs and leaves the weights' sums
 // over at most kSampChunks runs of the vocabulary; a draw then scans those
-// sums and walks the one run that holds it.  One block used to read whole
-// rows, each thread a run of its own: 48 sampled tokens of the 8B widths (4
-// layers, 128256 tokens) took 43.8 ms, now 25.3 (the bf16 decode attention
-// changed in between, about 2 of the 18.5 ms).
+// sums and walks the one run that holds it.  When one block read whole rows,
+// each thread a run of its own, 48 sampled tokens of the 8B widths (4 layers,
+// 128256 tokens) took 43.8 ms; this took them to 25.3 (about 2 of the 18.5 ms
+// came from the bf16 decode attention).
 // Every reduction below runs in a fixed order that depends on the vocabulary
 // alone, so a draw depends only on the logits and the uniform, never on
 // scheduling.

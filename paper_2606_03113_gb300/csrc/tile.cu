@@ -13,10 +13,10 @@
 //  - the input rows come as bf16 high and low parts (x = hi + lo to ~16
 //    significant bits), written by the kernel that produced them and already
 //    multiplied by the RMSNorm weights of the product that reads them: one TMA
-//    box is a unit's operand tile.  (When the workers split fp32 slices in
-//    shared memory, one more hand-over per unit and at each phase's start, the
-//    single-row chained launch took 98.5 us on the Llama-2-7B shape, now 90.1,
-//    and 131.7 on the 13B shape, now 120.0.)
+//    box is a unit's operand tile.  (Before, the workers split fp32 slices in
+//    shared memory, one more hand-over per unit and at each phase's start; this
+//    took the single-row chained launch from 98.5 to 90.1 us on the Llama-2-7B
+//    shape and from 131.7 to 120.0 on the 13B shape.)
 //  - warp roles (320 threads): a TMA warp fills a 5- or 6-deep ring with the
 //    unit's weight boxes and its input box; one MMA warp issues tcgen05.mma (M
 //    = 128 rows per half, N = 16, 32 or 48 token columns, K = 16) for both

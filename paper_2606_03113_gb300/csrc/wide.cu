@@ -27,19 +27,19 @@
 //    TMEM lanes of different warps: they swap halves through shared memory.
 // Bound by the tensor cores and by the copies out of L2 (48 KB per stage of
 // a 128-token tile in 512 cycles of tcgen05.mma at full rate).  512 rows of
-// the Llama-2-7B shape: gate/up 126.6 us (1.46 PFLOP/s with both parts), QKV
-// 83.7, down 75.0, O 35.3 us; a 512-token prompt through four layers takes
-// 1.9 ms against 18.0 ms in 32 passes of 16 rows, 2043 tokens of the 13B
-// shape 9.6 ms against 104.6 ms.  The exit head of a prompt's last rows (20 of
-// them feed the C_trace window) is such a product too, one pass over the LM
-// head instead of one per 16 rows: a 93-token prompt of the 8B widths (4
-// layers, 128256 tokens) takes 1912 us against 2188, 512 tokens of the 7B
-// widths 2281 against 2371.
+// the Llama-2-7B shape: gate/up 122 us (1.51 PFLOP/s with both parts), QKV 84,
+// down 75, O 38 us.  In passes of 16 rows through the decode kernels a 508-token
+// prompt through four layers and its last rows' logits took 18.8 ms, in chunks
+// 2.2 ms; 2043 tokens of the 13B shape 105 ms and 9.8 ms.  The exit head of a
+// prompt's last rows (20 of them feed the C_trace window) is such a product
+// too, one pass over the LM head instead of one per 16 rows: that took a
+// 93-token prompt of the 8B widths (4 layers, 128256 tokens) from 2188 to 1912
+// us, splitting K then to 1740.
 // Attention (k_attn_wide): 64 query rows x one head per block, 64-key steps
 // with a running maximum; scores and outputs on mma.sync with the fp32
 // operand (queries, probabilities) in three bf16 parts, 24 bits, so nothing
 // is rounded below fp32.  Bound by mma.sync: 512 rows of the Llama-2-7B shape
-// take 41 us a layer, rows 1024-1919 of the 13B shape 252 us (328 TFLOP/s with
+// take 42 us a layer, rows 1024-1919 of the 13B shape 252 us (328 TFLOP/s with
 // the three parts).
 #include <math.h>
 
