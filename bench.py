@@ -281,8 +281,9 @@ KERNEL_NAMES = {0: "k_qkv", 1: "k_attn", 2: "k_resid(wo)", 3: "k_gate_up",
 
 def kernel_roofline(eng, w, peak: float, pos0: int, iters: int = 5, graphs: bool = True) -> dict:
     """Live CUDA-event timing, on the engine's stream where the kernels are
-    launched, of each hot-path kernel of a single-row pass: one launch per
-    layer over all layers (so a launch never finds its weights in L2),
+    launched, of each hot-path kernel of a single-row pass (launched on their
+    own, QKV, gate/up and the head of a bf16 model come with the short kernel that
+    splits their rows): one launch per layer over all layers (so a launch never finds its weights in L2),
     replayed from a CUDA graph so host launch cost does not enter.  Bytes are
     the algorithmic ones: the launch's weight matrix; attention counts its
     K/V reads at context pos0."""
